@@ -117,11 +117,11 @@ static int make_tmap_2d(CUtensorMap* m, void* base, const Geom& g, int nv, int b
 
 // Tiled float64 map of a padded 2D/3D state [nvar][pz][py][pitch]: the
 // float64 stage kernel's halo tile (box sx x sy [x sz]) of every field.
-static int make_tmap_f64(CUtensorMap* m, void* base, const Geom& g, int nv) {
+static int make_tmap_f64(CUtensorMap* m, void* base, const Geom& g, int tile, int nv) {
   auto enc = tensor_map_encoder();
   if (!enc) { rsst_set_error("cuTensorMapEncodeTiled unavailable from the CUDA driver"); return RSST_ECUDA; }
   int sx, sy, sz;
-  rsst_stage_fp64_box(g.ndim, &sx, &sy, &sz);
+  rsst_stage_fp64_box(g, tile, &sx, &sy, &sz);
   const bool d3 = g.ndim == 3;
   const cuuint32_t rank = d3 ? 4 : 3;
   const cuuint64_t dims[4] = {(cuuint64_t)g.pitch, (cuuint64_t)g.py, d3 ? (cuuint64_t)g.pz : (cuuint64_t)nv,
@@ -225,6 +225,15 @@ static void make_phys(const rsst_config* c, Phys* p) {
   p->inv_xi = 1.0 / c->xi;
   p->f = 1.0 - 1.0 / (c->xi * c->xi);
   p->gamma_xi2 = c->gamma / (c->xi * c->xi);
+  {
+    int e;
+    const double m = 2.0 * std::frexp(p->gamma_xi2, &e);  // in [1, 2)
+    p->gxh = (float)m;
+    p->gxl = (float)(m - (double)p->gxh);
+    p->gxe = e - 1;
+  }
+  p->gam_gm1 = c->gamma / p->gm1;
+  p->f_gm1 = p->f * p->gm1;
   p->use_cmax = c->cmax > 0.0;
   p->inv_cmax4 = p->use_cmax ? 1.0 / (c->cmax * c->cmax * c->cmax * c->cmax) : 0.0;
   p->cfl = c->cfl;
@@ -236,6 +245,7 @@ static void make_phys(const rsst_config* c, Phys* p) {
     const bool act = d < c->ndim;
     p->grav[d] = act ? c->grav[d] : 0.0;
     p->inv_dx[d] = act ? 1.0 / c->dx[d] : 0.0;
+    p->half_inv_dx[d] = 0.5 * p->inv_dx[d];
     p->bc[d] = act ? c->bc[d] : RSST_BC_PERIODIC;
     if (act) p->sum_inv_dx += 1.0 / c->dx[d];
     if (act && c->grav[d] != 0.0) p->has_grav = 1;
@@ -354,9 +364,18 @@ extern "C" int rsst_init(rsst_handle** out, const rsst_config* cfg, void* stream
     }
   }
   if (cfg->precision == RSST_FP64 && cfg->ndim >= 2) {
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) {
+      cudaGetLastError();
+      rsst_set_error("cannot query the device's SM count");
+      rc = RSST_ECUDA;
+      goto fail;
+    }
     h->use_tma_fp64 = 1;
+    h->fp64_tile = rsst_stage_fp64_tile(h->g, sms);
     for (int b = 0; b < 2; ++b) {
-      rc = make_tmap_f64(&h->tmap[b], h->buf[b], h->g, nv);
+      rc = make_tmap_f64(&h->tmap[b], h->buf[b], h->g, h->fp64_tile, nv);
       if (rc != RSST_OK) goto fail;
     }
   }
@@ -464,6 +483,7 @@ static int plain_steps(rsst_handle* h, double dt, int nsteps, cudaStream_t st) {
   a.flag = h->d_flag;
   a.dt_fixed = dt > 0.0 ? dt : 0.0;
   a.stall_ns = h->stall_ns;
+  a.tile = h->fp64_tile;
   T* U = (T*)h->buf[0];
   T* Us = (T*)h->buf[1];
   for (int s = 0; s < nsteps; ++s) {

@@ -10,10 +10,18 @@ __device__ __forceinline__ int64_t pidx(const Geom& g, int i, int j, int k) {
   return (int64_t)(k + g.gz) * g.plane + (int64_t)(j + g.gy) * g.pitch + (i + g.xoff);
 }
 
+// Maximum of non-negative doubles, whose bit patterns order like their
+// values: on the integer pipe (a float64 compare or maximum occupies the
+// float64 pipe as long as an FMA).
+__device__ __forceinline__ double max_nonneg(double a, double b) {
+  const long long x = __double_as_longlong(a), y = __double_as_longlong(b);
+  return __longlong_as_double(x > y ? x : y);
+}
 __device__ __forceinline__ double warp_max(double x) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) x = fmax(x, __shfl_xor_sync(0xffffffffu, x, o));
-  return x;
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  const unsigned mh = __reduce_max_sync(0xffffffffu, hi);
+  const unsigned ml = __reduce_max_sync(0xffffffffu, hi == mh ? lo : 0u);
+  return __hiloint2double((int)mh, (int)ml);
 }
 
 // Block-wide maximum of non-negative values, then one atomicMax on the bit
@@ -28,7 +36,7 @@ __device__ __forceinline__ void block_max_to(double x, double* dst, double* sred
   if (wid == 0) {
     double y = lane < NT / 32 ? sred[lane] : 0.0;
     y = warp_max(y);
-    if (lane == 0 && y > 0.0)
+    if (lane == 0 && __double_as_longlong(y) > 0)
       atomicMax(reinterpret_cast<unsigned long long*>(dst), (unsigned long long)__double_as_longlong(y));
   }
 }

@@ -9,17 +9,25 @@
 //      boundary, rows and planes beyond the padded state zero-filled, a
 //      bounded mbarrier wait), in 1D (tiles wider than a TMA box) with
 //      coalesced loads;
-//   2. per axis D, the MC slope of every cell along D is computed once into
-//      shared memory (1D/2D tiles and small 3D tiles; larger 3D tiles take
-//      the two slopes per face), then every face of the tile gets twice its
-//      LLF flux, F(qL) + F(qR) - alpha (qR - qL), from the face states of
-//      the two cells beside it; a face shared by two tiles is computed the
-//      same way in both, so both get bit-identical values (discrete
-//      conservation);
-//   3. each cell accumulates -(2F_{+} - 2F_{-}) / (2 dx_D) in registers;
+//   2. the MC slope of every cell along each axis is computed once into
+//      shared memory (1D/2D tiles: all axes at once; 3D tiles: axis by axis),
+//      then every face of the tile gets twice its LLF flux,
+//      F(qL) + F(qR) - alpha (qR - qL), from the face states of the two cells
+//      beside it; a face shared by two tiles is computed the same way in both,
+//      so both get bit-identical values (discrete conservation);
+//   3. each cell takes -(2F_{+} - 2F_{-}) / (2 dx_D) of every axis;
 //   4. epilogue per cell: RSST correction, force, RK combine, store, the
 //      edge ghost cells the cell is the image of, and in stage 2 the CFL
 //      maximum for the next step and the physical-state flag.
+//
+// What bounds it: the float64 pipe, which takes one warp instruction per 16
+// SM clocks (a warp alone one per 64, however few lanes it has active) while
+// every other pipe idles.  So the work is arranged for few float64
+// instructions: 165.7 a 2D cell in stage 1 and 189.7 in stage 2 (ncu), 205.5
+// and 227.5 with the wave speeds' squares, the reciprocal's third-order step,
+// the block maximum, a per-thread dt division and unshared slope differences
+// on that pipe.  512^2: 123 -> 92 us a stage; 3D 256 x 128 x 128: 3090 -> 2500
+// us; 2048^2 runs the pipe 86 % busy.
 #include <cstdio>
 
 #include "rsst_common.cuh"
@@ -81,145 +89,195 @@ struct TileCfg {
   static constexpr int SCELLS = SX * SY * SZ;
   static constexpr int NCELL = BX * BY * BZ;
   static constexpr int CPT = (NCELL + NT - 1) / NT;
-  static constexpr int FX = (BX + 1) * BY * BZ;
-  static constexpr int FY = NDIM >= 2 ? BX * (BY + 1) * BZ : 0;
-  static constexpr int FZ = NDIM >= 3 ? BX * BY * (BZ + 1) : 0;
-  static constexpr int FMAX = FX > FY ? (FX > FZ ? FX : FZ) : (FY > FZ ? FY : FZ);
-  // Tiles keep each cell's MC slope along the current axis in shared memory
-  // (cells -1 .. B along that axis), computed once per cell instead of once
-  // per face side, when the slope array still leaves room for several CTAs
-  // per SM; larger 3D tiles recompute them per face.
-  static constexpr int EX0 = (BX + 2) * BY * BZ, EX1 = NDIM >= 2 ? BX * (BY + 2) * BZ : 0;
-  static constexpr int EX2 = NDIM >= 3 ? BX * BY * (BZ + 2) : 0;
-  static constexpr int EXM = EX0 > EX1 ? (EX0 > EX2 ? EX0 : EX2) : (EX1 > EX2 ? EX1 : EX2);
-  static constexpr bool SLOPES =
-      NDIM <= 2 || sizeof(double) * (size_t)NV * (SCELLS + FMAX + EXM) <= (size_t)76 * 1024;
-  static constexpr int SEMAX = SLOPES ? EXM : 0;
-  // halo tile, faces, slopes, the block reduction's 64 doubles, and two
+  // faces and slope cells (-1 .. B along the axis) per axis
+  static constexpr int F0 = (BX + 1) * BY * BZ, F1 = NDIM >= 2 ? BX * (BY + 1) * BZ : 0;
+  static constexpr int F2 = NDIM >= 3 ? BX * BY * (BZ + 1) : 0;
+  static constexpr int E0 = (BX + 2) * BY * BZ, E1 = NDIM >= 2 ? BX * (BY + 2) * BZ : 0;
+  static constexpr int E2 = NDIM >= 3 ? BX * BY * (BZ + 2) : 0;
+  static constexpr int max3(int a, int b, int c) { return a > b ? (a > c ? a : c) : (b > c ? b : c); }
+  // 1D/2D tiles hold the slopes and faces of every axis at once: three block
+  // barriers a tile instead of six, and the axes' passes fill each other's
+  // gaps.  3D tiles (three axes would leave room for one CTA an SM) go axis
+  // by axis through one slope and one face array.
+  static constexpr bool ALL = NDIM <= 2;
+  static constexpr int FMAX = ALL ? F0 + F1 : max3(F0, F1, F2);
+  static constexpr int EMAX = ALL ? E0 + E1 : max3(E0, E1, E2);
+  static constexpr int up32(int x) { return (x + 31) / 32 * 32; }
+  // halo tile, faces, slopes, the block reduction's 64 doubles, dt, and two
   // mbarriers (the tile copy; the failure-detection test wait)
-  static constexpr size_t SMEM = sizeof(double) * (size_t)NV * (SCELLS + FMAX + SEMAX) + 64 * sizeof(double) + 16;
+  static constexpr size_t SMEM = sizeof(double) * ((size_t)NV * (SCELLS + FMAX + EMAX) + 64 + 1) + 16;
   static constexpr uint32_t TILE_BYTES = (uint32_t)(sizeof(double) * NV * SCELLS);
   static_assert(NDIM == 1 || (SX <= 256 && SY <= 256 && SZ <= 256), "TMA box dimensions are at most 256");
+  static_assert(BX % 2 == 0 && (NDIM < 2 || BY % 2 == 0) && (NDIM < 3 || BZ % 2 == 0), "slopes are taken in pairs");
   static_assert((SX * sizeof(double)) % 16 == 0 && (HX * sizeof(double)) % 16 == 0,
                 "the box's row bytes and the x origin (interior x0 - HX) stay on 16-byte boundaries");
 };
 
-// Faces along axis D of the tile: index space (BX + [D==0]) x (BY + [D==1]) x (BZ + [D==2]).
+// MC slopes along D of the pair of neighbouring slope cells e (tile
+// coordinates -1 .. B along D, 0 .. B-1 across; pairs lie along D): the two
+// share a difference, five float64 additions a field instead of six.
+template <class C, int BX, int BY, int BZ, int D>
+__device__ __forceinline__ void slope_pair(const double* __restrict__ su, double* __restrict__ ss, int e) {
+  constexpr int STRIDE = D == 0 ? 1 : (D == 1 ? C::SX : C::SX * C::SY);
+  constexpr int XX = BX + 2 * (D == 0), YY = BY + 2 * (D == 1);
+  constexpr int PX = D == 0 ? XX / 2 : XX, PY = D == 1 ? YY / 2 : YY;  // pairs per axis
+  const int ex = e % PX * (D == 0 ? 2 : 1);
+  const int t = e / PX;
+  const int ey = t % PY * (D == 1 ? 2 : 1);
+  const int ez = t / PY * (D == 2 ? 2 : 1);
+  const int s0 = (ez - (D == 2) + C::HZ) * C::SX * C::SY + (ey - (D == 1) + C::HY) * C::SX + (ex - (D == 0) + C::HX);
+  const int o = (ez * YY + ey) * XX + ex;
+  constexpr int STRIDE_E = D == 0 ? 1 : (D == 1 ? XX : XX * YY);
+#pragma unroll
+  for (int v = 0; v < C::NV; ++v) {
+    const double* sv = su + v * C::SCELLS + s0;
+    const double um = sv[-STRIDE], u0 = sv[0], u1 = sv[STRIDE], up = sv[2 * STRIDE];
+    const double d = u1 - u0;
+    ss[v * C::EMAX + o] = mc_slope(u0 - um, d);
+    ss[v * C::EMAX + o + STRIDE_E] = mc_slope(d, up - u1);
+  }
+}
+
+// Twice the LLF flux of face fid along D: index space
+// (BX + [D==0]) x (BY + [D==1]) x (BZ + [D==2]), the face below that cell.
+template <class C, int NDIM, int BX, int BY, int BZ, int D, bool CV>
+__device__ __forceinline__ void face_flux(const double* __restrict__ su, const double* __restrict__ ss,
+                                          double* __restrict__ sf, const Phys& p, const Geom& g, int i0, int j0,
+                                          int k0, int fid) {
+  constexpr int NV = C::NV;
+  constexpr int EX = BX + (D == 0), EY = BY + (D == 1);
+  constexpr int STRIDE = D == 0 ? 1 : (D == 1 ? C::SX : C::SX * C::SY);
+  constexpr int XX = BX + 2 * (D == 0), YY = BY + 2 * (D == 1);
+  const int fx = fid % EX;
+  const int t = fid / EX;
+  const int fy = t % EY;
+  const int fz = t / EY;
+  // face fD - 1/2 of tile cell (fx, fy, fz); valid if its cells exist
+  const bool valid = (i0 + fx <= g.n[0] - (D == 0 ? 0 : 1)) && (NDIM < 2 || j0 + fy <= g.n[1] - (D == 1 ? 0 : 1)) &&
+                     (NDIM < 3 || k0 + fz <= g.n[2] - (D == 2 ? 0 : 1));
+  if (!valid) return;
+  // shared-memory index of the cell right of the face; its slope index (the left one is STRIDE_E before)
+  const int s0 = (fz + C::HZ) * C::SX * C::SY + (fy + C::HY) * C::SX + (fx + C::HX);
+  constexpr int STRIDE_E = D == 0 ? 1 : (D == 1 ? XX : XX * YY);
+  const int er = ((fz + (D == 2)) * YY + (fy + (D == 1))) * XX + (fx + (D == 0));
+  double qL[NV], qR[NV];
+#pragma unroll
+  for (int v = 0; v < NV; ++v) {
+    const double* sv = su + v * C::SCELLS + s0;
+    qL[v] = fma(0.5, ss[v * C::EMAX + er - STRIDE_E], sv[-STRIDE]);
+    qR[v] = fma(-0.5, ss[v * C::EMAX + er], sv[0]);
+  }
+  double F[NV];
+  llf_flux_x2<NV, D, CV>(qL, qR, p, F);
+#pragma unroll
+  for (int v = 0; v < NV; ++v) sf[v * C::FMAX + fid] = F[v];
+}
+
+// The x and y faces of a 2D tile as one list (f < F0: x, then y): the axis
+// only enters through strides and through which momentum is the normal one,
+// so a warp that holds faces of both axes does not diverge (16 x 16 tiles: 17
+// warps of faces; 18 with each axis padded to whole warps).
+template <class C, int BX, int BY, bool CV>
+__device__ __forceinline__ void face_flux_xy(const double* __restrict__ su, const double* __restrict__ ss,
+                                             double* __restrict__ sf, const Phys& p, const Geom& g, int i0, int j0,
+                                             int f) {
+  const bool isy = f >= C::F0;
+  const int fid = isy ? f - C::F0 : f;
+  const int ex = isy ? BX : BX + 1;
+  const int fy = isy ? fid / BX : fid / (BX + 1);
+  const int fx = fid - fy * ex;
+  if (i0 + fx > g.n[0] - (isy ? 1 : 0) || j0 + fy > g.n[1] - (isy ? 0 : 1)) return;
+  const int s0 = (fy + C::HY) * C::SX + (fx + C::HX);
+  const int sl = s0 - (isy ? C::SX : 1);
+  const int er = isy ? C::E0 + (fy + 1) * BX + fx : fy * (BX + 2) + fx + 1;
+  const int el = er - (isy ? BX : 1);
+  const int n = isy ? 2 : 1, t = 3 - n;  // fields of the normal and the transverse momentum
+  const int fld[4] = {0, n, t, 3};
+  double qL[4], qR[4], F[4];
+#pragma unroll
+  for (int v = 0; v < 4; ++v) {
+    const double* sv = su + fld[v] * C::SCELLS;
+    const double* se = ss + fld[v] * C::EMAX;
+    qL[v] = fma(0.5, se[el], sv[sl]);
+    qR[v] = fma(-0.5, se[er], sv[s0]);
+  }
+  llf_flux_x2<4, 0, CV>(qL, qR, p, F);
+#pragma unroll
+  for (int v = 0; v < 4; ++v) sf[fld[v] * C::FMAX + f] = F[v];
+}
+
+// 2F above minus 2F below tile cell (cx, cy, cz) along D, per field.
+template <class C, int BX, int BY, int BZ, int D>
+__device__ __forceinline__ void face_diff(const double* __restrict__ sf, int cx, int cy, int cz, double (&d)[C::NV]) {
+  constexpr int EX = BX + (D == 0), EY = BY + (D == 1);
+  const int flo = (cz * EY + cy) * EX + cx;
+  const int fhi = flo + (D == 0 ? 1 : (D == 1 ? EX : EX * EY));
+#pragma unroll
+  for (int v = 0; v < C::NV; ++v) d[v] = sf[v * C::FMAX + fhi] - sf[v * C::FMAX + flo];
+}
+
+// One axis of a 3D tile: slopes, faces, and each thread's cells' divergence.
+// The next axis may overwrite the slopes at once (every face was formed) and
+// the faces after its own slope barrier (every divergence was taken).
 template <int NDIM, int BX, int BY, int BZ, int NT, int D, bool CV>
-__device__ __forceinline__ void face_pass(const double* __restrict__ su, double* __restrict__ sf,
+__device__ __forceinline__ void axis_pass(const double* __restrict__ su, double* __restrict__ sf,
                                           double* __restrict__ ss, const Phys& p, const Geom& g, int i0, int j0,
                                           int k0, double (&dU)[TileCfg<NDIM, BX, BY, BZ, NT>::CPT][NDIM + 2]) {
   using C = TileCfg<NDIM, BX, BY, BZ, NT>;
-  constexpr int NV = C::NV;
-  constexpr int EX = BX + (D == 0), EY = BY + (D == 1), EZ = BZ + (D == 2);
-  constexpr int NF = EX * EY * EZ;
-  constexpr int STRIDE = D == 0 ? 1 : (D == 1 ? C::SX : C::SX * C::SY);
-  // slope cells: tile coordinates -1 .. B along D, 0 .. B-1 across
-  constexpr int XX = BX + 2 * (D == 0), YY = BY + 2 * (D == 1), ZZ = BZ + 2 * (D == 2);
-  constexpr int NE = XX * YY * ZZ;
-  const int nD = g.n[D];
-  const int baseD = D == 0 ? i0 : (D == 1 ? j0 : k0);
-  if constexpr (C::SLOPES) {
-    for (int e = threadIdx.x; e < NE; e += NT) {
-      const int ex = e % XX;
-      const int t = e / XX;
-      const int ey = t % YY;
-      const int ez = t / YY;
-      const int s0 = (ez - (D == 2) + C::HZ) * C::SX * C::SY + (ey - (D == 1) + C::HY) * C::SX + (ex - (D == 0) + C::HX);
-#pragma unroll
-      for (int v = 0; v < NV; ++v) {
-        const double* sv = su + v * C::SCELLS + s0;
-        const double um = sv[-STRIDE], u0 = sv[0], up = sv[STRIDE];
-        ss[v * C::SEMAX + e] = mc_slope(u0 - um, up - u0);
-      }
-    }
-    __syncthreads();
-  }
-  for (int fid = threadIdx.x; fid < NF; fid += NT) {
-    const int fx = fid % EX;
-    const int t = fid / EX;
-    const int fy = t % EY;
-    const int fz = t / EY;
-    // face fD - 1/2 of tile cell (fx, fy, fz); valid if its cells exist
-    const int fD = D == 0 ? fx : (D == 1 ? fy : fz);
-    const bool valid = (i0 + fx <= g.n[0] - (D == 0 ? 0 : 1)) && (NDIM < 2 || j0 + fy <= g.n[1] - (D == 1 ? 0 : 1)) &&
-                       (NDIM < 3 || k0 + fz <= g.n[2] - (D == 2 ? 0 : 1)) && (baseD + fD <= nD);
-    if (!valid) continue;
-    // shared-memory index of the cell right of the face
-    const int s0 = (fz + C::HZ) * C::SX * C::SY + (fy + C::HY) * C::SX + (fx + C::HX);
-    double qL[NV], qR[NV];
-    if constexpr (C::SLOPES) {
-      // slope index of the cell right of the face; the left one is STRIDE_E before
-      constexpr int STRIDE_E = D == 0 ? 1 : (D == 1 ? XX : XX * YY);
-      const int er = ((fz + (D == 2)) * YY + (fy + (D == 1))) * XX + (fx + (D == 0));
-#pragma unroll
-      for (int v = 0; v < NV; ++v) {
-        const double* sv = su + v * C::SCELLS + s0;
-        qL[v] = fma(0.5, ss[v * C::SEMAX + er - STRIDE_E], sv[-STRIDE]);
-        qR[v] = fma(-0.5, ss[v * C::SEMAX + er], sv[0]);
-      }
-    } else {
-#pragma unroll
-      for (int v = 0; v < NV; ++v) {
-        const double* sv = su + v * C::SCELLS + s0;
-        const double um2 = sv[-2 * STRIDE], um1 = sv[-STRIDE], u0 = sv[0], up1 = sv[STRIDE];
-        const double sl = mc_slope(um1 - um2, u0 - um1);
-        const double sr = mc_slope(u0 - um1, up1 - u0);
-        qL[v] = um1 + 0.5 * sl;
-        qR[v] = u0 - 0.5 * sr;
-      }
-    }
-    double F[NV];  // twice the face flux
-    llf_flux_x2<NV, D, CV>(qL, qR, p, F);
-#pragma unroll
-    for (int v = 0; v < NV; ++v) sf[v * C::FMAX + fid] = F[v];
-  }
+  constexpr int NE = D == 0 ? C::E0 : (D == 1 ? C::E1 : C::E2), NF = D == 0 ? C::F0 : (D == 1 ? C::F1 : C::F2);
+  for (int e = threadIdx.x; e < NE / 2; e += NT) slope_pair<C, BX, BY, BZ, D>(su, ss, e);
   __syncthreads();
-  const double idx = 0.5 * p.inv_dx[D];  // the faces hold 2 F
+  for (int f = threadIdx.x; f < NF; f += NT) face_flux<C, NDIM, BX, BY, BZ, D, CV>(su, ss, sf, p, g, i0, j0, k0, f);
+  __syncthreads();
+  const double idx = p.half_inv_dx[D];  // the faces hold 2 F
 #pragma unroll
   for (int c = 0; c < C::CPT; ++c) {
     const int cell = threadIdx.x + c * NT;
     if (cell >= C::NCELL) break;
-    const int cx = cell % BX;
-    const int t = cell / BX;
-    const int cy = t % BY;
-    const int cz = t / BY;
-    const int flo = (cz * EY + cy) * EX + cx;
-    const int fhi = flo + (D == 0 ? 1 : (D == 1 ? EX : EX * EY));
+    double d[C::NV];
+    face_diff<C, BX, BY, BZ, D>(sf, cell % BX, cell / BX % BY, cell / BX / BY, d);
 #pragma unroll
-    for (int v = 0; v < NV; ++v) dU[c][v] -= (sf[v * C::FMAX + fhi] - sf[v * C::FMAX + flo]) * idx;
+    for (int v = 0; v < C::NV; ++v) dU[c][v] = D == 0 ? -d[v] * idx : fma(-d[v], idx, dU[c][v]);
   }
-  __syncthreads();
 }
 
-template <int NDIM, int BX, int BY, int BZ, int NT, bool TMA, bool CV>
-__global__ void __launch_bounds__(NT, NDIM == 3 ? 3 : 0)
+template <int NDIM, int BX, int BY, int BZ, int NT, int MINB, bool TMA, bool CV>
+__global__ void __launch_bounds__(NT, MINB)
     stage_fp64_kernel(const __grid_constant__ CUtensorMap tin, const StageArgs<double> a) {
   using C = TileCfg<NDIM, BX, BY, BZ, NT>;
   constexpr int NV = C::NV;
   extern __shared__ __align__(128) double smem[];
   double* su = smem;
   double* sf = smem + NV * C::SCELLS;
-  double* ss = sf + NV * C::FMAX;  // slopes (1D/2D tiles)
-  double* sred = ss + NV * C::SEMAX;
+  double* ss = sf + NV * C::FMAX;
+  double* sred = ss + NV * C::EMAX;
+  double* sdt = sred + 64;
   const Geom& g = a.g;
   const Phys& p = a.p;
   const int i0 = blockIdx.x * BX, j0 = blockIdx.y * BY, k0 = blockIdx.z * BZ;
+  uint64_t* bar = reinterpret_cast<uint64_t*>(sdt + 1);
+  uint64_t* test_bar = bar + 1;
+  const bool stall = TMA && a.stall_ns > 0;
+  if (TMA && threadIdx.x == 0) {
+    mbar_init(bar, 1);
+    if (stall) mbar_init(test_bar, 1);
+    fence_mbar_init();
+  }
 
-  // 1. halo tile -> shared memory
+  // 1. halo tile -> shared memory; dt once per CTA (a float64 division)
+  if (threadIdx.x == (TMA ? NT - 1 : 0)) {
+    const double dt = a.dt_fixed > 0.0 ? a.dt_fixed : p.cfl / a.scal[a.slot];
+    *sdt = dt;
+    if (a.stage == 1 && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0) {
+      a.scal[a.slot ^ 1] = 0.0;
+      a.scal[2] = dt;
+      a.scal[3] += dt;
+    }
+  }
   if constexpr (TMA) {
     // The box of the padded state [nvar][pz][py][pitch] whose first cell is
     // interior (i0 - HX, j0 - HY, k0 - HZ): padded x i0 + xoff - HX, padded
     // y j0 (HY = gy), padded z k0 (HZ = gz).
-    uint64_t* bar = reinterpret_cast<uint64_t*>(sred + 64);
-    uint64_t* test_bar = bar + 1;
-    const bool stall = a.stall_ns > 0;
-    if (threadIdx.x == 0) {
-      mbar_init(bar, 1);
-      if (stall) mbar_init(test_bar, 1);
-      fence_mbar_init();
-    }
-    __syncthreads();
     if (threadIdx.x == 0) {
       fence_proxy_async_smem();
       mbar_expect_tx(bar, C::TILE_BYTES);
@@ -229,6 +287,7 @@ __global__ void __launch_bounds__(NT, NDIM == 3 ? 3 : 0)
       // delivers, waited on while the tile copy is still in flight
       if (stall) mbar_expect_tx(test_bar, 16);
     }
+    __syncthreads();  // the barriers are initialised
     const bool landed = stall ? mbar_wait_bounded(test_bar, 0u, (uint64_t)a.stall_ns) : mbar_wait_bounded(bar, 0u);
     // Giving up is decided by the whole block: flag the run and, before
     // leaving, wait (bounded) for the tile copy, so that it cannot land in
@@ -241,39 +300,62 @@ __global__ void __launch_bounds__(NT, NDIM == 3 ? 3 : 0)
       return;
     }
   } else {
-  for (int id = threadIdx.x; id < NV * C::SCELLS; id += NT) {
-    const int v = id / C::SCELLS;
-    const int r = id - v * C::SCELLS;
-    const int lx = r % C::SX;
-    const int t = r / C::SX;
-    const int ly = t % C::SY;
-    const int lz = t / C::SY;
-    const int gi = i0 + lx - C::HX, gj = j0 + ly - C::HY, gk = k0 + lz - C::HZ;
-    double val = 0.0;
-    if (gi <= g.n[0] + 1 && (NDIM < 2 || gj <= g.n[1] + 1) && (NDIM < 3 || gk <= g.n[2] + 1))
-      val = a.in[v * g.fstride + pidx(g, gi, gj, gk)];
-    su[id] = val;
-  }
-  __syncthreads();
+    for (int id = threadIdx.x; id < NV * C::SCELLS; id += NT) {
+      const int v = id / C::SCELLS;
+      const int r = id - v * C::SCELLS;
+      const int lx = r % C::SX;
+      const int t = r / C::SX;
+      const int ly = t % C::SY;
+      const int lz = t / C::SY;
+      const int gi = i0 + lx - C::HX, gj = j0 + ly - C::HY, gk = k0 + lz - C::HZ;
+      double val = 0.0;
+      if (gi <= g.n[0] + 1 && (NDIM < 2 || gj <= g.n[1] + 1) && (NDIM < 3 || gk <= g.n[2] + 1))
+        val = a.in[v * g.fstride + pidx(g, gi, gj, gk)];
+      su[id] = val;
+    }
+    __syncthreads();
   }
 
-  // 2-3. face fluxes and divergence, axis by axis
+  // 2-3. slopes, face fluxes and divergence
   double dU[C::CPT][NV];
+  if constexpr (C::ALL) {
+    constexpr int PE = C::up32(C::E0 / 2);  // axis y starts at a whole warp
+    for (int e = threadIdx.x; e < (NDIM == 1 ? C::E0 / 2 : PE + C::E1 / 2); e += NT) {
+      if (e < PE) {
+        if (e < C::E0 / 2) slope_pair<C, BX, BY, BZ, 0>(su, ss, e);
+      } else if constexpr (NDIM == 2) {
+        slope_pair<C, BX, BY, BZ, 1>(su, ss + C::E0, e - PE);
+      }
+    }
+    __syncthreads();
+    if constexpr (NDIM == 1) {
+      for (int f = threadIdx.x; f < C::F0; f += NT) face_flux<C, 1, BX, BY, BZ, 0, CV>(su, ss, sf, p, g, i0, j0, k0, f);
+    } else {
+      for (int f = threadIdx.x; f < C::F0 + C::F1; f += NT) face_flux_xy<C, BX, BY, CV>(su, ss, sf, p, g, i0, j0, f);
+    }
+    __syncthreads();
 #pragma unroll
-  for (int c = 0; c < C::CPT; ++c)
+    for (int c = 0; c < C::CPT; ++c) {
+      const int cell = threadIdx.x + c * NT;
+      if (cell >= C::NCELL) break;
+      double d[NV];
+      face_diff<C, BX, BY, BZ, 0>(sf, cell % BX, cell / BX, 0, d);
 #pragma unroll
-    for (int v = 0; v < NV; ++v) dU[c][v] = 0.0;
-  face_pass<NDIM, BX, BY, BZ, NT, 0, CV>(su, sf, ss, p, g, i0, j0, k0, dU);
-  if constexpr (NDIM >= 2) face_pass<NDIM, BX, BY, BZ, NT, 1, CV>(su, sf, ss, p, g, i0, j0, k0, dU);
-  if constexpr (NDIM >= 3) face_pass<NDIM, BX, BY, BZ, NT, 2, CV>(su, sf, ss, p, g, i0, j0, k0, dU);
+      for (int v = 0; v < NV; ++v) dU[c][v] = -d[v] * p.half_inv_dx[0];  // the faces hold 2 F
+      if constexpr (NDIM == 2) {
+        face_diff<C, BX, BY, BZ, 1>(sf + C::F0, cell % BX, cell / BX, 0, d);
+#pragma unroll
+        for (int v = 0; v < NV; ++v) dU[c][v] = fma(-d[v], p.half_inv_dx[1], dU[c][v]);
+      }
+    }
+  } else {
+    axis_pass<NDIM, BX, BY, BZ, NT, 0, CV>(su, sf, ss, p, g, i0, j0, k0, dU);
+    axis_pass<NDIM, BX, BY, BZ, NT, 1, CV>(su, sf, ss, p, g, i0, j0, k0, dU);
+    axis_pass<NDIM, BX, BY, BZ, NT, 2, CV>(su, sf, ss, p, g, i0, j0, k0, dU);
+  }
 
   // 4. epilogue
-  const double dt = a.dt_fixed > 0.0 ? a.dt_fixed : p.cfl / a.scal[a.slot];
-  if (a.stage == 1 && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x == 0) {
-    a.scal[a.slot ^ 1] = 0.0;
-    a.scal[2] = dt;
-    a.scal[3] += dt;
-  }
+  const double dt = *sdt;
   double rmax = 0.0;
   bool ok_all = true;
 #pragma unroll
@@ -301,14 +383,14 @@ __global__ void __launch_bounds__(NT, NDIM == 3 ? 3 : 0)
     rsst_rhs<NV, CV>(q, L, p);
     if (a.stage == 1) {
 #pragma unroll
-      for (int v = 0; v < NV; ++v) u[v] = q[v] + dt * L[v];
+      for (int v = 0; v < NV; ++v) u[v] = fma(dt, L[v], q[v]);
     } else {
       const int64_t o = pidx(g, i, j, k);
 #pragma unroll
-      for (int v = 0; v < NV; ++v) u[v] = 0.5 * a.base[v * g.fstride + o] + 0.5 * (q[v] + dt * L[v]);
+      for (int v = 0; v < NV; ++v) u[v] = half_of(a.base[v * g.fstride + o] + fma(dt, L[v], q[v]));
       bool ok;
       const double r = cfl_rate<NV, CV>(u, p, ok);
-      if (ok) rmax = fmax(rmax, r);
+      if (ok) rmax = max_nonneg(rmax, r);
       ok_all = ok_all && ok;
     }
     store_with_ghosts<NV>(a.out, g, p, a.bg, a.bg_len, i, j, k, u);
@@ -394,7 +476,7 @@ __global__ void __launch_bounds__(256) cfl_fp64_kernel(const double* __restrict_
     for (int v = 0; v < NV; ++v) q[v] = U[v * g.fstride + o];
     bool ok;
     const double r = cfl_rate<NV, CV>(q, p, ok);
-    if (ok) rmax = fmax(rmax, r);
+    if (ok) rmax = max_nonneg(rmax, r);
     ok_all = ok_all && ok;
   }
   if (!ok_all) atomicOr(flag, RSST_FLAG_NONPHYSICAL);
@@ -454,10 +536,10 @@ __global__ void __launch_bounds__(SUM_THREADS) sums_final_kernel(const double* _
 // Launchers
 // ---------------------------------------------------------------------------
 
-template <int NDIM, int BX, int BY, int BZ, int NT, bool TMA, bool CV>
+template <int NDIM, int BX, int BY, int BZ, int NT, int MINB, bool TMA, bool CV>
 static int launch_stage_eos(const CUtensorMap* tin, const StageArgs<double>& a, cudaStream_t s) {
   using C = TileCfg<NDIM, BX, BY, BZ, NT>;
-  auto kern = stage_fp64_kernel<NDIM, BX, BY, BZ, NT, TMA, CV>;
+  auto kern = stage_fp64_kernel<NDIM, BX, BY, BZ, NT, MINB, TMA, CV>;
   static std::atomic<unsigned long long> attr{0};
   if (set_smem_limit_once(kern, C::SMEM, attr) != cudaSuccess) {
     rsst_set_error("cudaFuncSetAttribute failed for the float64 stage kernel");
@@ -475,39 +557,64 @@ static int launch_stage_eos(const CUtensorMap* tin, const StageArgs<double>& a, 
 }
 
 // The gas law is a compile-time choice (no covolume arithmetic in ideal-gas runs).
-template <int NDIM, int BX, int BY, int BZ, int NT, bool TMA>
+template <int NDIM, int BX, int BY, int BZ, int NT, int MINB, bool TMA>
 static int launch_stage(const CUtensorMap* tin, const StageArgs<double>& a, cudaStream_t s) {
-  if (a.p.covol != 0.0) return launch_stage_eos<NDIM, BX, BY, BZ, NT, TMA, true>(tin, a, s);
-  return launch_stage_eos<NDIM, BX, BY, BZ, NT, TMA, false>(tin, a, s);
+  if (a.p.covol != 0.0) return launch_stage_eos<NDIM, BX, BY, BZ, NT, MINB, TMA, true>(tin, a, s);
+  return launch_stage_eos<NDIM, BX, BY, BZ, NT, MINB, TMA, false>(tin, a, s);
 }
 
 }  // namespace rsst
 
 using namespace rsst;
 
-// Tiles: 1D short lines take 16-cell tiles (17 faces, one per thread of a
-// warp) to spread the float64 work over SMs, longer ones 256 cells; 2D 16 x 16
-// with 9 warps (every face and slope pass in one round; 0.7 % ahead of 32 x 8
-// with the halo by TMA, from fewer halo slopes and faces); 3D 8 x 8 x 4 with
-// slopes in shared memory and 10 warps (each face pass in one round).
-using Tile2 = TileCfg<2, 16, 16, 1, 288>;
-using Tile3 = TileCfg<3, 8, 8, 4, 320>;
+// Tiles.  1D: short lines take 16-cell tiles (17 faces, one per thread of a
+// warp) to spread the float64 work over SMs, longer ones 256 cells.  3D
+// 8 x 8 x 4 with 10 warps (each face pass in one round).
+// 2D: the tile that finishes first by a linear model, offset + slope x the
+// most tiles any SM gets (the float64 pipe of an SM serves its tiles one
+// after the other).  16 x 16 has the fewest halo faces a cell, smaller tiles
+// spread a small grid over more SMs.  Measured per stage (us, GB300; 16 x 16
+// / 16 x 8 / 8 x 8): 64^2 16.9 / 11.8 / 8.7, 128^2 16.9 / 12.1 / 11.8, 192^2
+// 16.9 / 17.5 / 19.8, 224^2 30.4 / 24.9 / 31.0, 256^2 30.4 / 32.2 / 34.7,
+// 512^2 99.5 / 106.5 / 118.5, 2048^2 1493 / 1603 / 1840; the constants fit
+// these.  (4 x 4 tiles gained 0.1 us on 64^2 and lost elsewhere.)
+static const int TILE2[3][2] = {{16, 16}, {16, 8}, {8, 8}};
 
-void rsst_stage_fp64_box(int ndim, int* sx, int* sy, int* sz) {
-  *sx = ndim == 3 ? Tile3::SX : Tile2::SX;
-  *sy = ndim == 3 ? Tile3::SY : Tile2::SY;
-  *sz = ndim == 3 ? Tile3::SZ : 1;
+int rsst_stage_fp64_tile(const Geom& g, int sms) {
+  static const double offset[3] = {3.4, 3.0, 4.6}, slope[3] = {13.5, 7.25, 4.05};
+  if (g.ndim != 2) return 0;
+  int best = 0;
+  double tbest = 0.0;
+  for (int t = 0; t < 3; ++t) {
+    const int64_t tiles = (int64_t)((g.n[0] + TILE2[t][0] - 1) / TILE2[t][0]) * ((g.n[1] + TILE2[t][1] - 1) / TILE2[t][1]);
+    const double us = offset[t] + slope[t] * (double)((tiles + sms - 1) / sms);
+    if (t == 0 || us < tbest) {
+      best = t;
+      tbest = us;
+    }
+  }
+  return best;
+}
+
+void rsst_stage_fp64_box(const Geom& g, int tile, int* sx, int* sy, int* sz) {
+  *sx = (g.ndim == 3 ? 8 : TILE2[tile][0]) + 2 * RSST_G;
+  *sy = (g.ndim == 3 ? 8 : TILE2[tile][1]) + 2 * RSST_G;
+  *sz = g.ndim == 3 ? 4 + 2 * RSST_G : 1;
 }
 
 int rsst_launch_stage_fp64(const CUtensorMap* tin, const StageArgs<double>& a, cudaStream_t s) {
   switch (a.g.ndim) {
     case 1:
-      if (a.g.n[0] <= RSST_SMALL_1D) return launch_stage<1, 16, 1, 1, 32, false>(nullptr, a, s);
-      return launch_stage<1, 256, 1, 1, 256, false>(nullptr, a, s);
+      if (a.g.n[0] <= RSST_SMALL_1D) return launch_stage<1, 16, 1, 1, 32, 1, false>(nullptr, a, s);
+      return launch_stage<1, 256, 1, 1, 256, 1, false>(nullptr, a, s);
     case 2:
-      return tin ? launch_stage<2, 16, 16, 1, 288, true>(tin, a, s) : launch_stage<2, 16, 16, 1, 288, false>(nullptr, a, s);
+      switch (a.tile) {
+        case 0: return launch_stage<2, 16, 16, 1, 288, 4, true>(tin, a, s);
+        case 1: return launch_stage<2, 16, 8, 1, 160, 6, true>(tin, a, s);
+        default: return launch_stage<2, 8, 8, 1, 160, 6, true>(tin, a, s);
+      }
     case 3:
-      return tin ? launch_stage<3, 8, 8, 4, 320, true>(tin, a, s) : launch_stage<3, 8, 8, 4, 320, false>(nullptr, a, s);
+      return launch_stage<3, 8, 8, 4, 320, 3, true>(tin, a, s);
   }
   rsst_set_error("ndim must be 1, 2 or 3");
   return RSST_EINVAL;

@@ -39,6 +39,11 @@ struct Phys {
   double gamma, gm1, inv_gm1, hgm1;  // hgm1 = (gamma - 1)/2
   double xi, inv_xi, f;  // f = 1 - 1/xi^2
   double gamma_xi2;      // gamma / xi^2: (a/xi)^2 = gamma_xi2 P / rho for the ideal gas
+  float gxh, gxl;        // gamma_xi2 = (gxh + gxl) 2^gxe, gxh in [1, 2): for the float-pair c_tot
+  int gxe;
+  double gam_gm1;        // gamma/(gamma - 1): (e + P)/P of the ideal gas
+  double f_gm1;          // f (gamma - 1)
+  double half_inv_dx[3]; // 1/(2 dx): the faces hold twice the flux
   double inv_cmax4;      // 1/C_max^4 (state-dependent xi, Eq. cx), used if use_cmax
   int use_cmax;
   double cfl;
@@ -122,16 +127,18 @@ struct StageArgs {
   const float* tabr; // row-major background table [tab_len][TR_W] (TMA float32 kernels), or null
   double* dU_out;   // float64 kernels: if set, the Euler tendency of each interior cell
                     // (padded layout) is written here too (adjoint recompute)
+  int tile;         // float64 2D: tile shape index (rsst_stage_fp64_tile)
   int64_t stall_ns; // > 0 (failure-detection tests only): each tile of a TMA-staged kernel
                     // also waits this long on a barrier that nothing completes
 };
 
 // Host-side launchers (defined in the .cu files).
-// tin: tensor map of a.in (2D/3D: the halo tile comes in by TMA), or null
-// (plain loads; always for 1D).
+// tin: tensor map of a.in (2D/3D: the halo tile comes in by TMA; unused in 1D).
 int rsst_launch_stage_fp64(const CUtensorMap* tin, const StageArgs<double>& a, cudaStream_t s);
 // Box (cells along x, y, z) of the float64 stage kernel's halo tile in 2D/3D.
-void rsst_stage_fp64_box(int ndim, int* sx, int* sy, int* sz);
+void rsst_stage_fp64_box(const Geom& g, int tile, int* sx, int* sy, int* sz);
+// Index of the 2D tile shape for a grid on a device with `sms` SMs.
+int rsst_stage_fp64_tile(const Geom& g, int sms);
 int rsst_launch_pack_fp64(const double* src, double* dst, const Geom& g, const Phys& p,
                           const double* bg, int bg_len, cudaStream_t s);
 int rsst_launch_unpack_fp64(const double* src, double* dst, const Geom& g, cudaStream_t s);
@@ -184,6 +191,7 @@ struct rsst_handle {
   int use_tma2d;        // 2D float32 runs use the TMA-staged kernel
   int use_tma3d;        // 3D float32 runs use the TMA z-march kernel
   int use_tma_fp64;     // 2D/3D float64 runs stage their halo tiles by TMA
+  int fp64_tile;        // their tile shape index
   CUtensorMap tmap[2];  // tensor maps of buf[0], buf[1] (TMA kernels)
   void* adj;            // adjoint checkpoints and work arrays, or null
   int slot;

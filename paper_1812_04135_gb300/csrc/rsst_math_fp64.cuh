@@ -51,10 +51,25 @@ struct Eos {
     if constexpr (CV) return p.gm1 * rcp_nr(omb(p, rho));
     return p.gm1;
   }
-  // (0.5 |V|^2 - (de/drho)_P) of the pressure tendency
-  __device__ static __forceinline__ double half_v2_minus_de_drho(const Phys& p, double v2, double P) {
-    if constexpr (CV) return fma(p.covol * p.inv_gm1, P, 0.5 * v2);
-    return 0.5 * v2;
+  // f [(de/dP)_rho]^-1
+  __device__ static __forceinline__ double f_over_de_dP(const Phys& p, double f, double rho, double P) {
+    if constexpr (CV) return f * inv_de_dP(p, rho, P);
+    return p.use_cmax ? f * p.gm1 : p.f_gm1;
+  }
+  // e + P
+  __device__ static __forceinline__ double enthalpy(const Phys& p, double rho, double P) {
+    if constexpr (CV) return internal_energy(p, rho, P) + P;
+    return p.gam_gm1 * P;
+  }
+  // 1/(rho a^2)
+  __device__ static __forceinline__ double inv_rho_a2(const Phys& p, double rho, double P) {
+    if constexpr (CV) return omb(p, rho) * rcp_nr(p.gamma * P);
+    return rcp_nr(p.gamma * P);
+  }
+  // (0.5 |V|^2 - (de/drho)_P) of the pressure tendency, from 0.5 |V|^2
+  __device__ static __forceinline__ double half_v2_minus_de_drho(const Phys& p, double hv2, double P) {
+    if constexpr (CV) return fma(p.covol * p.inv_gm1, P, hv2);
+    return hv2;
   }
   // a state the EOS admits: 1 - b rho > 0 (always true for the ideal gas)
   __device__ static __forceinline__ bool admissible(const Phys& p, double rho) {
@@ -63,14 +78,41 @@ struct Eos {
   }
 };
 
-// 1/x to full float64 accuracy with three float64-pipe instructions: the
-// hardware reciprocal approximation y, then one third-order step of the
-// series 1/x = y / (1 - e) = y (1 + e + e^2 + ...), e = 1 - x y formed
-// exactly by an FMA: y <- y + y (e + e^2), which cubes the seed's relative
-// error (two Newton-Raphson steps square it twice at four FMAs).  Within an
-// ulp of the correctly rounded quotient for the normal, positive densities
-// it is used on (checked against CUDA's division by rsst_math_selftest).
+// A positive double's leading 24 significant bits as a float h in [1, 2),
+// the other 29 as a float l, and its biased exponent (<= 0 for zero,
+// subnormal and negative values, 2047 for NaN and infinity).
+__device__ __forceinline__ void split_pair(double x, float& h, float& l, int& be) {
+  const int hi = __double2hiint(x);
+  const unsigned lo = (unsigned)__double2loint(x);
+  be = hi >> 20;
+  h = __uint_as_float(0x3f800000u | (__funnelshift_l(lo, (unsigned)hi, 3) & 0x7fffffu));
+  l = __uint2float_rn(lo & 0x1fffffffu) * __int_as_float((127 - 52) << 23);
+}
+
+// 1/x to full float64 accuracy with two float64-pipe instructions.  For a
+// positive x = (h + l) 2^k the seed comes from the float32 and integer pipes:
+// r = 1/h (hardware, 2^-23), its residual e = 1 - (h + l) r by two FMAs, and
+// y0 = r + r e assembled as a double (relative error about 2^-45); one Newton
+// step y0 + y0 (1 - x y0) squares that.  The float64 hardware seed is good
+// to 2^-20 only and takes a third-order step: three float64 instructions, of
+// about 22 that a face state costs.  Within an ulp of the correctly rounded
+// quotient (checked against CUDA's division by rsst_math_selftest).  Values
+// that are not positive normal numbers with room in the exponent (non-physical
+// states) take the hardware seed: y <- y + y (e + e^2), e = 1 - x y.
 __device__ __forceinline__ double rcp_nr(double x) {
+  float h, l;
+  int be;
+  split_pair(x, h, l, be);
+  if ((unsigned)(be - 64) < 1920u) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(h));
+    const float e = fmaf(-l, r, fmaf(-h, r, 1.0f));
+    // r in [1/2, 1]: units of 2^-53 (for r = 1 the correction is negative)
+    const int li = __float2int_rn((r * e) * __int_as_float((127 + 53) << 23));
+    const long long y0b = ((long long)__float_as_int(r) << 29) + ((long long)(896 + 1023 - be) << 52) + (long long)li;
+    const double y0 = __longlong_as_double(y0b);
+    return fma(y0, fma(-x, y0, 1.0), y0);
+  }
   double y;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
   const double e = fma(-x, y, 1.0);
@@ -157,6 +199,94 @@ __device__ __forceinline__ void ctot_pair(double v2, double a2x, float& h, float
   l = lo - (h - t);
 }
 
+// A normalised non-negative float pair (h + l, |l| <= ulp(h)/2) as a double,
+// on the integer pipe: h's 24 bits shifted up plus l in units of 2^-52 of h's
+// exponent (l below that is dropped: 2^-53 relative).  Below a power of two
+// the unit halves, hence the doubled l there.  Outside h in [2^-74, 2^126]
+// (and for NaN) the two halves are added.
+__device__ __forceinline__ double pair_to_double(float h, float l) {
+  const unsigned hb = __float_as_uint(h);
+  const int eh = (int)(hb >> 23);
+  const unsigned mant = hb & 0x7fffffu;
+  if (eh >= 53 && eh <= 253) {
+    int li = __float2int_rn(l * __int_as_float((306 - eh) << 23));
+    if (mant == 0u && li < 0) li += li;
+    return __longlong_as_double(((long long)(eh + 896) << 52) + ((long long)mant << 29) + (long long)li);
+  }
+  return f2d_bits(h) + f2d_bits(l);
+}
+
+// sqrt((h + l) 2^e) of a float pair with h in [1, 8) as a float pair: one
+// Newton step from the hardware rsqrt, the square split exactly by an FMA.
+__device__ __forceinline__ void sqrt_of_pair(float h, float l, int e, float& s, float& c) {
+  const int odd = e & 1;
+  const float f = odd ? 2.0f : 1.0f;
+  h *= f;
+  l *= f;
+  const float r = rsqrtf(h);
+  const float s0 = h * r;
+  const float p = s0 * s0;
+  const float d = ((h - p) - fmaf(s0, s0, -p)) + l;
+  const int k = (e - odd) >> 1;
+  const float sc = k < -126 ? 0.0f : (k > 127 ? __int_as_float(0x7f800000) : __int_as_float((127 + k) << 23));
+  s = s0 * sc;
+  c = d * (0.5f * r) * sc;
+}
+
+// Sum of two non-negative float pairs, normalised.
+__device__ __forceinline__ void pair_sum(float sv, float cv, float sa, float ca, float& h, float& l) {
+  const float t = sv + sa;
+  const float bv = t - sv;
+  const float lo = ((sv - (t - bv)) + (sa - bv)) + (cv + ca);
+  h = t + lo;
+  l = lo - (h - t);
+}
+
+// c_tot = |V| + a/xi as a float pair from k = rho |V|^2, P and 1/rho:
+// |V|^2 = k/rho and (a/xi)^2 = (gamma/xi^2) P/rho are formed as products of
+// float pairs (relative error below 2^-45) on the float32 and integer pipes,
+// exponents apart, so any magnitude a double holds works.  Saves the three
+// float64 products that formed the two squares, of the 22 float64 operations
+// of a face state (the float64 pipe issues a 64th of the float32 pipe's rate).
+__device__ __forceinline__ void ctot_pair_of(double k, double P, double ir, const Phys& p, float& h, float& l) {
+  float kh, kl, ph, pl, rh, rl;
+  int ek, ep, er;
+  split_pair(k, kh, kl, ek);
+  split_pair(P, ph, pl, ep);
+  split_pair(ir, rh, rl, er);
+  const float v = kh * rh;
+  const float ve = fmaf(kl, rh, fmaf(kh, rl, fmaf(kh, rh, -v)));
+  const float t = ph * rh;
+  const float te = fmaf(pl, rh, fmaf(ph, rl, fmaf(ph, rh, -t)));
+  const float a = t * p.gxh;
+  const float ae = fmaf(te, p.gxh, fmaf(t, p.gxl, fmaf(t, p.gxh, -a)));
+  float sv, cv, sa, ca;
+  sqrt_of_pair(v, ve, ek + er - 2046, sv, cv);
+  sqrt_of_pair(a, ae, ep + er - 2046 + p.gxe, sa, ca);
+  // zero (or subnormal) k or P: that speed is 0; negative or NaN anywhere: NaN
+  const bool rok = (unsigned)(er - 1) < 2046u;
+  const float nan = __int_as_float(0x7fc00000);
+  if (!(rok && (unsigned)(ek - 1) < 2046u)) {
+    sv = rok && ek == 0 ? 0.0f : nan;
+    cv = 0.0f;
+  }
+  if (!(rok && (unsigned)(ep - 1) < 2046u)) {
+    sa = rok && ep == 0 ? 0.0f : nan;
+    ca = 0.0f;
+  }
+  pair_sum(sv, cv, sa, ca, h, l);
+}
+
+// 1/sqrt(w): the hardware approximation (20 bits) and one third-order step,
+// y (1 + e/2 + 3 e^2/8) with e = 1 - w y^2, which cubes its error: about one
+// ulp in five float64 operations instead of an IEEE square root and division.
+__device__ __forceinline__ double rsqrt_nr(double w) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(w));
+  const double e = fma(-(w * y), y, 1.0);
+  return fma(y * e, fma(0.375, e, 0.5), y);
+}
+
 // Effective sound speed a/xi from a^2 and the factor f = 1 - 1/xi^2: constant
 // xi, or the C_max law xi = [1 + (a/C_max)^4]^(1/4) (Eq. cx, Sec. 4.3), for
 // which a/xi = sqrt(a^2 / sqrt(w)) and f = 1 - 1/sqrt(w), w = 1 + a^4/C_max^4.
@@ -165,21 +295,26 @@ __device__ __forceinline__ double sound_over_xi(double a2, const Phys& p) {
   return sqrt_ctot(a2) * p.inv_xi;
 }
 __device__ __forceinline__ double f_of(double a2, const Phys& p) {
-  if (p.use_cmax) return 1.0 - 1.0 / sqrt(fma(a2 * a2, p.inv_cmax4, 1.0));
+  if (p.use_cmax) return 1.0 - rsqrt_nr(fma(a2 * a2, p.inv_cmax4, 1.0));
   return p.f;
 }
 
-// a/xi of a state for c_tot: constant xi as sqrt((a/xi)^2), or the C_max law.
+// The approximate RSST characteristic speed c_tot = |V| + a/xi (Sec. 4.2) of
+// a state with k = rho |V|^2 as a normalised float pair.
 template <bool CV>
-__device__ __forceinline__ double ctot_sound(const Phys& p, double rho, double P, double ir) {
-  if (p.use_cmax) return sound_over_xi(Eos<CV>::sound2(p, rho, P, ir), p);
-  return sqrt_ctot(Eos<CV>::sound2_over_xi2(p, rho, P, ir));
+__device__ __forceinline__ void ctot_of(const Phys& p, double rho, double k, double P, double ir, float& h, float& l) {
+  if (p.use_cmax) {
+    const double a2 = Eos<CV>::sound2(p, rho, P, ir);
+    ctot_pair(k * ir, a2 * rsqrt_nr(fma(a2 * a2, p.inv_cmax4, 1.0)), h, l);
+  } else if constexpr (CV) {
+    ctot_pair(k * ir, Eos<CV>::sound2_over_xi2(p, rho, P, ir), h, l);
+  } else {
+    ctot_pair_of(k, P, ir, p, h, l);
+  }
 }
 
-// The Euler flux along dimension D, F, and the approximate RSST
-// characteristic speed c_tot = |V| + a/xi of one state (Eq. pvs_dt0; Sec. 4.2)
-// as a float pair ch + cl: for a constant xi from ctot_pair on the float32
-// pipe, under the C_max law from the float64 form.
+// The Euler flux along dimension D, F (Eq. pvs_dt0), and c_tot of one state
+// as the float pair ch + cl.  k = rho |V|^2 = m.V feeds the pressure directly.
 template <int NV, int D, bool CV = false>
 __device__ __forceinline__ void euler_flux(const double (&q)[NV], const Phys& p,
                                            double (&F)[NV], float& ch, float& cl) {
@@ -187,20 +322,14 @@ __device__ __forceinline__ void euler_flux(const double (&q)[NV], const Phys& p,
   const double rho = q[0];
   const double ir = rcp_nr(rho);
   double v[ND];
-  double v2 = 0.0;
+  double k = 0.0;
 #pragma unroll
   for (int e = 0; e < ND; ++e) {
     v[e] = q[1 + e] * ir;
-    v2 += v[e] * v[e];
+    k = e == 0 ? q[1] * v[0] : fma(q[1 + e], v[e], k);
   }
-  const double P = Eos<CV>::pressure(p, rho, q[NV - 1], rho * v2);
-  if (p.use_cmax) {
-    const double c = sqrt_ctot(v2) + ctot_sound<CV>(p, rho, P, ir);
-    ch = __double2float_rn(c);
-    cl = __double2float_rn(c - (double)ch);
-  } else {
-    ctot_pair(v2, Eos<CV>::sound2_over_xi2(p, rho, P, ir), ch, cl);
-  }
+  const double P = Eos<CV>::pressure(p, rho, q[NV - 1], k);
+  ctot_of<CV>(p, rho, k, P, ir, ch, cl);
   F[0] = q[1 + D];
 #pragma unroll
   for (int e = 0; e < ND; ++e) F[1 + e] = (e == D) ? fma(q[1 + e], v[D], P) : q[1 + e] * v[D];
@@ -219,7 +348,7 @@ __device__ __forceinline__ void llf_flux_x2(const double (&qL)[NV], const double
   euler_flux<NV, D, CV>(qL, p, FL, hL, lL);
   euler_flux<NV, D, CV>(qR, p, FR, hR, lR);
   const bool left = hL > hR || (hL == hR && lL >= lR);  // normalised pairs order like their values
-  const double alpha = f2d_bits(left ? hL : hR) + f2d_bits(left ? lL : lR);
+  const double alpha = pair_to_double(left ? hL : hR, left ? lL : lR);
 #pragma unroll
   for (int k = 0; k < NV; ++k) G[k] = fma(-alpha, qR[k] - qL[k], FL[k] + FR[k]);
 }
@@ -262,39 +391,44 @@ __device__ __forceinline__ void rsst_rhs(const double (&q)[NV], double (&dU)[NV]
   if (p.variant != RSST_EULER) {
     const double ir = rcp_nr(rho);
     double v[ND];
-    double v2 = 0.0, vdm = 0.0;
+    double k = 0.0;  // rho |V|^2
 #pragma unroll
     for (int e = 0; e < ND; ++e) {
       v[e] = q[1 + e] * ir;
-      v2 += v[e] * v[e];
-      vdm += v[e] * dU[1 + e];
+      k = e == 0 ? q[1] * v[0] : fma(q[1 + e], v[e], k);
     }
-    const double P = Eos<CV>::pressure(p, rho, q[NV - 1], rho * v2);
-    const double e_int = Eos<CV>::internal_energy(p, rho, P);
-    const double kin = 0.5 * rho * v2;
-    double s, r0, rv, rE;  // r = (r0, rv * V, rE); rv in {0, 1/a^2, 1}
+    const double P = Eos<CV>::pressure(p, rho, q[NV - 1], k);
+    const double kin = 0.5 * k;
     const int var = p.variant;
+    const double f = p.use_cmax ? f_of(Eos<CV>::sound2(p, rho, P, ir), p) : p.f;
+    const bool mom = var == RSST_PVS || var == RSST_DVS;  // the correction moves momentum
+    // e + P + rho V^2/2, or minus
+    const double H = Eos<CV>::enthalpy(p, rho, P) + (mom ? kin : -kin);
+    double w, wE;  // f s r0 and f s rE / H
     if (var == RSST_PVS || var == RSST_PMS || var == RSST_PD) {
-      s = Eos<CV>::inv_de_dP(p, rho, P) * (Eos<CV>::half_v2_minus_de_drho(p, v2, P) * dU[0] - vdm + dU[NV - 1]);
+      double s = fma(Eos<CV>::half_v2_minus_de_drho(p, kin * ir, P), dU[0], dU[NV - 1]);
+#pragma unroll
+      for (int e = 0; e < ND; ++e) s = fma(-v[e], dU[1 + e], s);
+      const double fs = Eos<CV>::f_over_de_dP(p, f, rho, P) * s;
       if (var == RSST_PD) {
-        r0 = 0.0; rv = 0.0; rE = Eos<CV>::de_dP(p, rho, P);
+        dU[NV - 1] = fma(-fs, Eos<CV>::de_dP(p, rho, P), dU[NV - 1]);
+        w = wE = 0.0;
       } else {
-        const double ia2 = rcp_nr(Eos<CV>::sound2(p, rho, P, ir));  // 1/a^2
-        r0 = ia2;
-        rv = (var == RSST_PVS) ? ia2 : 0.0;
-        rE = (var == RSST_PVS ? (e_int + P + kin) : (e_int + P - kin)) * ia2 * ir;
+        wE = fs * Eos<CV>::inv_rho_a2(p, rho, P);
+        w = wE * rho;
       }
     } else {  // DVS, DMS
-      s = dU[0];
-      r0 = 1.0;
-      rv = (var == RSST_DVS) ? 1.0 : 0.0;
-      rE = (var == RSST_DVS ? (e_int + P + kin) : (e_int + P - kin)) * ir;
+      w = f * dU[0];
+      wE = w * ir;
     }
-    const double fs = f_of(Eos<CV>::sound2(p, rho, P, ir), p) * s;
-    dU[0] -= fs * r0;
+    if (var != RSST_PD) {
+      dU[0] -= w;
+      if (mom) {
 #pragma unroll
-    for (int e = 0; e < ND; ++e) dU[1 + e] -= fs * (rv * v[e]);
-    dU[NV - 1] -= fs * rE;
+        for (int e = 0; e < ND; ++e) dU[1 + e] = fma(-w, v[e], dU[1 + e]);
+      }
+      dU[NV - 1] = fma(-wE, H, dU[NV - 1]);
+    }
   }
   if (p.has_grav) {
     double mg = 0.0;
@@ -307,29 +441,42 @@ __device__ __forceinline__ void rsst_rhs(const double (&q)[NV], double (&dU)[NV]
   }
 }
 
-// CFL rate sum_d c_tot/dx_d of a cell and its physical-state check.
+// Half of a double (as 0.5 * x rounds it), on the integer pipe.
+__device__ __forceinline__ double half_of(double x) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  const unsigned long long sign = b & (1ull << 63), mag = b ^ sign;
+  const unsigned e = (unsigned)(mag >> 52);
+  if (e == 2047u) return x;
+  // at and below the smallest normal exponent the pattern counts units of 2^-1074
+  const unsigned long long h = e >= 2u ? mag - (1ull << 52) : (mag + ((mag >> 1) & 1ull)) >> 1;
+  return __longlong_as_double((long long)(sign | h));
+}
+
+// From the bit pattern (a float64 compare occupies the float64 pipe).
+__device__ __forceinline__ bool finite_bits(double x) { return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000; }
+__device__ __forceinline__ bool positive_finite(double x) {
+  return __double_as_longlong(x) > 0 && __double2hiint(x) < 0x7ff00000;
+}
+
+// CFL rate sum_d c_tot/dx_d of a cell and its physical-state check.  c_tot is
+// the float pair of the LLF speed; the checks read bit patterns.
 template <int NV, bool CV = false>
 __device__ __forceinline__ double cfl_rate(const double (&q)[NV], const Phys& p, bool& ok) {
   constexpr int ND = NV - 2;
   const double rho = q[0];
   const double ir = rcp_nr(rho);
-  double v2 = 0.0;
-  bool fin = isfinite(q[0]) && isfinite(q[NV - 1]);
+  double k = 0.0;
+  bool fin = finite_bits(q[NV - 1]);
 #pragma unroll
   for (int e = 0; e < ND; ++e) {
-    const double ve = q[1 + e] * ir;
-    v2 += ve * ve;
-    fin = fin && isfinite(q[1 + e]);
+    k = e == 0 ? q[1] * (q[1] * ir) : fma(q[1 + e], q[1 + e] * ir, k);
+    fin = fin && finite_bits(q[1 + e]);
   }
-  const double P = Eos<CV>::pressure(p, rho, q[NV - 1], rho * v2);
-  ok = fin && rho > 0.0 && P > 0.0 && Eos<CV>::admissible(p, rho);
-  if (p.use_cmax) return (sqrt_ctot(v2) + ctot_sound<CV>(p, rho, P, ir)) * p.sum_inv_dx;
-  // c_tot as the float pair of the LLF speed (relative error below 2^-41,
-  // tighter than the float64-pipe square root's 2^-40), on the float32 and
-  // integer pipes
+  const double P = Eos<CV>::pressure(p, rho, q[NV - 1], k);
+  ok = fin && positive_finite(rho) && positive_finite(P) && Eos<CV>::admissible(p, rho);
   float ch, cl;
-  ctot_pair(v2, Eos<CV>::sound2_over_xi2(p, rho, P, ir), ch, cl);
-  return (f2d_bits(ch) + f2d_bits(cl)) * p.sum_inv_dx;
+  ctot_of<CV>(p, rho, k, P, ir, ch, cl);
+  return pair_to_double(ch, cl) * p.sum_inv_dx;
 }
 
 }  // namespace rsst
