@@ -115,13 +115,15 @@ static int make_tmap_2d(CUtensorMap* m, void* base, const Geom& g, int nv, int b
   return RSST_OK;
 }
 
-// Tiled float64 map of a padded 2D/3D state [nvar][pz][py][pitch]: the
-// float64 stage kernel's halo tile (box sx x sy [x sz]) of every field.
-static int make_tmap_f64(CUtensorMap* m, void* base, const Geom& g, int tile, int nv) {
+// Tiled map of a padded 2D/3D state [nvar][pz][py][pitch] of 8-byte values
+// (float64, or double-float moved as such): the stage kernel's halo tile (box
+// sx x sy [x sz]) of every field.
+static int make_tmap_f64(CUtensorMap* m, void* base, const Geom& g, bool dfp, int tile, int nv) {
   auto enc = tensor_map_encoder();
   if (!enc) { rsst_set_error("cuTensorMapEncodeTiled unavailable from the CUDA driver"); return RSST_ECUDA; }
   int sx, sy, sz;
-  rsst_stage_fp64_box(g, tile, &sx, &sy, &sz);
+  if (dfp) rsst_stage_df_box(g, tile, &sx, &sy, &sz);
+  else rsst_stage_fp64_box(g, tile, &sx, &sy, &sz);
   const bool d3 = g.ndim == 3;
   const cuuint32_t rank = d3 ? 4 : 3;
   const cuuint64_t dims[4] = {(cuuint64_t)g.pitch, (cuuint64_t)g.py, d3 ? (cuuint64_t)g.pz : (cuuint64_t)nv,
@@ -363,7 +365,8 @@ extern "C" int rsst_init(rsst_handle** out, const rsst_config* cfg, void* stream
       if (rc != RSST_OK) goto fail;
     }
   }
-  if (cfg->precision == RSST_FP64 && cfg->ndim >= 2) {
+  if (cfg->precision != RSST_FP32_PERT && cfg->ndim >= 2) {
+    const bool dfp = cfg->precision == RSST_FP64_DF;
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) {
@@ -372,10 +375,10 @@ extern "C" int rsst_init(rsst_handle** out, const rsst_config* cfg, void* stream
       rc = RSST_ECUDA;
       goto fail;
     }
-    h->use_tma_fp64 = 1;
-    h->fp64_tile = rsst_stage_fp64_tile(h->g, sms);
+    h->use_tma_fp64 = !dfp;
+    h->tile = dfp ? rsst_stage_df_tile(h->g, sms) : rsst_stage_fp64_tile(h->g, sms);
     for (int b = 0; b < 2; ++b) {
-      rc = make_tmap_f64(&h->tmap[b], h->buf[b], h->g, h->fp64_tile, nv);
+      rc = make_tmap_f64(&h->tmap[b], h->buf[b], h->g, dfp, h->tile, nv);
       if (rc != RSST_OK) goto fail;
     }
   }
@@ -483,7 +486,7 @@ static int plain_steps(rsst_handle* h, double dt, int nsteps, cudaStream_t st) {
   a.flag = h->d_flag;
   a.dt_fixed = dt > 0.0 ? dt : 0.0;
   a.stall_ns = h->stall_ns;
-  a.tile = h->fp64_tile;
+  a.tile = h->tile;
   T* U = (T*)h->buf[0];
   T* Us = (T*)h->buf[1];
   for (int s = 0; s < nsteps; ++s) {
@@ -494,7 +497,7 @@ static int plain_steps(rsst_handle* h, double dt, int nsteps, cudaStream_t st) {
     a.out = Us;
     a.dU_out = h->rec_dU[0];
     if constexpr (std::is_same<T, double>::value) RC_TRY(rsst_launch_stage_fp64(h->use_tma_fp64 ? &h->tmap[0] : nullptr, a, st));
-    else if constexpr (std::is_same<T, float2>::value) RC_TRY(rsst_launch_stage_df(a, st));
+    else if constexpr (std::is_same<T, float2>::value) RC_TRY(rsst_launch_stage_df(&h->tmap[0], a, st));
     else if (h->use_tma2d) RC_TRY(rsst_launch_stage2d_tma(&h->tmap[0], a, st));
     else if (h->use_tma3d) RC_TRY(rsst_launch_stage3d_tma(&h->tmap[0], a, st));
     else RC_TRY(rsst_launch_stage_fp32(a, st));
@@ -504,7 +507,7 @@ static int plain_steps(rsst_handle* h, double dt, int nsteps, cudaStream_t st) {
     a.out = U;
     a.dU_out = h->rec_dU[1];
     if constexpr (std::is_same<T, double>::value) RC_TRY(rsst_launch_stage_fp64(h->use_tma_fp64 ? &h->tmap[1] : nullptr, a, st));
-    else if constexpr (std::is_same<T, float2>::value) RC_TRY(rsst_launch_stage_df(a, st));
+    else if constexpr (std::is_same<T, float2>::value) RC_TRY(rsst_launch_stage_df(&h->tmap[1], a, st));
     else if (h->use_tma2d) RC_TRY(rsst_launch_stage2d_tma(&h->tmap[1], a, st));
     else if (h->use_tma3d) RC_TRY(rsst_launch_stage3d_tma(&h->tmap[1], a, st));
     else RC_TRY(rsst_launch_stage_fp32(a, st));

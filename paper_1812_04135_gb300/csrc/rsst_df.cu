@@ -1,11 +1,22 @@
 // Double-float kernels (precision RSST_FP64_DF): the state is stored as
 // float32 pairs (hi, lo) in the padded layout (8 bytes per value, like
 // float64) and the fused stage kernel computes in double-float on the
-// float32 pipe.  Tile structure as in the float64 kernel (rsst_fp64.cu).
+// float32 pipe.  Tile structure as in the float64 kernel (rsst_fp64.cu): the
+// halo tile by one TMA copy in 2D and 3D, 1D/2D tiles with every axis at once,
+// 3D tiles axis by axis.
+//
+// What bounds it: instruction issue and the float32 pipe (a double-float
+// operation is 7 to 15 float32 instructions).  Thread instructions a 2D cell
+// in stage 1 (ncu, 512^2): 4100 -> 2743, by products fed unnormalised into
+// sums (df_fma, the three-term sum of the LLF flux), twice-flux faces, slopes
+// in pairs that share a difference, rho |V|^2 = m.V, the C_max law and the
+// stage as template arguments, and the tile by TMA instead of loads and index
+// arithmetic.  512^2: 40.9 -> 27.2 us a stage; 3D 90 x 70 x 50: 112 -> 74 us.
 #include "rsst_common.cuh"
 #include "rsst_internal.h"
 #include "rsst_attr.h"
 #include "rsst_math_df.cuh"
+#include "rsst_tma.cuh"
 
 namespace rsst {
 
@@ -81,6 +92,8 @@ __device__ __forceinline__ void block_max_df(df x, double* dst, df* sred) {
   }
 }
 
+// Tile structure of the float64 kernel (rsst_fp64.cu): 1D/2D tiles hold the
+// half slopes and faces of every axis at once, 3D tiles go axis by axis.
 template <int NDIM, int BX, int BY, int BZ, int NT>
 struct TileCfgDF {
   static constexpr int NV = NDIM + 2;
@@ -89,98 +102,106 @@ struct TileCfgDF {
   static constexpr int SCELLS = SX * SY * SZ;
   static constexpr int NCELL = BX * BY * BZ;
   static constexpr int CPT = (NCELL + NT - 1) / NT;
-  static constexpr int FX = (BX + 1) * BY * BZ;
-  static constexpr int FY = NDIM >= 2 ? BX * (BY + 1) * BZ : 0;
-  static constexpr int FZ = NDIM >= 3 ? BX * BY * (BZ + 1) : 0;
-  static constexpr int FMAX = FX > FY ? (FX > FZ ? FX : FZ) : (FY > FZ ? FY : FZ);
-  // each cell's MC slope along the current axis, once per cell (cells -1 .. B
-  // along that axis), when it fits beside the tile with room for several CTAs
-  static constexpr int EX0 = (BX + 2) * BY * BZ, EX1 = NDIM >= 2 ? BX * (BY + 2) * BZ : 0;
-  static constexpr int EX2 = NDIM >= 3 ? BX * BY * (BZ + 2) : 0;
-  static constexpr int EXM = EX0 > EX1 ? (EX0 > EX2 ? EX0 : EX2) : (EX1 > EX2 ? EX1 : EX2);
-  static constexpr bool SLOPES = NDIM <= 2 || sizeof(df) * (size_t)NV * (SCELLS + FMAX + EXM) <= (size_t)76 * 1024;
-  static constexpr int SEMAX = SLOPES ? EXM : 0;
-  static constexpr size_t SMEM = sizeof(df) * ((size_t)NV * (SCELLS + FMAX + SEMAX) + 64);
+  static constexpr int F0 = (BX + 1) * BY * BZ, F1 = NDIM >= 2 ? BX * (BY + 1) * BZ : 0;
+  static constexpr int F2 = NDIM >= 3 ? BX * BY * (BZ + 1) : 0;
+  static constexpr int E0 = (BX + 2) * BY * BZ, E1 = NDIM >= 2 ? BX * (BY + 2) * BZ : 0;
+  static constexpr int E2 = NDIM >= 3 ? BX * BY * (BZ + 2) : 0;
+  static constexpr int max3(int a, int b, int c) { return a > b ? (a > c ? a : c) : (b > c ? b : c); }
+  static constexpr bool ALL = NDIM <= 2;
+  static constexpr int FMAX = ALL ? F0 + F1 : max3(F0, F1, F2);
+  static constexpr int EMAX = ALL ? E0 + E1 : max3(E0, E1, E2);
+  // halo tile, faces, half slopes, the block reduction and dt (64 values), the tile copy's mbarrier
+  static constexpr size_t SMEM = sizeof(df) * ((size_t)NV * (SCELLS + FMAX + EMAX) + 64) + 16;
+  static constexpr uint32_t TILE_BYTES = (uint32_t)(sizeof(df) * NV * SCELLS);
+  static_assert(BX % 2 == 0 && (NDIM < 2 || BY % 2 == 0) && (NDIM < 3 || BZ % 2 == 0), "slopes are taken in pairs");
 };
 
-template <int NDIM, int BX, int BY, int BZ, int NT, int D>
-__device__ __forceinline__ void face_pass_df(const df* __restrict__ su, df* __restrict__ sf, df* __restrict__ ss,
+// Half MC slopes along D of the pair of neighbouring slope cells e (tile
+// coordinates -1 .. B along D, 0 .. B-1 across); the two share a difference.
+template <class C, int BX, int BY, int BZ, int D>
+__device__ __forceinline__ void slope_pair_df(const df* __restrict__ su, df* __restrict__ ss, int e) {
+  constexpr int STRIDE = D == 0 ? 1 : (D == 1 ? C::SX : C::SX * C::SY);
+  constexpr int XX = BX + 2 * (D == 0), YY = BY + 2 * (D == 1);
+  constexpr int PX = D == 0 ? XX / 2 : XX, PY = D == 1 ? YY / 2 : YY;
+  const int ex = e % PX * (D == 0 ? 2 : 1);
+  const int t = e / PX;
+  const int ey = t % PY * (D == 1 ? 2 : 1);
+  const int ez = t / PY * (D == 2 ? 2 : 1);
+  const int s0 = (ez - (D == 2) + C::HZ) * C::SX * C::SY + (ey - (D == 1) + C::HY) * C::SX + (ex - (D == 0) + C::HX);
+  const int o = (ez * YY + ey) * XX + ex;
+  constexpr int STRIDE_E = D == 0 ? 1 : (D == 1 ? XX : XX * YY);
+#pragma unroll
+  for (int v = 0; v < C::NV; ++v) {
+    const df* sv = su + v * C::SCELLS + s0;
+    const df um = sv[-STRIDE], u0 = sv[0], u1 = sv[STRIDE], up = sv[2 * STRIDE];
+    const df d = u1 - u0;
+    ss[v * C::EMAX + o] = half_mc_df(u0 - um, d);
+    ss[v * C::EMAX + o + STRIDE_E] = half_mc_df(d, up - u1);
+  }
+}
+
+// Twice the LLF flux of the face between tile cells sl | s0 (slopes el, er);
+// fld lists the fields with the normal momentum second.
+template <class C, bool CMAX, int D>
+__device__ __forceinline__ void face_df(const df* __restrict__ su, const df* __restrict__ ss, df* __restrict__ sf,
+                                        const PhysDF& p, int sl, int s0, int el, int er, int f,
+                                        const int (&fld)[C::NV]) {
+  constexpr int NV = C::NV;
+  df qL[NV], qR[NV], F[NV];
+#pragma unroll
+  for (int v = 0; v < NV; ++v) {
+    qL[v] = su[fld[v] * C::SCELLS + sl] + ss[fld[v] * C::EMAX + el];
+    qR[v] = su[fld[v] * C::SCELLS + s0] - ss[fld[v] * C::EMAX + er];
+  }
+  llf_flux_x2_df<NV, D, CMAX>(qL, qR, p, F);
+#pragma unroll
+  for (int v = 0; v < NV; ++v) sf[fld[v] * C::FMAX + f] = F[v];
+}
+
+// 2F above minus 2F below tile cell (cx, cy, cz) along D, per field.
+template <class C, int BX, int BY, int BZ, int D>
+__device__ __forceinline__ void face_diff_df(const df* __restrict__ sf, int cx, int cy, int cz, df (&d)[C::NV]) {
+  constexpr int EX = BX + (D == 0), EY = BY + (D == 1);
+  const int flo = (cz * EY + cy) * EX + cx;
+  const int fhi = flo + (D == 0 ? 1 : (D == 1 ? EX : EX * EY));
+#pragma unroll
+  for (int v = 0; v < C::NV; ++v) d[v] = sf[v * C::FMAX + fhi] - sf[v * C::FMAX + flo];
+}
+
+// One axis of a 3D tile: slopes, faces, and each thread's cells' divergence.
+template <int NDIM, int BX, int BY, int BZ, int NT, int D, bool CMAX>
+__device__ __forceinline__ void axis_pass_df(const df* __restrict__ su, df* __restrict__ sf, df* __restrict__ ss,
                                              const PhysDF& p, const Geom& g, int i0, int j0, int k0,
                                              df (&dU)[TileCfgDF<NDIM, BX, BY, BZ, NT>::CPT][NDIM + 2]) {
   using C = TileCfgDF<NDIM, BX, BY, BZ, NT>;
-  constexpr int NV = C::NV;
-  constexpr int EX = BX + (D == 0), EY = BY + (D == 1), EZ = BZ + (D == 2);
-  constexpr int NF = EX * EY * EZ;
+  constexpr int NE = D == 0 ? C::E0 : (D == 1 ? C::E1 : C::E2), NF = D == 0 ? C::F0 : (D == 1 ? C::F1 : C::F2);
+  constexpr int EX = BX + (D == 0), EY = BY + (D == 1);
   constexpr int STRIDE = D == 0 ? 1 : (D == 1 ? C::SX : C::SX * C::SY);
-  constexpr int XX = BX + 2 * (D == 0), YY = BY + 2 * (D == 1), ZZ = BZ + 2 * (D == 2);
-  constexpr int NE = XX * YY * ZZ;
-  const int baseD = D == 0 ? i0 : (D == 1 ? j0 : k0);
-  if constexpr (C::SLOPES) {
-    for (int e = threadIdx.x; e < NE; e += NT) {
-      const int ex = e % XX;
-      const int t = e / XX;
-      const int ey = t % YY;
-      const int ez = t / YY;
-      const int s0 = (ez - (D == 2) + C::HZ) * C::SX * C::SY + (ey - (D == 1) + C::HY) * C::SX + (ex - (D == 0) + C::HX);
-#pragma unroll
-      for (int v = 0; v < NV; ++v) {
-        const df* sv = su + v * C::SCELLS + s0;
-        ss[v * C::SEMAX + e] = mc_df(sv[0] - sv[-STRIDE], sv[STRIDE] - sv[0]);
-      }
-    }
-    __syncthreads();
-  }
-  for (int fid = threadIdx.x; fid < NF; fid += NT) {
-    const int fx = fid % EX;
-    const int t = fid / EX;
-    const int fy = t % EY;
-    const int fz = t / EY;
-    const int fD = D == 0 ? fx : (D == 1 ? fy : fz);
-    const bool valid = (i0 + fx <= g.n[0] - (D == 0 ? 0 : 1)) && (NDIM < 2 || j0 + fy <= g.n[1] - (D == 1 ? 0 : 1)) &&
-                       (NDIM < 3 || k0 + fz <= g.n[2] - (D == 2 ? 0 : 1)) && (baseD + fD <= g.n[D]);
-    if (!valid) continue;
+  constexpr int XX = BX + 2 * (D == 0), YY = BY + 2 * (D == 1);
+  constexpr int STRIDE_E = D == 0 ? 1 : (D == 1 ? XX : XX * YY);
+  constexpr int fld[5] = {0, 1, 2, 3, 4};
+  for (int e = threadIdx.x; e < NE / 2; e += NT) slope_pair_df<C, BX, BY, BZ, D>(su, ss, e);
+  __syncthreads();
+  for (int f = threadIdx.x; f < NF; f += NT) {
+    const int fx = f % EX, t = f / EX, fy = t % EY, fz = t / EY;
+    if (i0 + fx > g.n[0] - (D == 0 ? 0 : 1) || j0 + fy > g.n[1] - (D == 1 ? 0 : 1) ||
+        k0 + fz > g.n[2] - (D == 2 ? 0 : 1))
+      continue;
     const int s0 = (fz + C::HZ) * C::SX * C::SY + (fy + C::HY) * C::SX + (fx + C::HX);
-    df qL[NV], qR[NV];
-    if constexpr (C::SLOPES) {
-      constexpr int STRIDE_E = D == 0 ? 1 : (D == 1 ? XX : XX * YY);
-      const int er = ((fz + (D == 2)) * YY + (fy + (D == 1))) * XX + (fx + (D == 0));
-#pragma unroll
-      for (int v = 0; v < NV; ++v) {
-        const df* sv = su + v * C::SCELLS + s0;
-        qL[v] = sv[-STRIDE] + scale(ss[v * C::SEMAX + er - STRIDE_E], 0.5f);
-        qR[v] = sv[0] - scale(ss[v * C::SEMAX + er], 0.5f);
-      }
-    } else {
-#pragma unroll
-      for (int v = 0; v < NV; ++v) {
-        const df* sv = su + v * C::SCELLS + s0;
-        const df um2 = sv[-2 * STRIDE], um1 = sv[-STRIDE], u0 = sv[0], up1 = sv[STRIDE];
-        const df dm = um1 - um2, d0 = u0 - um1, dp = up1 - u0;
-        qL[v] = um1 + scale(mc_df(dm, d0), 0.5f);
-        qR[v] = u0 - scale(mc_df(d0, dp), 0.5f);
-      }
-    }
-    df F[NV];
-    llf_flux_df<NV, D>(qL, qR, p, F);
-#pragma unroll
-    for (int v = 0; v < NV; ++v) sf[v * C::FMAX + fid] = F[v];
+    const int er = ((fz + (D == 2)) * YY + (fy + (D == 1))) * XX + (fx + (D == 0));
+    face_df<C, CMAX, D>(su, ss, sf, p, s0 - STRIDE, s0, er - STRIDE_E, er, f, fld);
   }
   __syncthreads();
-  const df idx = p.inv_dx[D];
 #pragma unroll
   for (int c = 0; c < C::CPT; ++c) {
     const int cell = threadIdx.x + c * NT;
     if (cell >= C::NCELL) break;
-    const int cx = cell % BX;
-    const int t = cell / BX;
-    const int cy = t % BY;
-    const int cz = t / BY;
-    const int flo = (cz * EY + cy) * EX + cx;
-    const int fhi = flo + (D == 0 ? 1 : (D == 1 ? EX : EX * EY));
+    df d[C::NV];
+    face_diff_df<C, BX, BY, BZ, D>(sf, cell % BX, cell / BX % BY, cell / BX / BY, d);
 #pragma unroll
-    for (int v = 0; v < NV; ++v) dU[c][v] = dU[c][v] - (sf[v * C::FMAX + fhi] - sf[v * C::FMAX + flo]) * idx;
+    for (int v = 0; v < C::NV; ++v)
+      dU[c][v] = D == 0 ? d[v] * p.nhalf_inv_dx[D] : df_fma(d[v], p.nhalf_inv_dx[D], dU[c][v]);
   }
-  __syncthreads();
 }
 
 struct DFArgs {
@@ -198,15 +219,16 @@ struct DFArgs {
   double dt_fixed;
 };
 
-template <int NDIM, int BX, int BY, int BZ, int NT>
-__global__ void __launch_bounds__(NT) stage_df_kernel(const DFArgs a) {
+template <int NDIM, int BX, int BY, int BZ, int NT, int MINB, bool CMAX, int ST>
+__global__ void __launch_bounds__(NT, MINB)
+    stage_df_kernel(const __grid_constant__ CUtensorMap tin, const DFArgs a) {
   using C = TileCfgDF<NDIM, BX, BY, BZ, NT>;
   constexpr int NV = C::NV;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
+  extern __shared__ __align__(128) unsigned char smem_raw[];
   df* su = reinterpret_cast<df*>(smem_raw);
   df* sf = su + NV * C::SCELLS;
-  df* ss = sf + NV * C::FMAX;  // slopes, when they fit
-  df* sred = ss + NV * C::SEMAX;
+  df* ss = sf + NV * C::FMAX;  // half slopes
+  df* sred = ss + NV * C::EMAX;
   double* sdt = reinterpret_cast<double*>(sred + 32);
   const Geom& g = a.g;
   const PhysDF& p = a.q;
@@ -214,36 +236,92 @@ __global__ void __launch_bounds__(NT) stage_df_kernel(const DFArgs a) {
   if (threadIdx.x == 0) {
     const double dt = a.dt_fixed > 0.0 ? a.dt_fixed : a.p.cfl / a.scal[a.slot];
     *sdt = dt;
-    if (a.stage == 1 && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0) {
+    if (ST == 1 && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0) {
       a.scal[a.slot ^ 1] = 0.0;
       a.scal[2] = dt;
       a.scal[3] += dt;
     }
   }
-  for (int id = threadIdx.x; id < NV * C::SCELLS; id += NT) {
-    const int v = id / C::SCELLS;
-    const int r = id - v * C::SCELLS;
-    const int lx = r % C::SX;
-    const int t = r / C::SX;
-    const int ly = t % C::SY;
-    const int lz = t / C::SY;
-    const int gi = i0 + lx - C::HX, gj = j0 + ly - C::HY, gk = k0 + lz - C::HZ;
-    df val = {0.0f, 0.0f};
-    if (gi <= g.n[0] + 1 && (NDIM < 2 || gj <= g.n[1] + 1) && (NDIM < 3 || gk <= g.n[2] + 1))
-      val = ld_df(a.in, v * g.fstride + pidx(g, gi, gj, gk));
-    su[id] = val;
+  if constexpr (NDIM >= 2) {
+    // the halo tile of all fields by one TMA copy (as in rsst_fp64.cu: a
+    // double-float is an 8-byte element of the same layout)
+    uint64_t* bar = reinterpret_cast<uint64_t*>(sred + 64);
+    if (threadIdx.x == 32) {
+      mbar_init(bar, 1);
+      fence_mbar_init();
+      fence_proxy_async_smem();
+      mbar_expect_tx(bar, C::TILE_BYTES);
+      if constexpr (NDIM == 2) tma_load_3d(su, &tin, bar, i0 + g.xoff - C::HX, j0, 0);
+      else tma_load_4d(su, &tin, bar, i0 + g.xoff - C::HX, j0, k0, 0);
+    }
+    __syncthreads();  // the barrier is initialised, dt is there
+    // giving up (flag, one more bounded wait for the copy) is decided by the whole block
+    if (__syncthreads_or(!mbar_wait_bounded(bar, 0u))) {
+      if (threadIdx.x == 0) {
+        atomicOr(a.flag, RSST_FLAG_TIMEOUT);
+        mbar_wait_bounded(bar, 0u);
+      }
+      return;
+    }
+  } else {
+    for (int id = threadIdx.x; id < NV * C::SCELLS; id += NT) {
+      const int v = id / C::SCELLS, lx = id - v * C::SCELLS;
+      const int gi = i0 + lx - C::HX;
+      su[id] = gi <= g.n[0] + 1 ? ld_df(a.in, v * g.fstride + pidx(g, gi, 0, 0)) : df{0.0f, 0.0f};
+    }
+    __syncthreads();
   }
-  __syncthreads();
   const df dt = df_from(*sdt);
 
   df dU[C::CPT][NV];
+  if constexpr (C::ALL) {
+    constexpr int PE = (C::E0 / 2 + 31) / 32 * 32;  // axis y starts at a whole warp
+    for (int e = threadIdx.x; e < (NDIM == 1 ? C::E0 / 2 : PE + C::E1 / 2); e += NT) {
+      if (e < PE) {
+        if (e < C::E0 / 2) slope_pair_df<C, BX, BY, BZ, 0>(su, ss, e);
+      } else if constexpr (NDIM == 2) {
+        slope_pair_df<C, BX, BY, BZ, 1>(su, ss + C::E0, e - PE);
+      }
+    }
+    __syncthreads();
+    // the x and y faces as one list; the axis enters through strides and the
+    // order of the momenta only (no divergence in a warp that holds both)
+    for (int f = threadIdx.x; f < C::F0 + C::F1; f += NT) {
+      const bool isy = NDIM == 2 && f >= C::F0;
+      const int fid = isy ? f - C::F0 : f;
+      const int fy = isy ? fid / BX : fid / (BX + 1);
+      const int fx = fid - fy * (isy ? BX : BX + 1);
+      if (i0 + fx > g.n[0] - (isy ? 1 : 0) || (NDIM == 2 && j0 + fy > g.n[1] - (isy ? 0 : 1))) continue;
+      const int s0 = (fy + C::HY) * C::SX + (fx + C::HX);
+      const int er = isy ? C::E0 + (fy + 1) * BX + fx : fy * (BX + 2) + fx + 1;
+      if constexpr (NDIM == 1) {
+        const int fld[3] = {0, 1, 2};
+        face_df<C, CMAX, 0>(su, ss, sf, p, s0 - 1, s0, er - 1, er, f, fld);
+      } else {
+        const int fld[4] = {0, isy ? 2 : 1, isy ? 1 : 2, 3};
+        face_df<C, CMAX, 0>(su, ss, sf, p, s0 - (isy ? C::SX : 1), s0, er - (isy ? BX : 1), er, f, fld);
+      }
+    }
+    __syncthreads();
 #pragma unroll
-  for (int c = 0; c < C::CPT; ++c)
+    for (int c = 0; c < C::CPT; ++c) {
+      const int cell = threadIdx.x + c * NT;
+      if (cell >= C::NCELL) break;
+      df d[NV];
+      face_diff_df<C, BX, BY, BZ, 0>(sf, cell % BX, cell / BX, 0, d);
 #pragma unroll
-    for (int v = 0; v < NV; ++v) dU[c][v] = {0.0f, 0.0f};
-  face_pass_df<NDIM, BX, BY, BZ, NT, 0>(su, sf, ss, p, g, i0, j0, k0, dU);
-  if constexpr (NDIM >= 2) face_pass_df<NDIM, BX, BY, BZ, NT, 1>(su, sf, ss, p, g, i0, j0, k0, dU);
-  if constexpr (NDIM >= 3) face_pass_df<NDIM, BX, BY, BZ, NT, 2>(su, sf, ss, p, g, i0, j0, k0, dU);
+      for (int v = 0; v < NV; ++v) dU[c][v] = d[v] * p.nhalf_inv_dx[0];
+      if constexpr (NDIM == 2) {
+        face_diff_df<C, BX, BY, BZ, 1>(sf + C::F0, cell % BX, cell / BX, 0, d);
+#pragma unroll
+        for (int v = 0; v < NV; ++v) dU[c][v] = df_fma(d[v], p.nhalf_inv_dx[1], dU[c][v]);
+      }
+    }
+  } else {
+    axis_pass_df<NDIM, BX, BY, BZ, NT, 0, CMAX>(su, sf, ss, p, g, i0, j0, k0, dU);
+    axis_pass_df<NDIM, BX, BY, BZ, NT, 1, CMAX>(su, sf, ss, p, g, i0, j0, k0, dU);
+    axis_pass_df<NDIM, BX, BY, BZ, NT, 2, CMAX>(su, sf, ss, p, g, i0, j0, k0, dU);
+  }
 
   df rmax = {0.0f, 0.0f};
   bool ok_all = true;
@@ -264,14 +342,14 @@ __global__ void __launch_bounds__(NT) stage_df_kernel(const DFArgs a) {
       q[v] = su[v * C::SCELLS + s0];
       L[v] = dU[c][v];
     }
-    rsst_rhs_df<NV>(q, L, p);
-    if (a.stage == 1) {
+    rsst_rhs_df<NV, CMAX>(q, L, p);
+    if constexpr (ST == 1) {
 #pragma unroll
-      for (int v = 0; v < NV; ++v) u[v] = q[v] + dt * L[v];
+      for (int v = 0; v < NV; ++v) u[v] = df_fma(dt, L[v], q[v]);
     } else {
       const int64_t o = pidx(g, i, j, k);
 #pragma unroll
-      for (int v = 0; v < NV; ++v) u[v] = scale(ld_df(a.base, v * g.fstride + o) + (q[v] + dt * L[v]), 0.5f);
+      for (int v = 0; v < NV; ++v) u[v] = scale(ld_df(a.base, v * g.fstride + o) + df_fma(dt, L[v], q[v]), 0.5f);
       bool ok;
       const df r = cfl_rate_df<NV>(u, p, ok);
       if (ok && df_lt(rmax, r)) rmax = r;
@@ -279,7 +357,7 @@ __global__ void __launch_bounds__(NT) stage_df_kernel(const DFArgs a) {
     }
     store_ghosts_df<NV>(a.out, g, a.p, a.bg, a.bg_len, i, j, k, u);
   }
-  if (a.stage == 2) {
+  if constexpr (ST == 2) {
     if (!ok_all) atomicOr(a.flag, RSST_FLAG_NONPHYSICAL);
     block_max_df<NT>(rmax, a.scal + (a.slot ^ 1), sred);
   }
@@ -418,14 +496,16 @@ static PhysDF make_physdf(const Phys& p) {
   PhysDF q;
   q.gamma = split_host(p.gamma);
   q.gm1 = split_host(p.gm1);
-  q.hgm1 = split_host(p.hgm1);
+  q.nhgm1 = split_host(-p.hgm1);
   q.inv_gm1 = split_host(p.inv_gm1);
-  q.inv_xi = split_host(p.inv_xi);
-  q.f = split_host(p.f);
+  q.gam_gm1 = split_host(p.gam_gm1);
+  q.gx = split_host(p.gamma_xi2);
+  q.nf = split_host(-p.f);
+  q.nf_gm1 = split_host(-p.f_gm1);
   q.inv_cmax4 = split_host(p.inv_cmax4);
   for (int d = 0; d < 3; ++d) {
     q.grav[d] = split_host(p.grav[d]);
-    q.inv_dx[d] = split_host(p.inv_dx[d]);
+    q.nhalf_inv_dx[d] = split_host(-p.half_inv_dx[d]);
   }
   q.sum_inv_dx = split_host(p.sum_inv_dx);
   q.variant = p.variant;
@@ -434,18 +514,19 @@ static PhysDF make_physdf(const Phys& p) {
   return q;
 }
 
-template <int NDIM, int BX, int BY, int BZ, int NT>
-static int launch_df(const DFArgs& a, cudaStream_t s) {
+template <int NDIM, int BX, int BY, int BZ, int NT, int MINB, bool CMAX, int ST>
+static int launch_df_kernel(const CUtensorMap* tin, const DFArgs& a, cudaStream_t s) {
   using C = TileCfgDF<NDIM, BX, BY, BZ, NT>;
-  auto kern = stage_df_kernel<NDIM, BX, BY, BZ, NT>;
-  const size_t smem = C::SMEM + 64;
+  auto kern = stage_df_kernel<NDIM, BX, BY, BZ, NT, MINB, CMAX, ST>;
+  const size_t smem = C::SMEM;
+  static const CUtensorMap none = {};
   static std::atomic<unsigned long long> attr{0};
   if (set_smem_limit_once(kern, smem, attr) != cudaSuccess) {
     rsst_set_error("cudaFuncSetAttribute failed for the double-float stage kernel");
     return RSST_ECUDA;
   }
   dim3 grid((a.g.n[0] + BX - 1) / BX, NDIM >= 2 ? (a.g.n[1] + BY - 1) / BY : 1, NDIM >= 3 ? (a.g.n[2] + BZ - 1) / BZ : 1);
-  kern<<<grid, NT, smem, s>>>(a);
+  kern<<<grid, NT, smem, s>>>(NDIM >= 2 ? *tin : none, a);
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) {
     rsst_set_error("double-float stage kernel launch: %s", cudaGetErrorString(e));
@@ -454,11 +535,44 @@ static int launch_df(const DFArgs& a, cudaStream_t s) {
   return RSST_OK;
 }
 
+// The C_max law and the stage are compile-time (no branches on them in the flux).
+template <int NDIM, int BX, int BY, int BZ, int NT, int MINB>
+static int launch_df(const CUtensorMap* tin, const DFArgs& a, cudaStream_t s) {
+  if (a.q.use_cmax)
+    return a.stage == 1 ? launch_df_kernel<NDIM, BX, BY, BZ, NT, MINB, true, 1>(tin, a, s)
+                        : launch_df_kernel<NDIM, BX, BY, BZ, NT, MINB, true, 2>(tin, a, s);
+  return a.stage == 1 ? launch_df_kernel<NDIM, BX, BY, BZ, NT, MINB, false, 1>(tin, a, s)
+                      : launch_df_kernel<NDIM, BX, BY, BZ, NT, MINB, false, 2>(tin, a, s);
+}
+
 }  // namespace rsst
 
 using namespace rsst;
 
-int rsst_launch_stage_df(const StageArgs<float2>& sa, cudaStream_t s) {
+// 2D tiles: the one that finishes first by a linear model, as for float64
+// (rsst_stage_fp64_tile): 16 x 16, or 8 x 8 where a grid is too small to fill
+// the SMs.  Measured per stage (us, 16 x 16 / 8 x 8): 64^2 9.5 / 6.7, 128^2
+// 9.6 / 7.5, 256^2 12.6 / 17.4, 512^2 33.7 / 47.8.
+static const int TILE2_DF[2] = {16, 8};
+
+int rsst_stage_df_tile(const Geom& g, int sms) {
+  static const double offset[2] = {5.0, 5.2}, slope[2] = {4.1, 1.6};
+  if (g.ndim != 2) return 0;
+  double us[2];
+  for (int t = 0; t < 2; ++t) {
+    const int b = TILE2_DF[t];
+    const int64_t tiles = (int64_t)((g.n[0] + b - 1) / b) * ((g.n[1] + b - 1) / b);
+    us[t] = offset[t] + slope[t] * (double)((tiles + sms - 1) / sms);
+  }
+  return us[1] < us[0] ? 1 : 0;
+}
+
+void rsst_stage_df_box(const Geom& g, int tile, int* sx, int* sy, int* sz) {
+  *sx = *sy = (g.ndim == 3 ? 8 : TILE2_DF[tile]) + 2 * RSST_G;
+  *sz = g.ndim == 3 ? 4 + 2 * RSST_G : 1;
+}
+
+int rsst_launch_stage_df(const CUtensorMap* tin, const StageArgs<float2>& sa, cudaStream_t s) {
   DFArgs a;
   a.in = sa.in;
   a.base = sa.base;
@@ -475,10 +589,12 @@ int rsst_launch_stage_df(const StageArgs<float2>& sa, cudaStream_t s) {
   a.dt_fixed = sa.dt_fixed;
   switch (a.g.ndim) {
     case 1:
-      if (a.g.n[0] <= RSST_SMALL_1D) return launch_df<1, 16, 1, 1, 32>(a, s);
-      return launch_df<1, 256, 1, 1, 256>(a, s);
-    case 2: return launch_df<2, 32, 8, 1, 288>(a, s);  // 9 warps: each face pass in one round
-    case 3: return launch_df<3, 8, 8, 4, 320>(a, s);  // 10 warps: each face pass in one round
+      if (a.g.n[0] <= RSST_SMALL_1D) return launch_df<1, 16, 1, 1, 32, 1>(nullptr, a, s);
+      return launch_df<1, 256, 1, 1, 256, 1>(nullptr, a, s);
+    case 2:
+      return sa.tile ? launch_df<2, 8, 8, 1, 160, 6>(tin, a, s) : launch_df<2, 16, 16, 1, 288, 4>(tin, a, s);
+    case 3:
+      return launch_df<3, 8, 8, 4, 320, 3>(tin, a, s);  // 10 warps: each face pass in one round
   }
   rsst_set_error("ndim must be 1, 2 or 3");
   return RSST_EINVAL;

@@ -127,7 +127,7 @@ struct StageArgs {
   const float* tabr; // row-major background table [tab_len][TR_W] (TMA float32 kernels), or null
   double* dU_out;   // float64 kernels: if set, the Euler tendency of each interior cell
                     // (padded layout) is written here too (adjoint recompute)
-  int tile;         // float64 2D: tile shape index (rsst_stage_fp64_tile)
+  int tile;         // float64 / double-float 2D: tile shape index (rsst_stage_fp64_tile, rsst_stage_df_tile)
   int64_t stall_ns; // > 0 (failure-detection tests only): each tile of a TMA-staged kernel
                     // also waits this long on a barrier that nothing completes
 };
@@ -148,7 +148,10 @@ int rsst_launch_sums_fp64(const double* U, const Geom& g, double* partial, doubl
                           double scale, cudaStream_t s);
 
 int rsst_launch_stage_fp32(const StageArgs<float>& a, cudaStream_t s);
-int rsst_launch_stage_df(const StageArgs<float2>& a, cudaStream_t s);
+// Double-float stage kernel: tensor map, box and tile as for float64.
+int rsst_launch_stage_df(const CUtensorMap* tin, const StageArgs<float2>& a, cudaStream_t s);
+void rsst_stage_df_box(const Geom& g, int tile, int* sx, int* sy, int* sz);
+int rsst_stage_df_tile(const Geom& g, int sms);
 int rsst_launch_pack_df(const double* src, float2* dst, const Geom& g, const Phys& p, const double* bg, int bg_len,
                         cudaStream_t s);
 int rsst_launch_unpack_df(const float2* src, double* dst, const Geom& g, cudaStream_t s);
@@ -191,7 +194,7 @@ struct rsst_handle {
   int use_tma2d;        // 2D float32 runs use the TMA-staged kernel
   int use_tma3d;        // 3D float32 runs use the TMA z-march kernel
   int use_tma_fp64;     // 2D/3D float64 runs stage their halo tiles by TMA
-  int fp64_tile;        // their tile shape index
+  int tile;             // 2D float64 / double-float: tile shape index
   CUtensorMap tmap[2];  // tensor maps of buf[0], buf[1] (TMA kernels)
   void* adj;            // adjoint checkpoints and work arrays, or null
   int slot;
