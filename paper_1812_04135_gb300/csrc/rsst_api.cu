@@ -365,6 +365,7 @@ extern "C" int rsst_init(rsst_handle** out, const rsst_config* cfg, void* stream
       if (rc != RSST_OK) goto fail;
     }
   }
+  if (cfg->precision == RSST_FP64) h->use_line = rsst_line_fp64_ok(h->g, h->p);
   if (cfg->precision != RSST_FP32_PERT && cfg->ndim >= 2) {
     const bool dfp = cfg->precision == RSST_FP64_DF;
     int dev = 0, sms = 0;
@@ -471,7 +472,7 @@ extern "C" int rsst_get_state(rsst_handle* h, double* U, int on_host) {
 }
 
 template <typename T>
-static int plain_steps(rsst_handle* h, double dt, int nsteps, cudaStream_t st) {
+static StageArgs<T> stage_args(const rsst_handle* h, double dt) {
   StageArgs<T> a;
   memset(&a, 0, sizeof a);
   a.g = h->g;
@@ -487,6 +488,12 @@ static int plain_steps(rsst_handle* h, double dt, int nsteps, cudaStream_t st) {
   a.dt_fixed = dt > 0.0 ? dt : 0.0;
   a.stall_ns = h->stall_ns;
   a.tile = h->tile;
+  return a;
+}
+
+template <typename T>
+static int plain_steps(rsst_handle* h, double dt, int nsteps, cudaStream_t st) {
+  StageArgs<T> a = stage_args<T>(h, dt);
   T* U = (T*)h->buf[0];
   T* Us = (T*)h->buf[1];
   for (int s = 0; s < nsteps; ++s) {
@@ -580,7 +587,22 @@ static int run_steps(rsst_handle* h, double dt, int nsteps) {
   return plain_steps<T>(h, dt, nsteps, h->stream);
 }
 
+// Steps of a short line on the cluster kernel (the adjoint's recompute, which
+// also records each stage's Euler tendency, takes the stage kernels).
+static int line_steps(rsst_handle* h, double dt, int nsteps) {
+  StageArgs<double> a = stage_args<double>(h, dt);
+  a.slot = h->slot;
+  a.in = (const double*)h->buf[0];
+  a.out = (double*)h->buf[0];
+  int launches = 0;
+  const int rc = rsst_launch_line_fp64(a, nsteps, &launches, h->stream);
+  h->launches += launches;
+  if (rc == RSST_OK) h->slot ^= nsteps & 1;
+  return rc;
+}
+
 int rsst_handle_steps(rsst_handle* h, double dt, int nsteps) {
+  if (h->use_line && !h->rec_dU[0] && !h->rec_dU[1]) return line_steps(h, dt, nsteps);
   if (h->cfg.precision == RSST_FP32_PERT) return run_steps<float>(h, dt, nsteps);
   if (h->cfg.precision == RSST_FP64_DF) return run_steps<float2>(h, dt, nsteps);
   return run_steps<double>(h, dt, nsteps);

@@ -41,6 +41,50 @@ __device__ __forceinline__ void block_max_to(double x, double* dst, double* sred
   }
 }
 
+// Store a float64 cell and the edge ghost cells that mirror or wrap it (across a
+// wall along the vertical axis with the background difference added).
+template <int NV>
+__device__ __forceinline__ void store_with_ghosts(double* __restrict__ out, const Geom& g,
+                                                  const Phys& p, const double* __restrict__ bg,
+                                                  int bg_len, int i, int j, int k,
+                                                  const double (&u)[NV]) {
+  constexpr int ND = NV - 2;
+  const int64_t fs = g.fstride;
+  const int64_t o = pidx(g, i, j, k);
+#pragma unroll
+  for (int v = 0; v < NV; ++v) out[v * fs + o] = u[v];
+  const int c[3] = {i, j, k};
+#pragma unroll
+  for (int d = 0; d < ND; ++d) {
+    const int n = g.n[d], cd = c[d];
+#pragma unroll
+    for (int side = 0; side < 2; ++side) {
+      const bool hit = side == 0 ? (cd < RSST_G) : (cd >= n - RSST_G);
+      if (!hit) continue;
+      int gp;
+      double w[NV];
+#pragma unroll
+      for (int v = 0; v < NV; ++v) w[v] = u[v];
+      if (p.bc[d] == RSST_BC_PERIODIC) {
+        gp = side == 0 ? cd + n : cd - n;
+      } else {
+        gp = side == 0 ? -1 - cd : 2 * n - 1 - cd;
+        w[1 + d] = -w[1 + d];
+        if (bg != nullptr && d == p.vertical) {
+          const double* rho0 = bg;
+          const double* e0 = bg + bg_len;
+          w[0] += rho0[gp + RSST_G] - rho0[cd + RSST_G];
+          w[NV - 1] += e0[gp + RSST_G] - e0[cd + RSST_G];
+        }
+      }
+      const int ii = d == 0 ? gp : i, jj = d == 1 ? gp : j, kk = d == 2 ? gp : k;
+      const int64_t og = pidx(g, ii, jj, kk);
+#pragma unroll
+      for (int v = 0; v < NV; ++v) out[v * fs + og] = w[v];
+    }
+  }
+}
+
 // Store a perturbation-state cell and the edge ghost cells that wrap it or
 // mirror it (normal momentum negated).  The perturbation about a background
 // is mirrored without a background term: U1(ghost) = mirror(U1(image)).

@@ -139,6 +139,9 @@ int rsst_launch_stage_fp64(const CUtensorMap* tin, const StageArgs<double>& a, c
 void rsst_stage_fp64_box(const Geom& g, int tile, int* sx, int* sy, int* sz);
 // Index of the 2D tile shape for a grid on a device with `sms` SMs.
 int rsst_stage_fp64_tile(const Geom& g, int sms);
+// Short 1D float64 lines: many steps in one launch on a thread-block cluster.
+int rsst_line_fp64_ok(const Geom& g, const Phys& p);
+int rsst_launch_line_fp64(const StageArgs<double>& a, int nsteps, int* launches, cudaStream_t s);
 int rsst_launch_pack_fp64(const double* src, double* dst, const Geom& g, const Phys& p,
                           const double* bg, int bg_len, cudaStream_t s);
 int rsst_launch_unpack_fp64(const double* src, double* dst, const Geom& g, cudaStream_t s);
@@ -195,6 +198,7 @@ struct rsst_handle {
   int use_tma3d;        // 3D float32 runs use the TMA z-march kernel
   int use_tma_fp64;     // 2D/3D float64 runs stage their halo tiles by TMA
   int tile;             // 2D float64 / double-float: tile shape index
+  int use_line;         // short 1D float64 lines: the cluster kernel
   CUtensorMap tmap[2];  // tensor maps of buf[0], buf[1] (TMA kernels)
   void* adj;            // adjoint checkpoints and work arrays, or null
   int slot;

@@ -384,61 +384,88 @@ __device__ __forceinline__ double mc_slope(double a, double b) {
 // with dP = (gamma-1)(V^2/2 drho - V.dm + dE) (Eq. pvs_dt_dpr, ideal gas),
 // evaluated at the cell centre of the stage state; force terms
 // (0, rho F, m.F) of App. B are added after (dP excludes them).
+//
+// In two parts: what depends on the state alone, and what needs the Euler
+// tendency (the 1D line kernel forms the first while the fluxes are computed).
+// s is scaled by a; b turns it into the E row's factor: 1/(rho a^2) (PVS, PMS),
+// 1/rho (DVS, DMS) or (de/dP)_rho (PD).
+template <int NV>
+struct RhsPrep {
+  double v[NV - 2], hv2, H, a, b;  // hv2: |V|^2/2 - (de/drho)_P; H = e + P +- rho V^2/2
+};
 template <int NV, bool CV = false>
-__device__ __forceinline__ void rsst_rhs(const double (&q)[NV], double (&dU)[NV], const Phys& p) {
+__device__ __forceinline__ void rhs_prep(const double (&q)[NV], const Phys& p, RhsPrep<NV>& r) {
   constexpr int ND = NV - 2;
   const double rho = q[0];
-  if (p.variant != RSST_EULER) {
-    const double ir = rcp_nr(rho);
-    double v[ND];
-    double k = 0.0;  // rho |V|^2
+  const double ir = rcp_nr(rho);
+  double k = 0.0;  // rho |V|^2
 #pragma unroll
-    for (int e = 0; e < ND; ++e) {
-      v[e] = q[1 + e] * ir;
-      k = e == 0 ? q[1] * v[0] : fma(q[1 + e], v[e], k);
-    }
-    const double P = Eos<CV>::pressure(p, rho, q[NV - 1], k);
-    const double kin = 0.5 * k;
-    const int var = p.variant;
-    const double f = p.use_cmax ? f_of(Eos<CV>::sound2(p, rho, P, ir), p) : p.f;
-    const bool mom = var == RSST_PVS || var == RSST_DVS;  // the correction moves momentum
-    // e + P + rho V^2/2, or minus
-    const double H = Eos<CV>::enthalpy(p, rho, P) + (mom ? kin : -kin);
+  for (int e = 0; e < ND; ++e) {
+    r.v[e] = q[1 + e] * ir;
+    k = e == 0 ? q[1] * r.v[0] : fma(q[1 + e], r.v[e], k);
+  }
+  const double P = Eos<CV>::pressure(p, rho, q[NV - 1], k);
+  const double kin = 0.5 * k;
+  const int var = p.variant;
+  const double f = p.use_cmax ? f_of(Eos<CV>::sound2(p, rho, P, ir), p) : p.f;
+  r.H = Eos<CV>::enthalpy(p, rho, P) + (var == RSST_PVS || var == RSST_DVS ? kin : -kin);
+  if (var == RSST_PVS || var == RSST_PMS || var == RSST_PD) {
+    r.hv2 = Eos<CV>::half_v2_minus_de_drho(p, kin * ir, P);
+    r.a = Eos<CV>::f_over_de_dP(p, f, rho, P);
+    r.b = var == RSST_PD ? Eos<CV>::de_dP(p, rho, P) : Eos<CV>::inv_rho_a2(p, rho, P);
+  } else {
+    r.hv2 = 0.0;
+    r.a = f;
+    r.b = ir;
+  }
+}
+template <int NV>
+__device__ __forceinline__ void rhs_apply(const double (&q)[NV], double (&dU)[NV], const Phys& p,
+                                          const RhsPrep<NV>& r) {
+  constexpr int ND = NV - 2;
+  const int var = p.variant;
+  if (var != RSST_EULER) {
     double w, wE;  // f s r0 and f s rE / H
     if (var == RSST_PVS || var == RSST_PMS || var == RSST_PD) {
-      double s = fma(Eos<CV>::half_v2_minus_de_drho(p, kin * ir, P), dU[0], dU[NV - 1]);
+      double s = fma(r.hv2, dU[0], dU[NV - 1]);
 #pragma unroll
-      for (int e = 0; e < ND; ++e) s = fma(-v[e], dU[1 + e], s);
-      const double fs = Eos<CV>::f_over_de_dP(p, f, rho, P) * s;
+      for (int e = 0; e < ND; ++e) s = fma(-r.v[e], dU[1 + e], s);
+      const double fs = r.a * s;
+      wE = fs * r.b;
       if (var == RSST_PD) {
-        dU[NV - 1] = fma(-fs, Eos<CV>::de_dP(p, rho, P), dU[NV - 1]);
-        w = wE = 0.0;
+        dU[NV - 1] = fma(-fs, r.b, dU[NV - 1]);
+        w = 0.0;
       } else {
-        wE = fs * Eos<CV>::inv_rho_a2(p, rho, P);
-        w = wE * rho;
+        w = wE * q[0];
       }
     } else {  // DVS, DMS
-      w = f * dU[0];
-      wE = w * ir;
+      w = r.a * dU[0];
+      wE = w * r.b;
     }
     if (var != RSST_PD) {
       dU[0] -= w;
-      if (mom) {
+      if (var == RSST_PVS || var == RSST_DVS) {
 #pragma unroll
-        for (int e = 0; e < ND; ++e) dU[1 + e] = fma(-w, v[e], dU[1 + e]);
+        for (int e = 0; e < ND; ++e) dU[1 + e] = fma(-w, r.v[e], dU[1 + e]);
       }
-      dU[NV - 1] = fma(-wE, H, dU[NV - 1]);
+      dU[NV - 1] = fma(-wE, r.H, dU[NV - 1]);
     }
   }
   if (p.has_grav) {
     double mg = 0.0;
 #pragma unroll
     for (int e = 0; e < ND; ++e) {
-      dU[1 + e] += rho * p.grav[e];
+      dU[1 + e] += q[0] * p.grav[e];
       mg += q[1 + e] * p.grav[e];
     }
     dU[NV - 1] += mg;
   }
+}
+template <int NV, bool CV = false>
+__device__ __forceinline__ void rsst_rhs(const double (&q)[NV], double (&dU)[NV], const Phys& p) {
+  RhsPrep<NV> r = {};
+  if (p.variant != RSST_EULER) rhs_prep<NV, CV>(q, p, r);
+  rhs_apply<NV>(q, dU, p, r);
 }
 
 // Half of a double (as 0.5 * x rounds it), on the integer pipe.
