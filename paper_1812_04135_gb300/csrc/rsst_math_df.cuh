@@ -200,10 +200,10 @@ __device__ __forceinline__ void rsst_rhs_df(const df (&q)[NV], df (&dU)[NV], con
     const bool mom = var == RSST_PVS || var == RSST_DVS;  // the correction moves momentum
     const df H = df_fma(p.gam_gm1, P, mom ? kin : -kin);  // e + P +- rho V^2/2
     if (var == RSST_PVS || var == RSST_PMS || var == RSST_PD) {
-      df s = df_fma(kin * ir, dU[0], dU[NV - 1]);
+      df s = (kin * ir) * dU[0];  // the small terms first: one rounding at dE's size
 #pragma unroll
       for (int e = 0; e < ND; ++e) s = df_fma(-v[e], dU[1 + e], s);
-      const df nfs = nf_gm1 * s;  // -f dP
+      const df nfs = nf_gm1 * (s + dU[NV - 1]);  // -f dP
       if (var == RSST_PD) {
         dU[NV - 1] = df_fma(nfs, p.inv_gm1, dU[NV - 1]);
       } else {

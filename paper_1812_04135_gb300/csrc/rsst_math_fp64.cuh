@@ -427,10 +427,10 @@ __device__ __forceinline__ void rhs_apply(const double (&q)[NV], double (&dU)[NV
   if (var != RSST_EULER) {
     double w, wE;  // f s r0 and f s rE / H
     if (var == RSST_PVS || var == RSST_PMS || var == RSST_PD) {
-      double s = fma(r.hv2, dU[0], dU[NV - 1]);
+      double s = r.hv2 * dU[0];  // the small terms first: one rounding at dE's size
 #pragma unroll
       for (int e = 0; e < ND; ++e) s = fma(-r.v[e], dU[1 + e], s);
-      const double fs = r.a * s;
+      const double fs = r.a * (s + dU[NV - 1]);
       wE = fs * r.b;
       if (var == RSST_PD) {
         dU[NV - 1] = fma(-fs, r.b, dU[NV - 1]);
