@@ -11,21 +11,25 @@
 //   adj_cell: per interior cell, with the Euler tendency dU that the forward
 //     kernel wrote while the segment was recomputed, nu = mu^T dC/d(dU) and
 //     the pointwise part mu^T d(C + force)/dq (C = reduced tendency, Sec. 3.2 /
-//     App. A; force of App. B) plus the identity part b lambda_out, and the
-//     xi partial;
-//   adj_face: per face, phi = (nu_right - nu_left)/dx, then phi^T dF/dU_k for
-//     the four stencil cells k of the face (MC slopes, face states, LLF flux
-//     of Sec. 4.2) and the xi partial;
-//   adj_gather: each padded cell (interior and edge ghosts) sums the
-//     contributions of the faces whose stencil holds it;
-//   adj_fold: ghost-cell adjoints go back to the cells they were copied from
-//     (wrap, or mirror with the normal momentum negated).
+//     App. A; force of App. B) plus the identity part b lambda_out (and, in
+//     stage 1, lambda^{n+1}/2), and the xi partial;
+//   adj_face: per face of any axis, phi = (nu_right - nu_left)/dx, then
+//     phi^T dF/dU_k for the four stencil cells k of the face (MC slopes, face
+//     states, LLF flux of Sec. 4.2) and the xi partial;
+//   adj_gather: each interior cell sums the contributions of the faces whose
+//     stencil holds it or a ghost cell it is the image of (wrap, or mirror
+//     with the normal momentum negated).
 // The derivatives are hand-derived reverse mode: each VJP recomputes its
 // forward values (holding the branches the forward pass took) and then runs
-// the chain rule backwards once, so a face costs about three flux
-// evaluations whatever the size of its stencil.  Divisions go through the
-// forward kernels' Newton-Raphson reciprocal and the square roots of c_tot
-// through their c_tot square root (float64 pipe economy; same readings).
+// the chain rule backwards once.
+//
+// What bounds it: the float64 pipe, in the face kernel above all.  A 2D face
+// takes 173 float64 instructions (295 when both sides carried the wave speed's
+// derivatives, speeds and their reciprocals came from float64 square roots,
+// limiter and flux halves were multiplications and each block summed its xi
+// partials by a float64 tree).  A stage's VJP on 256^2 (ncu, us): cells 21,
+// faces 50 (80 % of the float64 pipe; one launch for both axes, 94 in two),
+// gather 15; ghost fold, xi sum and axpby (together 18) are gone into these.
 #include <cstring>
 #include <vector>
 
@@ -36,167 +40,178 @@
 
 namespace rsst {
 
-// |V| with a zero subgradient at V = 0.
-__device__ __forceinline__ double speed_of(double v2) { return v2 > 0.0 ? sqrt_ctot(v2) : 0.0; }
-
-// MC branch (Sec. 4.2): 0 -> 0, 1 -> 2a, 2 -> 2b, 3 -> (a+b)/2; the
-// decisions of the oracle's comparisons (2|a| <= 2|b| and 2|a| <= |a+b|/2,
-// then 2|b| <= |a+b|/2), taken on the integer pipe as in mc_slope.
-__device__ __forceinline__ int mc_branch(double a, double b) {
+// Half the MC slope (Sec. 4.2) and the branch taken: 0 -> 0, 1 -> a, 2 -> b,
+// 3 -> (a+b)/4; decisions and values on the integer pipe as in mc_slope.
+__device__ __forceinline__ double half_mc(double a, double b, int& br) {
+  const long long two = 2ll << 52;             // x4 in the exponent field
   const unsigned long long four = 1ull << 54;  // x4 in the shifted exponent field
   const long long ia = __double_as_longlong(a), ib = __double_as_longlong(b);
   const unsigned long long ua = (unsigned long long)ia << 1, ub = (unsigned long long)ib << 1;
-  if (!(((ia ^ ib) >= 0) && ua != 0 && ub != 0)) return 0;
-  const unsigned long long us = (unsigned long long)__double_as_longlong(a + b) << 1;
-  if (ua <= ub && ua + four <= us) return 1;
-  return ub + four <= us ? 2 : 3;
+  const long long is = __double_as_longlong(a + b);
+  const unsigned long long us = (unsigned long long)is << 1;
+  const bool same = ((ia ^ ib) >= 0) && ua != 0 && ub != 0;
+  const bool pa = ua <= ub && ua + four <= us, pb = ub + four <= us;
+  br = !same ? 0 : (pa ? 1 : (pb ? 2 : 3));
+  return same ? __longlong_as_double(pa ? ia : (pb ? ib : is - two)) : 0.0;
 }
-__device__ __forceinline__ double mc_value(int br, double a, double b) {
-  return br == 0 ? 0.0 : (br == 1 ? 2.0 * a : (br == 2 ? 2.0 * b : 0.5 * (a + b)));
-}
-// d(slope)/da and d(slope)/db of the taken branch, times the slope's adjoint ds.
+// d(half slope)/da and /db of the taken branch, times the half slope's adjoint ds.
 __device__ __forceinline__ void mc_reverse(int br, double ds, double& da, double& db) {
-  da = br == 1 ? 2.0 * ds : (br == 3 ? 0.5 * ds : 0.0);
-  db = br == 2 ? 2.0 * ds : (br == 3 ? 0.5 * ds : 0.0);
+  const double q = half_of(half_of(ds));
+  da = br == 1 ? ds : (br == 3 ? q : 0.0);
+  db = br == 2 ? ds : (br == 3 ? q : 0.0);
 }
 
-// a/xi of a state (constant xi, or the C_max law, Eq. cx).
-__device__ __forceinline__ double sound_term(double a2, const Phys& p) {
-  if (p.use_cmax) return sqrt(a2 * rcp_nr(sqrt(1.0 + (a2 * a2) * p.inv_cmax4)));
-  return sqrt_ctot(a2) * p.inv_xi;
+// a/xi under the C_max law (Eq. cx).
+__device__ __forceinline__ double sound_cmax(double a2, const Phys& p) {
+  return sqrt(a2 * rcp_nr(sqrt(1.0 + (a2 * a2) * p.inv_cmax4)));
 }
 
-// The forward values of one face state that the reverse of its flux reuses:
-// 1/rho, V, |V|^2, P, a^2, |V| and (constant xi) a.
+// 1/x of a positive float pair as a double (relative error below 2^-43).
+__device__ __forceinline__ double rcp_of_pair(float h, float l) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(h));
+  return pair_to_double(r, r * fmaf(-l, r, fmaf(-h, r, 1.0f)));
+}
+
+// The forward values of one face state that the reverse of its flux reuses.
 template <int NV>
 struct StateFwd {
-  double ir, v[NV - 2], v2, P, a2, sv, sa;
+  double ir, v[NV - 2], hv2, P;  // 1/rho, V, |V|^2/2, P
+  double k;                      // rho |V|^2
 };
-
-// c_tot = |V| + a/xi of one face state (Sec. 4.2; the LLF speed), keeping the
-// values its flux's reverse needs.  (The flux itself enters the VJP only
-// through its derivatives.)
 template <int NV>
-__device__ __forceinline__ double state_fwd(const double (&q)[NV], const Phys& p, StateFwd<NV>& w) {
+__device__ __forceinline__ void state_fwd(const double (&q)[NV], const Phys& p, StateFwd<NV>& w) {
   constexpr int ND = NV - 2;
-  const double rho = q[0];
-  w.ir = rcp_nr(rho);
-  w.v2 = 0.0;
+  w.ir = rcp_nr(q[0]);
+#pragma unroll
   for (int e = 0; e < ND; ++e) {
     w.v[e] = q[1 + e] * w.ir;
-    w.v2 += w.v[e] * w.v[e];
+    w.k = e == 0 ? q[1] * w.v[0] : fma(q[1 + e], w.v[e], w.k);
   }
-  w.P = p.gm1 * (q[NV - 1] - 0.5 * (rho * w.v2));
-  w.a2 = p.gamma * w.P * w.ir;
-  w.sv = speed_of(w.v2);
-  if (p.use_cmax) {
-    w.sa = 0.0;
-    return w.sv + sound_term(w.a2, p);
-  }
-  w.sa = sqrt_ctot(w.a2);
-  return w.sv + w.sa * p.inv_xi;
+  w.P = p.gm1 * q[NV - 1] - p.hgm1 * w.k;
+  w.hv2 = half_of(w.k) * w.ir;
 }
 
-// Face states of the face between u0 | u1 from the stencil (um, u0 | u1, up):
-// MUSCL-MC reconstruction, with the branches taken.
+// Reverse of the Euler flux along the first momentum (F = (m_0, m V_0 + P e_0,
+// (E + P) V_0)) at q for the cotangent f: adds f^T dF/dq to dq, through
+// V_0 = m_0/rho and P = (gamma-1)(E - |m|^2/(2 rho)).
 template <int NV>
-__device__ __forceinline__ void face_states(const double (&s)[4][NV], double (&qL)[NV], double (&qR)[NV],
-                                            int (&bL)[NV], int (&bR)[NV]) {
-  for (int v = 0; v < NV; ++v) {
-    const double aL = s[1][v] - s[0][v], dL = s[2][v] - s[1][v];
-    const double aR = s[2][v] - s[1][v], dR = s[3][v] - s[2][v];
-    bL[v] = mc_branch(aL, dL);
-    bR[v] = mc_branch(aR, dR);
-    qL[v] = s[1][v] + 0.5 * mc_value(bL[v], aL, dL);
-    qR[v] = s[2][v] - 0.5 * mc_value(bR[v], aR, dR);
-  }
-}
-
-// Reverse of the Euler flux along D (F_D = (m_D, m V_D + P e_D, (E + P) V_D))
-// and of c_tot at q, with w = state_fwd's values at q: adds dF^T dF/dq +
-// dc dc/dq to dq and returns dF^T dF/d(1/xi) + dc dc/d(1/xi).  Hand-derived
-// chain rule through v = m/rho, P = (gamma-1)(E - rho|v|^2/2), a^2 = gamma P/rho.
-template <int NV, int D>
-__device__ __forceinline__ double flux_vjp(const double (&q)[NV], const Phys& p, const StateFwd<NV>& w,
-                                           const double (&dF)[NV], double dc, double (&dq)[NV]) {
+__device__ __forceinline__ void flux_vjp(const double (&q)[NV], const Phys& p, const StateFwd<NV>& w,
+                                         const double (&f)[NV], double (&dq)[NV]) {
   constexpr int ND = NV - 2;
-  const double rho = q[0], E = q[NV - 1];
-  const double ir = w.ir, v2 = w.v2, P = w.P, a2 = w.a2;
-  const double(&v)[ND] = w.v;
-  double dv[ND];
-  for (int e = 0; e < ND; ++e) dv[e] = 0.0;
-  double dP = dF[1 + D] + dF[NV - 1] * v[D], dv2 = 0.0, drho = 0.0, dE = dF[NV - 1] * v[D], dinv_xi = 0.0;
-  dq[1 + D] += dF[0];
-  for (int e = 0; e < ND; ++e) {
-    dq[1 + e] += dF[1 + e] * v[D];
-    dv[D] += dF[1 + e] * q[1 + e];
-  }
-  dv[D] += dF[NV - 1] * (E + P);
-  if (v2 > 0.0) dv2 += dc * 0.5 * rcp_nr(w.sv);
-  double da2 = 0.0;
-  if (p.use_cmax) {  // g = sqrt(u), u = a2 / t, t = sqrt(w), w = 1 + a2^2 / C^4
-    const double w = 1.0 + (a2 * a2) * p.inv_cmax4, t = sqrt(w), it = rcp_nr(t), u = a2 * it;
-    if (u > 0.0) {
-      const double du = dc * 0.5 * rcp_nr(sqrt(u));
-      const double dt = -du * u * it;
-      da2 += du * it + dt * it * a2 * p.inv_cmax4;
-    }
-  } else {
-    const double s = w.sa;
-    dinv_xi += dc * s;
-    if (a2 > 0.0) da2 += dc * p.inv_xi * 0.5 * rcp_nr(s);
-  }
-  dP += da2 * p.gamma * ir;
-  drho -= da2 * a2 * ir;
-  dE += dP * p.gm1;
-  drho -= dP * p.gm1 * 0.5 * v2;
-  dv2 -= dP * p.gm1 * 0.5 * rho;
-  for (int e = 0; e < ND; ++e) {
-    dv[e] += 2.0 * v[e] * dv2;
-    dq[1 + e] += dv[e] * ir;
-    drho -= dv[e] * v[e] * ir;
-  }
-  dq[0] += drho;
-  dq[NV - 1] += dE;
-  return dinv_xi;
+  const double v0 = w.v[0];
+  const double g = p.gm1 * fma(f[NV - 1], v0, f[1]);  // (gamma-1) dP
+  double dv = f[NV - 1] * (q[NV - 1] + w.P);
+#pragma unroll
+  for (int e = 0; e < ND; ++e) dv = fma(f[1 + e], q[1 + e], dv);
+  const double t = dv * w.ir;
+  dq[0] = fma(-t, v0, fma(g, w.hv2, dq[0]));
+  dq[1] += f[0] + t;
+#pragma unroll
+  for (int e = 0; e < ND; ++e) dq[1 + e] = fma(-g, w.v[e], fma(f[1 + e], v0, dq[1 + e]));
+  dq[NV - 1] = fma(f[NV - 1], v0, dq[NV - 1]) + g;
 }
 
-// Reverse of the face's LLF flux (Sec. 4.2, steps 2-4, through its MUSCL-MC
-// states): G[k] = phi^T dF/d(stencil cell k), and the return
-// value phi^T dF/d(1/xi).  The forward branches (MC branch, LLF side) are
-// recomputed and held.
-template <int NV, int D>
-__device__ __forceinline__ double face_vjp(const double (&s)[4][NV], const double (&phi)[NV], const Phys& p,
+// Reverse of twice the face's LLF flux (Sec. 4.2, steps 2-4, through its
+// MUSCL-MC states) for half the cotangent, f = phi/2; fields ordered with the
+// face's normal momentum first.  G[k] = phi^T dF/d(stencil cell k), and the
+// return value phi^T dF/d(1/xi).  The forward branches (MC branch, LLF side)
+// are recomputed and held; the LLF speed's derivatives are taken on the side
+// it came from only.
+template <int NV>
+__device__ __forceinline__ double face_vjp(const double (&s)[4][NV], const double (&f)[NV], const Phys& p,
                                            double (&G)[4][NV]) {
+  constexpr int ND = NV - 2;
   double qL[NV], qR[NV];
   int bL[NV], bR[NV];
-  face_states<NV>(s, qL, qR, bL, bR);
-  StateFwd<NV> wL, wR;
-  const double cL = state_fwd<NV>(qL, p, wL);
-  const double cR = state_fwd<NV>(qR, p, wR);
-  const bool left = cL >= cR;
-  const double alpha = left ? cL : cR;
-  double dF[NV], dqL[NV], dqR[NV], dalpha = 0.0;
+#pragma unroll
   for (int v = 0; v < NV; ++v) {
-    dF[v] = 0.5 * phi[v];
-    dqL[v] = 0.5 * alpha * phi[v];
-    dqR[v] = -0.5 * alpha * phi[v];
-    dalpha -= 0.5 * phi[v] * (qR[v] - qL[v]);
+    const double d0 = s[1][v] - s[0][v], d1 = s[2][v] - s[1][v], d2 = s[3][v] - s[2][v];
+    qL[v] = s[1][v] + half_mc(d0, d1, bL[v]);
+    qR[v] = s[2][v] - half_mc(d1, d2, bR[v]);
   }
-  double dinv_xi = flux_vjp<NV, D>(qL, p, wL, dF, left ? dalpha : 0.0, dqL);
-  dinv_xi += flux_vjp<NV, D>(qR, p, wR, dF, left ? 0.0 : dalpha, dqR);
+  StateFwd<NV> wL, wR;
+  state_fwd<NV>(qL, p, wL);
+  state_fwd<NV>(qR, p, wR);
+  double dalpha = 0.0;
+#pragma unroll
+  for (int v = 0; v < NV; ++v) dalpha = fma(f[v], qL[v] - qR[v], dalpha);
+  // LLF speed and, on its side: |V|, d(c)/d(m_e) = v_e iv / rho, and with
+  // ca = a/xi the products cP = dc dca/dP and cr = -dc dca/drho
+  bool left;
+  double alpha, sv, iv, cP, cr, dinv_xi = 0.0;
+  if (p.use_cmax) {
+    const double a2L = p.gamma * wL.P * wL.ir, a2R = p.gamma * wR.P * wR.ir;
+    const double vL = wL.k * wL.ir, vR = wR.k * wR.ir;
+    const double sL = vL > 0.0 ? sqrt_ctot(vL) : 0.0, sR = vR > 0.0 ? sqrt_ctot(vR) : 0.0;
+    const double cL = sL + sound_cmax(a2L, p), cR = sR + sound_cmax(a2R, p);
+    left = cL >= cR;
+    alpha = left ? cL : cR;
+    sv = left ? sL : sR;
+    iv = sv > 0.0 ? rcp_nr(sv) : 0.0;
+    // ca = sqrt(u), u = a2 / t, t = sqrt(w), w = 1 + a2^2 / C^4
+    const double a2 = left ? a2L : a2R, ir = left ? wL.ir : wR.ir;
+    const double t = sqrt(1.0 + (a2 * a2) * p.inv_cmax4), it = rcp_nr(t), u = a2 * it;
+    double da2 = 0.0;
+    if (u > 0.0) {
+      const double du = dalpha * 0.5 * rcp_nr(sqrt(u));
+      da2 = du * it - du * u * it * it * a2 * p.inv_cmax4;
+    }
+    cP = da2 * p.gamma * ir;
+    cr = da2 * a2 * ir;
+  } else {
+    float hL, lL, hR, lR;
+    ctot_pair_of(wL.k, wL.P, wL.ir, p, hL, lL);
+    ctot_pair_of(wR.k, wR.P, wR.ir, p, hR, lR);
+    left = hL > hR || (hL == hR && lL >= lR);
+    float h, l;
+    const double ir = left ? wL.ir : wR.ir, k = left ? wL.k : wR.k, P = left ? wL.P : wR.P;
+    alpha = pair_to_double(left ? hL : hR, left ? lL : lR);
+    sqrt_pair(k * ir, h, l);  // |V|
+    sv = h > 0.0f ? pair_to_double(h, l) : 0.0;
+    iv = h > 0.0f ? rcp_of_pair(h, l) : 0.0;
+    const double gir = p.gamma_xi2 * ir;
+    sqrt_pair(gir * P, h, l);  // a/xi
+    const double ca = pair_to_double(h, l), ica = h > 0.0f ? rcp_of_pair(h, l) : 0.0;
+    const double dh = half_of(dalpha);
+    cP = dh * (gir * ica);
+    cr = dh * (ca * ir);
+    dinv_xi = dalpha * (ca * p.xi);
+  }
+  double dqL[NV], dqR[NV];
+#pragma unroll
   for (int v = 0; v < NV; ++v) {
-    double da, db;
-    // qL = u0 + MC(u0 - um, u1 - u0)/2
-    mc_reverse(bL[v], 0.5 * dqL[v], da, db);
+    dqL[v] = alpha * f[v];
+    dqR[v] = -dqL[v];
+  }
+  flux_vjp<NV>(qL, p, wL, f, dqL);
+  flux_vjp<NV>(qR, p, wR, f, dqR);
+  {
+    // dc on its side: d|V|/dm_e = v_e/(rho |V|), d|V|/drho = -|V|/rho, and a/xi
+    // through P and rho
+    const double ir = left ? wL.ir : wR.ir, hv2 = left ? wL.hv2 : wR.hv2;
+    const double t = dalpha * ir, g = p.gm1 * cP, c = fma(t, iv, -g);
+    double x[NV];
+    x[0] = fma(g, hv2, fma(-t, sv, -cr));
+#pragma unroll
+    for (int e = 0; e < ND; ++e) x[1 + e] = c * (left ? wL.v[e] : wR.v[e]);
+    x[NV - 1] = g;
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+      const double y = (left ? dqL[v] : dqR[v]) + x[v];
+      dqL[v] = left ? y : dqL[v];
+      dqR[v] = left ? dqR[v] : y;
+    }
+  }
+#pragma unroll
+  for (int v = 0; v < NV; ++v) {
+    double da, db, ea, eb;
+    mc_reverse(bL[v], dqL[v], da, db);  // qL = u0 + h(u0 - um, u1 - u0)
+    mc_reverse(bR[v], dqR[v], ea, eb);  // qR = u1 - h(u1 - u0, up - u1)
     G[0][v] = -da;
-    G[1][v] = dqL[v] + da - db;
-    G[2][v] = db;
-    // qR = u1 - MC(u1 - u0, up - u1)/2
-    mc_reverse(bR[v], -0.5 * dqR[v], da, db);
-    G[1][v] -= da;
-    G[2][v] += dqR[v] + da - db;
-    G[3][v] = db;
+    G[1][v] = (dqL[v] + (da - db)) + ea;
+    G[2][v] = (dqR[v] - (ea - eb)) + db;
+    G[3][v] = -eb;
   }
   return dinv_xi;
 }
@@ -321,13 +336,16 @@ struct AdjArgs {
   const double* lam_out;  // lambda of the stage output, padded (interior used)
   double mu_scale;        // mu = mu_scale * lambda_out = b dt lambda_out
   double id_scale;        // the stage's identity part adds id_scale * lambda_out = b lambda_out
-  double* nu;        // padded, interior written (ghosts stay zero)
-  double* lam;       // padded output: pointwise part written to the interior
-  double* faceG;     // per axis: [face][4][NV]
-  double* part;      // per-block xi partials
+  const double* add;      // stage 1: lambda^{n+1}, half of which is added (may be lam itself); or null
+  double* nu;        // padded, interior written
+  double* lam;       // padded output (interior)
+  double* faceG;     // [4 stencil cells][NV][all faces]: coalesced for the faces and for the cells that gather
+  double* xi_part;   // [cells + all faces]: xi partials, accumulated over the stages
+  double xi_cell, xi_face;  // df/dxi and d(1/xi)/dxi
   Geom g;
   Phys p;
-  int64_t face_off[3];  // offset of each axis' block in faceG (in faces)
+  int64_t nfaces;       // of all axes
+  int64_t face_off[3];  // first face of each axis
 };
 
 __device__ __forceinline__ int64_t pidx_c(const Geom& g, const int (&c)[3]) { return pidx(g, c[0], c[1], c[2]); }
@@ -342,166 +360,130 @@ __device__ __forceinline__ void block_sum_to(double x, double* dst, double* sh) 
   if (threadIdx.x == 0) *dst = sh[0];
 }
 
-template <int NV, int D>
-__device__ __forceinline__ void load_stencil(const AdjArgs& a, const int (&c)[3], double (&s)[4][NV]) {
-  // cells c - 2 .. c + 1 along D (the face c - 1/2)
-  for (int k = 0; k < 4; ++k) {
-    int cc[3] = {c[0], c[1], c[2]};
-    cc[D] += k - 2;
-    const int64_t o = pidx_c(a.g, cc);
-    for (int v = 0; v < NV; ++v) s[k][v] = a.U[v * a.g.fstride + o];
-  }
-}
-
 template <int NV>
 __global__ void __launch_bounds__(128) adj_cell_kernel(AdjArgs a) {
-  __shared__ double sh[128];
   const Geom& g = a.g;
   const Phys& p = a.p;
-  double dxi = 0.0;
   const int64_t id = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (id < g.ncells) {
-    const int c[3] = {(int)(id % g.n[0]), (int)((id / g.n[0]) % g.n[1]), (int)(id / ((int64_t)g.n[0] * g.n[1]))};
-    const int64_t o = pidx_c(g, c);
-    double q[NV], dU[NV], mu[NV];
-    for (int v = 0; v < NV; ++v) {
-      q[v] = a.U[v * g.fstride + o];
-      mu[v] = a.mu_scale * a.lam_out[v * g.fstride + o];
-      dU[v] = a.dU[v * g.fstride + o];
-    }
-    // nu = mu^T dL/d(dU), pointwise mu^T dL/dq, xi partial (f = 1 - 1/xi^2)
-    double nu[NV], dq[NV];
-    const double df = rhs_vjp<NV>(q, dU, mu, p, nu, dq);
-    for (int v = 0; v < NV; ++v) {
-      a.nu[v * g.fstride + o] = nu[v];
-      a.lam[v * g.fstride + o] = fma(a.id_scale, a.lam_out[v * g.fstride + o], dq[v]);
-    }
-    const double xi = p.xi;
-    dxi = df * 2.0 / (xi * xi * xi);
+  if (id >= g.ncells) return;
+  const int c[3] = {(int)(id % g.n[0]), (int)((id / g.n[0]) % g.n[1]), (int)(id / ((int64_t)g.n[0] * g.n[1]))};
+  const int64_t o = pidx_c(g, c);
+  double q[NV], dU[NV], lo[NV], mu[NV];
+#pragma unroll
+  for (int v = 0; v < NV; ++v) {
+    q[v] = a.U[v * g.fstride + o];
+    lo[v] = a.lam_out[v * g.fstride + o];
+    mu[v] = a.mu_scale * lo[v];
+    dU[v] = a.dU[v * g.fstride + o];
   }
-  block_sum_to(dxi, a.part + blockIdx.x, sh);
+  // nu = mu^T dL/d(dU), pointwise mu^T dL/dq, xi partial (f = 1 - 1/xi^2)
+  double nu[NV], dq[NV];
+  const double df = rhs_vjp<NV>(q, dU, mu, p, nu, dq);
+#pragma unroll
+  for (int v = 0; v < NV; ++v) {
+    a.nu[v * g.fstride + o] = nu[v];
+    double l = fma(a.id_scale, lo[v], dq[v]);
+    if (a.add) l = fma(0.5, a.add[v * g.fstride + o], l);
+    a.lam[v * g.fstride + o] = l;
+  }
+  a.xi_part[id] = fma(df, a.xi_cell, a.xi_part[id]);
 }
 
-// Faces along D: index (f, other coords) with f in [0, n_D] (face f - 1/2).
-template <int NV, int D>
-__global__ void __launch_bounds__(128) adj_face_kernel(AdjArgs a, int part_off) {
-  __shared__ double sh[128];
+// Faces of axis blockIdx.y: index (f, other coords) with f in [0, n_D] (face
+// f - 1/2).  The axis enters through strides and the order of the momenta
+// only, so one launch takes all axes.
+template <int NV>
+__global__ void __launch_bounds__(128) adj_face_kernel(AdjArgs a) {
+  constexpr int ND = NV - 2;
   const Geom& g = a.g;
   const Phys& p = a.p;
+  const int D = blockIdx.y;
   int ext[3] = {g.n[0], g.n[1], g.n[2]};
   ext[D] += 1;
-  const int64_t nf = (int64_t)ext[0] * ext[1] * ext[2];
   const int64_t id = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  double dxi = 0.0;
-  if (id < nf) {
-    const int c[3] = {(int)(id % ext[0]), (int)((id / ext[0]) % ext[1]), (int)(id / ((int64_t)ext[0] * ext[1]))};
-    const int f = c[D];
-    double s[4][NV];
-    load_stencil<NV, D>(a, c, s);
-    // phi = (nu_right - nu_left) / dx, nu = 0 outside the interior
-    double phi[NV];
-    {
-      int cr[3] = {c[0], c[1], c[2]}, cl[3] = {c[0], c[1], c[2]};
-      cl[D] -= 1;
-      const bool has_r = f < g.n[D], has_l = f > 0;
-      const int64_t orr = pidx_c(g, cr), ol = pidx_c(g, cl);
-      for (int v = 0; v < NV; ++v) {
-        const double nr = has_r ? a.nu[v * g.fstride + orr] : 0.0;
-        const double nl = has_l ? a.nu[v * g.fstride + ol] : 0.0;
-        phi[v] = (nr - nl) * p.inv_dx[D];
-      }
-    }
-    double G[4][NV];
-    const double dinv_xi = face_vjp<NV, D>(s, phi, p, G);
-    double* dst = a.faceG + (a.face_off[D] + id) * (4 * NV);
-    for (int k = 0; k < 4; ++k)
-      for (int v = 0; v < NV; ++v) dst[k * NV + v] = G[k][v];
-    const double xi = p.xi;
-    dxi = -dinv_xi / (xi * xi);  // 1/xi -> xi
+  if (id >= (int64_t)ext[0] * ext[1] * ext[2]) return;
+  const int c[3] = {(int)(id % ext[0]), (int)((id / ext[0]) % ext[1]), (int)(id / ((int64_t)ext[0] * ext[1]))};
+  const int f = c[D];
+  const int64_t o = pidx_c(g, c);  // the cell right of the face
+  const int64_t st = D == 0 ? 1 : (D == 1 ? g.pitch : g.plane);
+  int fld[NV];  // normal momentum first
+  fld[0] = 0;
+  fld[NV - 1] = NV - 1;
+#pragma unroll
+  for (int e = 0; e < ND; ++e) fld[1 + e] = 1 + (e == 0 ? D : (e <= D ? e - 1 : e));
+  double s[4][NV], phi[NV], G[4][NV];
+  const bool has_r = f < g.n[D], has_l = f > 0;
+#pragma unroll
+  for (int v = 0; v < NV; ++v) {
+    const double* u = a.U + fld[v] * g.fstride + o;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) s[k][v] = u[(k - 2) * st];  // cells f - 2 .. f + 1
+    // phi/2 = (nu_right - nu_left) / (2 dx), nu = 0 outside the interior
+    const double* nu = a.nu + fld[v] * g.fstride + o;
+    phi[v] = ((has_r ? nu[0] : 0.0) - (has_l ? nu[-st] : 0.0)) * p.half_inv_dx[D];
   }
-  block_sum_to(dxi, a.part + part_off + blockIdx.x, sh);
+  const double dinv_xi = face_vjp<NV>(s, phi, p, G);
+  const int64_t fid = a.face_off[D] + id;
+#pragma unroll
+  for (int k = 0; k < 4; ++k)
+#pragma unroll
+    for (int v = 0; v < NV; ++v) a.faceG[(k * NV + fld[v]) * a.nfaces + fid] = G[k][v];
+  double* xp = a.xi_part + g.ncells + fid;
+  *xp = fma(dinv_xi, a.xi_face, *xp);
 }
 
-// Padded cell (interior, or an edge ghost along one axis) gathers the face
-// contributions of the faces f - 1/2, f in [c-1, c+2], along each axis.
+// Contributions to extended cell x along axis d of the line through cell c:
+// those of the faces f - 1/2, f in [x-1, x+2].
+template <int NV>
+__device__ __forceinline__ void gather_axis(const AdjArgs& a, const int (&c)[3], int d, int x, double (&acc)[NV]) {
+  const Geom& g = a.g;
+  int ext[3] = {g.n[0], g.n[1], g.n[2]};
+  ext[d] += 1;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {  // the cell's place in the face's stencil
+    const int f = x + 2 - k;
+    if (f < 0 || f > g.n[d]) continue;
+    int cf[3] = {c[0], c[1], c[2]};
+    cf[d] = f;
+    const double* G = a.faceG + a.face_off[d] + ((int64_t)cf[2] * ext[1] + cf[1]) * ext[0] + cf[0];
+#pragma unroll
+    for (int v = 0; v < NV; ++v) acc[v] += G[(k * NV + v) * a.nfaces];
+  }
+}
+
+// Each interior cell adds the face contributions to itself and to every ghost
+// cell that was copied from it.
 template <int NV>
 __global__ void __launch_bounds__(128) adj_gather_kernel(AdjArgs a) {
   constexpr int ND = NV - 2;
   const Geom& g = a.g;
-  const int ex = g.n[0] + 4, ey = ND >= 2 ? g.n[1] + 4 : 1, ez = ND >= 3 ? g.n[2] + 4 : 1;
-  const int64_t total = (int64_t)ex * ey * ez;
-  const int64_t id = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (id >= total) return;
-  const int c[3] = {(int)(id % ex) - 2, ND >= 2 ? (int)((id / ex) % ey) - 2 : 0,
-                    ND >= 3 ? (int)(id / ((int64_t)ex * ey)) - 2 : 0};
-  int outside = 0, oaxis = -1;
-  for (int d = 0; d < ND; ++d)
-    if (c[d] < 0 || c[d] >= g.n[d]) { ++outside; oaxis = d; }
-  if (outside > 1) return;  // corner ghosts take part in nothing
-  double acc[NV];
-  for (int v = 0; v < NV; ++v) acc[v] = 0.0;
-  for (int d = 0; d < ND; ++d) {
-    if (outside == 1 && oaxis != d) continue;  // a ghost along another axis is in no face of this axis
-    int ext[3] = {g.n[0], g.n[1], g.n[2]};
-    ext[d] += 1;
-    for (int f = c[d] - 1; f <= c[d] + 2; ++f) {
-      if (f < 0 || f > g.n[d]) continue;
-      int cf[3] = {c[0], c[1], c[2]};
-      cf[d] = f;
-      const int64_t fid = ((int64_t)cf[2] * ext[1] + cf[1]) * ext[0] + cf[0];
-      const int k = c[d] - f + 2;
-      const double* G = a.faceG + (a.face_off[d] + fid) * (4 * NV) + k * NV;
-      for (int v = 0; v < NV; ++v) acc[v] += G[v];
-    }
-  }
-  const int64_t o = pidx_c(g, c);
-  if (outside == 0) {
-    for (int v = 0; v < NV; ++v) a.lam[v * g.fstride + o] += acc[v];
-  } else {
-    for (int v = 0; v < NV; ++v) a.lam[v * g.fstride + o] = acc[v];
-  }
-}
-
-// Ghost adjoints back to their images: interior cell c within two cells of a
-// boundary adds every ghost that was copied from it.
-template <int NV>
-__global__ void __launch_bounds__(128) adj_fold_kernel(double* lam, Geom g, Phys p) {
-  constexpr int ND = NV - 2;
+  const Phys& p = a.p;
   const int64_t id = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (id >= g.ncells) return;
   const int c[3] = {(int)(id % g.n[0]), (int)((id / g.n[0]) % g.n[1]), (int)(id / ((int64_t)g.n[0] * g.n[1]))};
-  const int64_t o = pidx_c(g, c);
-  double add[NV];
-  for (int v = 0; v < NV; ++v) add[v] = 0.0;
+  double acc[NV];
+#pragma unroll
+  for (int v = 0; v < NV; ++v) acc[v] = 0.0;
+#pragma unroll
   for (int d = 0; d < ND; ++d) {
+    gather_axis<NV>(a, c, d, c[d], acc);
     const int n = g.n[d], cd = c[d];
+    if (cd >= RSST_G && cd < n - RSST_G) continue;
     for (int side = 0; side < 2; ++side) {
-      if (side == 0 ? !(cd < 2) : !(cd >= n - 2)) continue;
+      if (side == 0 ? cd >= RSST_G : cd < n - RSST_G) continue;
       const bool per = p.bc[d] == RSST_BC_PERIODIC;
       const int gp = per ? (side == 0 ? cd + n : cd - n) : (side == 0 ? -1 - cd : 2 * n - 1 - cd);
-      int cg[3] = {c[0], c[1], c[2]};
-      cg[d] = gp;
-      const int64_t og = pidx_c(g, cg);
-      for (int v = 0; v < NV; ++v) {
-        const double x = lam[v * g.fstride + og];
-        add[v] += (!per && v == 1 + d) ? -x : x;
-      }
+      double x[NV];
+#pragma unroll
+      for (int v = 0; v < NV; ++v) x[v] = 0.0;
+      gather_axis<NV>(a, c, d, gp, x);
+#pragma unroll
+      for (int v = 0; v < NV; ++v) acc[v] += (!per && v == 1 + d) ? -x[v] : x[v];
     }
   }
-  for (int v = 0; v < NV; ++v) lam[v * g.fstride + o] += add[v];
-}
-
-// out = alpha * x + beta * y over interior cells (padded arrays); ghosts of out set to 0.
-__global__ void axpby_kernel(double* out, const double* x, double alpha, const double* y, double beta, Geom g, int nv) {
-  const int64_t id = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (id >= g.ncells) return;
-  const int c[3] = {(int)(id % g.n[0]), (int)((id / g.n[0]) % g.n[1]), (int)(id / ((int64_t)g.n[0] * g.n[1]))};
   const int64_t o = pidx_c(g, c);
-  for (int v = 0; v < nv; ++v) {
-    const double xv = x ? x[v * g.fstride + o] : 0.0;
-    const double yv = y ? y[v * g.fstride + o] : 0.0;
-    out[v * g.fstride + o] = alpha * xv + beta * yv;
-  }
+#pragma unroll
+  for (int v = 0; v < NV; ++v) a.lam[v * g.fstride + o] += acc[v];
 }
 
 // caller layout <-> padded interior
@@ -547,6 +529,15 @@ __global__ void __launch_bounds__(128) ke_kernel(const double* U, Geom g, double
   block_sum_to(J, part + blockIdx.x, sh);
 }
 
+// Fixed-order sum of a block's share of x[0 .. n - 1] into part[blockIdx.x].
+__global__ void __launch_bounds__(256) sum_share_kernel(const double* x, int64_t n, double* part) {
+  __shared__ double sh[256];
+  const int64_t chunk = (n + gridDim.x - 1) / gridDim.x, lo = blockIdx.x * chunk, hi = min(n, lo + chunk);
+  double acc = 0.0;
+  for (int64_t i = lo + threadIdx.x; i < hi; i += 256) acc += x[i];
+  block_sum_to(acc, part + blockIdx.x, sh);
+}
+
 __global__ void sum_parts_kernel(const double* part, int n, double* out, int accumulate) {
   __shared__ double sh[256];
   double acc = 0.0;
@@ -575,16 +566,17 @@ struct AdjState {
   double* stages = nullptr;    // recompute storage: 2 * every padded states
   double* dUs = nullptr;       // their Euler tendencies (same layout)
   double* save = nullptr;      // the live state while a segment is recomputed
+  double* scal = nullptr;      // and its scalars
   double* lamA = nullptr;      // padded work arrays
   double* lamB = nullptr;
-  double* lamC = nullptr;
   double* nu = nullptr;
   double* faceG = nullptr;
-  double* part = nullptr;
-  double* dxi = nullptr;       // device accumulator
-  int64_t face_off[4] = {0, 0, 0, 0};
-  int part_len = 0;
+  double* xi_part = nullptr;   // xi partials of every cell and face of a segment
+  double* dxi = nullptr;       // [0] their sum, [1 ..] the sum's partials
+  int64_t face_off[3] = {0, 0, 0}, faces = 0;
 };
+
+constexpr int XI_BLOCKS = 256;  // blocks of the xi partials' sum
 
 static AdjState* adj_of(rsst_handle* h) { return reinterpret_cast<AdjState*>(h->adj); }
 
@@ -597,11 +589,11 @@ void rsst_adjoint_free(rsst_handle* h) {
   cudaFree(s->save);
   cudaFree(s->lamA);
   cudaFree(s->lamB);
-  cudaFree(s->lamC);
   cudaFree(s->nu);
   cudaFree(s->faceG);
-  cudaFree(s->part);
+  cudaFree(s->xi_part);
   cudaFree(s->dxi);
+  cudaFree(s->scal);
   delete s;
   h->adj = nullptr;
 }
@@ -632,42 +624,47 @@ extern "C" int rsst_adjoint_record(rsst_handle* h, double dt, int nsteps, int ev
     rsst_set_error("rsst_adjoint_record: the adjoint is derived for the ideal gas only");
     return RSST_EUNSUPPORTED;
   }
-  rsst_adjoint_free(h);
-  AdjState* s = new AdjState();
-  h->adj = s;
+  // A recording of the same shape reuses the last one's memory (allocating
+  // and freeing it costs milliseconds and synchronises the device).
+  const int nseg = (nsteps + every - 1) / every;
+  AdjState* s = adj_of(h);
+  if (!s || s->every != every || s->nseg != nseg) {
+    rsst_adjoint_free(h);
+    s = new AdjState();
+    h->adj = s;
+    s->every = every;
+    s->nseg = nseg;
+    const size_t sb = state_bytes(h);
+    const Geom& g = h->g;
+    for (int d = 0; d < g.ndim; ++d) {
+      s->face_off[d] = s->faces;
+      s->faces += g.ncells / g.n[d] * (g.n[d] + 1);
+    }
+    const int nv = g.ndim + 2;
+    bool ok = cudaMalloc((void**)&s->stages, 2 * (size_t)every * sb) == cudaSuccess &&
+              cudaMalloc((void**)&s->dUs, 2 * (size_t)every * sb) == cudaSuccess &&
+              cudaMalloc((void**)&s->save, sb) == cudaSuccess &&
+              cudaMalloc((void**)&s->scal, 16 * sizeof(double)) == cudaSuccess &&
+              cudaMalloc((void**)&s->lamA, sb) == cudaSuccess && cudaMalloc((void**)&s->lamB, sb) == cudaSuccess &&
+              cudaMalloc((void**)&s->nu, sb) == cudaSuccess &&
+              cudaMalloc((void**)&s->faceG, (size_t)s->faces * 4 * nv * sizeof(double)) == cudaSuccess &&
+              cudaMalloc((void**)&s->xi_part, (size_t)(g.ncells + s->faces) * sizeof(double)) == cudaSuccess &&
+              cudaMalloc((void**)&s->dxi, (1 + XI_BLOCKS) * sizeof(double)) == cudaSuccess;
+    for (int k = 0; ok && k < s->nseg; ++k) {
+      double* c = nullptr;
+      ok = cudaMalloc((void**)&c, sb) == cudaSuccess;
+      s->ckpt.push_back(c);
+    }
+    if (!ok) {
+      cudaGetLastError();
+      rsst_adjoint_free(h);
+      rsst_set_error("rsst_adjoint_record: device allocation failed");
+      return RSST_ENOMEM;
+    }
+  }
   s->dt = dt;
   s->nsteps = nsteps;
-  s->every = every;
-  s->nseg = (nsteps + every - 1) / every;
   const size_t sb = state_bytes(h);
-  const Geom& g = h->g;
-  int64_t faces = 0;
-  for (int d = 0; d < g.ndim; ++d) {
-    s->face_off[d] = faces;
-    faces += g.ncells / g.n[d] * (g.n[d] + 1);
-  }
-  s->part_len = blocks_for(g.ncells) + 3 * blocks_for(faces) + 8;
-  const int nv = g.ndim + 2;
-  bool ok = cudaMalloc((void**)&s->stages, 2 * (size_t)every * sb) == cudaSuccess &&
-            cudaMalloc((void**)&s->dUs, 2 * (size_t)every * sb) == cudaSuccess &&
-            cudaMalloc((void**)&s->save, sb) == cudaSuccess &&
-            cudaMalloc((void**)&s->lamA, sb) == cudaSuccess && cudaMalloc((void**)&s->lamB, sb) == cudaSuccess &&
-            cudaMalloc((void**)&s->lamC, sb) == cudaSuccess &&
-            cudaMalloc((void**)&s->nu, sb) == cudaSuccess &&
-            cudaMalloc((void**)&s->faceG, (size_t)faces * 4 * nv * sizeof(double)) == cudaSuccess &&
-            cudaMalloc((void**)&s->part, (size_t)s->part_len * sizeof(double)) == cudaSuccess &&
-            cudaMalloc((void**)&s->dxi, sizeof(double)) == cudaSuccess;
-  for (int k = 0; ok && k < s->nseg; ++k) {
-    double* c = nullptr;
-    ok = cudaMalloc((void**)&c, sb) == cudaSuccess;
-    s->ckpt.push_back(c);
-  }
-  if (!ok) {
-    cudaGetLastError();
-    rsst_adjoint_free(h);
-    rsst_set_error("rsst_adjoint_record: device allocation failed");
-    return RSST_ENOMEM;
-  }
   for (int step = 0; step < nsteps; ++step) {
     if (step % every == 0) {
       if (cudaMemcpyAsync(s->ckpt[step / every], h->buf[0], sb, cudaMemcpyDeviceToDevice, h->stream) != cudaSuccess) {
@@ -689,16 +686,14 @@ extern "C" int rsst_adjoint_segments(rsst_handle* h, int32_t* nseg) {
 
 // lam_out (padded, interior) -> its contribution through one stage.
 // in: the stage input state; b: coefficient of (in + dt L(in)).
-// Writes lam_in = b lam_out + (b dt lam_out)^T dL/d(in) into `res` (padded,
-// interior, ghosts folded) and adds the xi partials to s->dxi.
+// Writes b lam_out + (b dt lam_out)^T dL/d(in), plus add/2 if given, into
+// `res` (padded, interior; may be `add`) and adds the xi partials.
 static int stage_vjp(rsst_handle* h, AdjState* s, const double* in, const double* dU, const double* lam_out, double b,
-                     double* res) {
-  // No clearing is needed: the cell kernel writes nu and res at every
-  // interior cell, the face kernels read nu at interior cells only, and the
-  // gather writes every edge ghost of res that the fold reads.
+                     const double* add, double* res) {
   const Geom& g = h->g;
   const int nv = g.ndim + 2;
   cudaStream_t st = h->stream;
+  const double xi = h->p.xi;
   AdjArgs a;
   memset(&a, 0, sizeof a);
   a.U = in;
@@ -706,43 +701,36 @@ static int stage_vjp(rsst_handle* h, AdjState* s, const double* in, const double
   a.lam_out = lam_out;
   a.mu_scale = b * s->dt;
   a.id_scale = b;
+  a.add = add;
   a.nu = s->nu;
   a.lam = res;
   a.faceG = s->faceG;
-  a.part = s->part;
+  a.xi_part = s->xi_part;
+  a.xi_cell = 2.0 / (xi * xi * xi);
+  a.xi_face = -1.0 / (xi * xi);
   a.g = g;
   a.p = h->p;
+  a.nfaces = s->faces;
+  int64_t nf = 0;
   for (int d = 0; d < 3; ++d) a.face_off[d] = s->face_off[d];
-  const int cb = blocks_for(g.ncells);
-  switch (nv) {
-    case 3: adj_cell_kernel<3><<<cb, 128, 0, st>>>(a); break;
-    case 4: adj_cell_kernel<4><<<cb, 128, 0, st>>>(a); break;
-    default: adj_cell_kernel<5><<<cb, 128, 0, st>>>(a); break;
-  }
-  int rc = launch_err("adjoint cell kernel");
-  if (rc) return rc;
-  int off = cb;
   for (int d = 0; d < g.ndim; ++d) {
-    const int64_t nf = g.ncells / g.n[d] * (g.n[d] + 1);
-    const int fb = blocks_for(nf);
-#define FK(NVv, Dd) adj_face_kernel<NVv, Dd><<<fb, 128, 0, st>>>(a, off)
-    if (nv == 3) FK(3, 0);
-    else if (nv == 4) { if (d == 0) FK(4, 0); else FK(4, 1); }
-    else { if (d == 0) FK(5, 0); else if (d == 1) FK(5, 1); else FK(5, 2); }
-#undef FK
-    rc = launch_err("adjoint face kernel");
-    if (rc) return rc;
-    off += fb;
+    const int64_t m = g.ncells / g.n[d] * (g.n[d] + 1);
+    nf = m > nf ? m : nf;
   }
-  sum_parts_kernel<<<1, 256, 0, st>>>(s->part, off, s->dxi, 1);
-  const int64_t padded = (int64_t)(g.n[0] + 4) * (g.ndim >= 2 ? g.n[1] + 4 : 1) * (g.ndim >= 3 ? g.n[2] + 4 : 1);
+  const int cb = blocks_for(g.ncells);
+  const dim3 fb(blocks_for(nf), g.ndim);
+#define RSST_VJP(NVv)                                \
+  adj_cell_kernel<NVv><<<cb, 128, 0, st>>>(a);       \
+  adj_face_kernel<NVv><<<fb, 128, 0, st>>>(a);       \
+  adj_gather_kernel<NVv><<<cb, 128, 0, st>>>(a)
   switch (nv) {
-    case 3: adj_gather_kernel<3><<<blocks_for(padded), 128, 0, st>>>(a); adj_fold_kernel<3><<<cb, 128, 0, st>>>(res, g, h->p); break;
-    case 4: adj_gather_kernel<4><<<blocks_for(padded), 128, 0, st>>>(a); adj_fold_kernel<4><<<cb, 128, 0, st>>>(res, g, h->p); break;
-    default: adj_gather_kernel<5><<<blocks_for(padded), 128, 0, st>>>(a); adj_fold_kernel<5><<<cb, 128, 0, st>>>(res, g, h->p); break;
+    case 3: RSST_VJP(3); break;
+    case 4: RSST_VJP(4); break;
+    default: RSST_VJP(5); break;
   }
-  h->launches += 4 + g.ndim;
-  return launch_err("adjoint gather/fold");
+#undef RSST_VJP
+  h->launches += 3;
+  return launch_err("adjoint stage kernels");
 }
 
 extern "C" int rsst_adjoint_step(rsst_handle* h, int32_t seg, double* lam, double* dJ_dxi) {
@@ -765,10 +753,7 @@ extern "C" int rsst_adjoint_step(rsst_handle* h, int32_t seg, double* lam, doubl
   auto chk = [&](cudaError_t e) { if (ce == cudaSuccess && e != cudaSuccess) ce = e; };
   int rc = RSST_OK;
   const int slot0 = h->slot;
-  double save_scal[16];
-  chk(cudaMemcpyAsync(h->h_small, h->d_scal, 16 * sizeof(double), cudaMemcpyDeviceToHost, st));
-  chk(cudaStreamSynchronize(st));
-  memcpy(save_scal, h->h_small, sizeof save_scal);
+  chk(cudaMemcpyAsync(s->scal, h->d_scal, 16 * sizeof(double), cudaMemcpyDeviceToDevice, st));
   chk(cudaMemcpyAsync(s->save, h->buf[0], sb, cudaMemcpyDeviceToDevice, st));
   chk(cudaMemcpyAsync(h->buf[0], s->ckpt[seg], sb, cudaMemcpyDeviceToDevice, st));
   for (int i = 0; i < k && rc == RSST_OK && ce == cudaSuccess; ++i) {
@@ -781,18 +766,16 @@ extern "C" int rsst_adjoint_step(rsst_handle* h, int32_t seg, double* lam, doubl
     chk(cudaMemcpyAsync(s->stages + (2 * i + 1) * fe, h->buf[1], sb, cudaMemcpyDeviceToDevice, st));
   }
   chk(cudaMemcpyAsync(h->buf[0], s->save, sb, cudaMemcpyDeviceToDevice, st));
-  memcpy(h->h_small, save_scal, sizeof save_scal);
-  chk(cudaMemcpyAsync(h->d_scal, h->h_small, 16 * sizeof(double), cudaMemcpyHostToDevice, st));
-  chk(cudaStreamSynchronize(st));
+  chk(cudaMemcpyAsync(h->d_scal, s->scal, 16 * sizeof(double), cudaMemcpyDeviceToDevice, st));
   if (rc == RSST_OK && ce != cudaSuccess) {
     rsst_set_error("rsst_adjoint_step: segment recompute: %s", cudaGetErrorString(ce));
     rc = RSST_ECUDA;
   }
   h->slot = slot0;
   if (rc == RSST_OK) {
-    if (cudaMemsetAsync(s->dxi, 0, sizeof(double), st) != cudaSuccess ||
-        cudaMemsetAsync(s->lamA, 0, sb, st) != cudaSuccess) {
-      rsst_set_error("rsst_adjoint_step: clearing the work arrays failed");
+    const int64_t parts = g.ncells + s->faces;
+    if (cudaMemsetAsync(s->xi_part, 0, (size_t)parts * sizeof(double), st) != cudaSuccess) {
+      rsst_set_error("rsst_adjoint_step: clearing the xi partials failed");
       return RSST_ECUDA;
     }
     to_padded_kernel<<<blocks_for(g.ncells), 128, 0, st>>>(lam, s->lamA, g, nv);
@@ -800,14 +783,13 @@ extern "C" int rsst_adjoint_step(rsst_handle* h, int32_t seg, double* lam, doubl
       const double* Un = s->stages + (2 * i) * fe;
       const double* Us = s->stages + (2 * i + 1) * fe;
       // stage 2: U^{n+1} = 1/2 U^n + 1/2 (U* + dt L(U*)):  lamB = lambda_*
-      rc = stage_vjp(h, s, Us, s->dUs + (2 * i + 1) * fe, s->lamA, 0.5, s->lamB);
+      rc = stage_vjp(h, s, Us, s->dUs + (2 * i + 1) * fe, s->lamA, 0.5, nullptr, s->lamB);
       if (rc) break;
-      // stage 1: U* = U^n + dt L(U^n):  lamC = lambda_* dU*/dU^n
-      rc = stage_vjp(h, s, Un, s->dUs + (2 * i) * fe, s->lamB, 1.0, s->lamC);
-      if (rc) break;
-      // lambda^n = 1/2 lambda^{n+1} + lamC
-      axpby_kernel<<<blocks_for(g.ncells), 128, 0, st>>>(s->lamA, s->lamA, 0.5, s->lamC, 1.0, g, nv);
+      // stage 1: U* = U^n + dt L(U^n):  lambda^n = lambda_* dU*/dU^n + 1/2 lambda^{n+1}, in place
+      rc = stage_vjp(h, s, Un, s->dUs + (2 * i) * fe, s->lamB, 1.0, s->lamA, s->lamA);
     }
+    sum_share_kernel<<<XI_BLOCKS, 256, 0, st>>>(s->xi_part, parts, s->dxi + 1);
+    sum_parts_kernel<<<1, 256, 0, st>>>(s->dxi + 1, XI_BLOCKS, s->dxi, 0);
     from_padded_kernel<<<blocks_for(g.ncells), 128, 0, st>>>(s->lamA, lam, g, nv);
     rc = rc ? rc : launch_err("adjoint transfer");
   }
