@@ -408,7 +408,7 @@ __device__ __forceinline__ void rhs_prep(const double (&q)[NV], const Phys& p, R
   const double kin = 0.5 * k;
   const int var = p.variant;
   const double f = p.use_cmax ? f_of(Eos<CV>::sound2(p, rho, P, ir), p) : p.f;
-  r.H = Eos<CV>::enthalpy(p, rho, P) + (var == RSST_PVS || var == RSST_DVS ? kin : -kin);
+  r.H = fma(var == RSST_PVS || var == RSST_DVS ? 0.5 : -0.5, k, Eos<CV>::enthalpy(p, rho, P));
   if (var == RSST_PVS || var == RSST_PMS || var == RSST_PD) {
     r.hv2 = Eos<CV>::half_v2_minus_de_drho(p, kin * ir, P);
     r.a = Eos<CV>::f_over_de_dP(p, f, rho, P);
@@ -468,15 +468,16 @@ __device__ __forceinline__ void rsst_rhs(const double (&q)[NV], double (&dU)[NV]
   rhs_apply<NV>(q, dU, p, r);
 }
 
-// Half of a double (as 0.5 * x rounds it), on the integer pipe.
+// Half of a double (as 0.5 * x rounds it), on the integer pipe.  The sign is
+// taken off the high word (a 64-bit mask would become a float64 absolute value).
 __device__ __forceinline__ double half_of(double x) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-  const unsigned long long sign = b & (1ull << 63), mag = b ^ sign;
-  const unsigned e = (unsigned)(mag >> 52);
-  if (e == 2047u) return x;
+  const int hi = __double2hiint(x), lo = __double2loint(x);
+  const unsigned s = (unsigned)hi & 0x80000000u, e = ((unsigned)hi >> 20) & 0x7ffu;
+  if (e >= 2u) return __hiloint2double(e == 2047u ? hi : hi - (1 << 20), lo);
   // at and below the smallest normal exponent the pattern counts units of 2^-1074
-  const unsigned long long h = e >= 2u ? mag - (1ull << 52) : (mag + ((mag >> 1) & 1ull)) >> 1;
-  return __longlong_as_double((long long)(sign | h));
+  const unsigned long long mag = ((unsigned long long)((unsigned)hi ^ s) << 32) | (unsigned)lo;
+  const unsigned long long h = (mag + ((mag >> 1) & 1ull)) >> 1;
+  return __hiloint2double((int)((unsigned)(h >> 32) | s), (int)(unsigned)h);
 }
 
 // From the bit pattern (a float64 compare occupies the float64 pipe).
