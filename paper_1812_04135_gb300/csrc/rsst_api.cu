@@ -432,24 +432,15 @@ extern "C" int rsst_set_state(rsst_handle* h, const double* U, int on_host) {
     CUDA_TRY(cudaMemcpyAsync(h->d_stage, U, bytes, cudaMemcpyHostToDevice, h->stream));
     src = h->d_stage;
   }
-  const bool f32 = h->cfg.precision == RSST_FP32_PERT;
-  const bool dfp = h->cfg.precision == RSST_FP64_DF;
-  if (f32)
-    RC_TRY(rsst_launch_pack_fp32(src, (float*)h->buf[0], h->g, h->p, h->d_bg, h->bg_len, h->stream));
-  else if (dfp)
-    RC_TRY(rsst_launch_pack_df(src, (float2*)h->buf[0], h->g, h->p, h->d_bg, h->bg_len, h->stream));
+  double* cfl = h->d_scal + h->slot;
+  RC_TRY(rsst_launch_reset(h->d_scal, h->slot, h->d_flag, h->stream));
+  if (h->cfg.precision == RSST_FP32_PERT)
+    RC_TRY(rsst_launch_pack_fp32(src, (float*)h->buf[0], h->g, h->p, h->pf, h->d_bg, h->bg_len, h->d_tab, cfl,
+                                 h->d_flag, h->stream));
+  else if (h->cfg.precision == RSST_FP64_DF)
+    RC_TRY(rsst_launch_pack_df(src, (float2*)h->buf[0], h->g, h->p, h->d_bg, h->bg_len, cfl, h->d_flag, h->stream));
   else
-    RC_TRY(rsst_launch_pack_fp64(src, (double*)h->buf[0], h->g, h->p, h->d_bg, h->bg_len, h->stream));
-  CUDA_TRY(cudaMemsetAsync(h->d_flag, 0, sizeof(unsigned int), h->stream));
-  CUDA_TRY(cudaMemsetAsync(h->d_scal + h->slot, 0, sizeof(double), h->stream));
-  CUDA_TRY(cudaMemsetAsync(h->d_scal + 3, 0, sizeof(double), h->stream));  // simulated time
-  if (dfp)
-    RC_TRY(rsst_launch_cfl_df((const float2*)h->buf[0], h->g, h->p, h->d_scal + h->slot, h->d_flag, h->stream));
-  else if (f32)
-    RC_TRY(rsst_launch_cfl_fp32((const float*)h->buf[0], h->g, h->p, h->pf, h->d_tab, h->bg_len, h->d_scal + h->slot,
-                                h->d_flag, h->stream));
-  else
-    RC_TRY(rsst_launch_cfl_fp64((const double*)h->buf[0], h->g, h->p, h->d_scal + h->slot, h->d_flag, h->stream));
+    RC_TRY(rsst_launch_pack_fp64(src, (double*)h->buf[0], h->g, h->p, h->d_bg, h->bg_len, cfl, h->d_flag, h->stream));
   h->launches += 2;
   return RSST_OK;
 }

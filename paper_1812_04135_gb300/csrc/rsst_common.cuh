@@ -10,6 +10,47 @@ __device__ __forceinline__ int64_t pidx(const Geom& g, int i, int j, int k) {
   return (int64_t)(k + g.gz) * g.plane + (int64_t)(j + g.gy) * g.pitch + (i + g.xoff);
 }
 
+// Conversions between float64 and float32 on the integer pipe: the conversion
+// instructions run at the float64 pipe's rate (a warp instruction per 16 SM
+// clocks), which bounds a kernel that only moves data.  The same values and
+// rounding (to nearest even, subnormals included; a NaN becomes the quiet one).
+// Signs are taken off the high word: a 64-bit mask or xor of the sign is turned
+// back into a float64 absolute value or negation.
+static __device__ __noinline__ unsigned d2f_rare(unsigned long long m) {  // not a normal float (out of line: it rarely runs)
+  const int e = (int)(m >> 52);
+  if (e > 1150) return m > 0x7ff0000000000000ull ? 0x7fc00000u : 0x7f800000u;
+  // units of 2^-149: the significand shifted by 29 + (897 - e)
+  const int sh = min(926 - e, 63);
+  const unsigned long long q = (m & 0xfffffffffffffull) | (e > 0 ? 1ull << 52 : 0ull);
+  return (unsigned)((q + ((1ull << (sh - 1)) - 1ull) + ((q >> sh) & 1ull)) >> sh);
+}
+__device__ __forceinline__ float d2f_rn(double d) {
+  const unsigned hi = (unsigned)__double2hiint(d), s = hi & 0x80000000u;
+  const unsigned long long m = ((unsigned long long)(hi ^ s) << 32) | (unsigned)__double2loint(d);
+  const int e = (int)(m >> 52);
+  // normal floats; a carry past the largest gives infinity
+  unsigned f = (unsigned)((m + 0x0fffffffull + ((m >> 29) & 1ull)) >> 29) - (896u << 23);
+  if ((unsigned)(e - 897) >= 254u) f = m == 0ull ? 0u : d2f_rare(m);
+  return __uint_as_float(s | f);
+}
+__device__ __forceinline__ double f2d(float x) {
+  const unsigned b = __float_as_uint(x);
+  unsigned m = b & 0x7fffffffu;
+  int bias = 896;
+  if (m < 0x00800000u) {  // subnormal: normalise
+    const int n = __clz(m) - 8;
+    m = m == 0u ? 0u : m << n;
+    bias = m == 0u ? 0 : 896 - n;
+  } else if (m >= 0x7f800000u) {
+    bias = 1792;  // exponent 255 -> 2047
+  }
+  const unsigned long long v = ((unsigned long long)m << 29) + ((unsigned long long)bias << 52);
+  return __hiloint2double((int)((unsigned)(v >> 32) | (b & 0x80000000u)), (int)(unsigned)v);
+}
+__device__ __forceinline__ double flip_sign(double x) {
+  return __hiloint2double(__double2hiint(x) ^ (int)0x80000000u, __double2loint(x));
+}
+
 // Maximum of non-negative doubles, whose bit patterns order like their
 // values: on the integer pipe (a float64 compare or maximum occupies the
 // float64 pipe as long as an FMA).

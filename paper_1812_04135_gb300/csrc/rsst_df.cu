@@ -12,11 +12,14 @@
 // in pairs that share a difference, rho |V|^2 = m.V, the C_max law and the
 // stage as template arguments, and the tile by TMA instead of loads and index
 // arithmetic.  512^2: 40.9 -> 27.2 us a stage; 3D 90 x 70 x 50: 112 -> 74 us.
+#include <climits>
+
 #include "rsst_common.cuh"
 #include "rsst_internal.h"
 #include "rsst_attr.h"
 #include "rsst_math_df.cuh"
 #include "rsst_tma.cuh"
+#include "rsst_transfer.cuh"
 
 namespace rsst {
 
@@ -367,79 +370,31 @@ __global__ void __launch_bounds__(NT, MINB)
 // Packing, CFL maximum, sums (double-float storage)
 // ---------------------------------------------------------------------------
 
-__global__ void pack_df_kernel(const double* __restrict__ src, float2* __restrict__ dst, Geom g, Phys p,
-                               const double* __restrict__ bg, int bg_len) {
-  const int nv = g.ndim + 2;
-  const int ex = g.n[0] + 2 * RSST_G;
-  const int ey = g.ndim >= 2 ? g.n[1] + 2 * RSST_G : 1;
-  const int ez = g.ndim >= 3 ? g.n[2] + 2 * RSST_G : 1;
-  const int64_t total = (int64_t)ex * ey * ez;
-  for (int64_t id = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; id < total; id += (int64_t)gridDim.x * blockDim.x) {
-    const int c[3] = {(int)(id % ex) - RSST_G, g.ndim >= 2 ? (int)((id / ex) % ey) - RSST_G : 0,
-                      g.ndim >= 3 ? (int)(id / ((int64_t)ex * ey)) - RSST_G : 0};
-    int s[3] = {c[0], c[1], c[2]};
-    double sign[3] = {1.0, 1.0, 1.0};
-    int vimg = 0, vgh = 0;
-    bool vmirror = false;
-    for (int d = 0; d < g.ndim; ++d) {
-      const int n = g.n[d];
-      if (s[d] >= 0 && s[d] < n) continue;
-      if (p.bc[d] == RSST_BC_PERIODIC) {
-        s[d] = (s[d] + n) % n;
-      } else {
-        const int img = s[d] < 0 ? -1 - s[d] : 2 * n - 1 - s[d];
-        if (d == p.vertical) { vgh = s[d]; vimg = img; vmirror = true; }
-        s[d] = img;
-        sign[d] = -1.0;
-      }
+// Storage of a double-float run (rsst_transfer.cuh), ghosts as in float64.
+template <int NV_>
+struct StoreDF {
+  static constexpr int NV = NV_;
+  float2* u;
+  int64_t fs;
+  const double* bg;
+  int bg_len;
+  PhysDF p;
+  __device__ __forceinline__ void store(int64_t o, double (&w)[NV], int sv, int gv) const {
+    if (gv != INT_MIN && bg != nullptr) {
+      w[0] += bg[gv + RSST_G] - bg[sv + RSST_G];
+      w[NV - 1] += bg[bg_len + gv + RSST_G] - bg[bg_len + sv + RSST_G];
     }
-    const int64_t si = ((int64_t)s[2] * g.n[1] + s[1]) * g.n[0] + s[0];
-    const int64_t di = pidx(g, c[0], c[1], c[2]);
-    for (int v = 0; v < nv; ++v) {
-      double w = src[v * g.ncells + si];
-      if (v >= 1 && v <= g.ndim) w *= sign[v - 1];
-      if (bg != nullptr && vmirror && (v == 0 || v == nv - 1)) {
-        const double* row = bg + (v == 0 ? 0 : bg_len);
-        w += row[vgh + RSST_G] - row[vimg + RSST_G];
-      }
-      st_df(dst, v * g.fstride + di, df_from(w));
-    }
+#pragma unroll
+    for (int v = 0; v < NV; ++v) st_df(u, v * fs + o, df_from_bits(w[v]));
   }
-}
-
-__global__ void unpack_df_kernel(const float2* __restrict__ src, double* __restrict__ dst, Geom g) {
-  const int nv = g.ndim + 2;
-  for (int64_t id = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; id < g.ncells; id += (int64_t)gridDim.x * blockDim.x) {
-    const int i = (int)(id % g.n[0]);
-    const int j = (int)((id / g.n[0]) % g.n[1]);
-    const int k = (int)(id / ((int64_t)g.n[0] * g.n[1]));
-    const int64_t o = pidx(g, i, j, k);
-    for (int v = 0; v < nv; ++v) dst[v * g.ncells + id] = df_to(ld_df(src, v * g.fstride + o));
-  }
-}
-
-template <int NV>
-__global__ void __launch_bounds__(256) cfl_df_kernel(const float2* __restrict__ U, Geom g, PhysDF p, double* dst,
-                                                     unsigned int* flag) {
-  __shared__ df sred[32];
-  df rmax = {0.0f, 0.0f};
-  bool ok_all = true;
-  for (int64_t id = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; id < g.ncells; id += (int64_t)gridDim.x * blockDim.x) {
-    const int i = (int)(id % g.n[0]);
-    const int j = (int)((id / g.n[0]) % g.n[1]);
-    const int k = (int)(id / ((int64_t)g.n[0] * g.n[1]));
-    const int64_t o = pidx(g, i, j, k);
+  __device__ __forceinline__ double rate(const double (&w)[NV], int, bool& ok) const {
     df q[NV];
 #pragma unroll
-    for (int v = 0; v < NV; ++v) q[v] = ld_df(U, v * g.fstride + o);
-    bool ok;
-    const df r = cfl_rate_df<NV>(q, p, ok);
-    if (ok && df_lt(rmax, r)) rmax = r;
-    ok_all = ok_all && ok;
+    for (int v = 0; v < NV; ++v) q[v] = df_from_bits(w[v]);
+    return df_to_bits(cfl_rate_df<NV>(q, p, ok));
   }
-  if (!ok_all) atomicOr(flag, RSST_FLAG_NONPHYSICAL);
-  block_max_df<256>(rmax, dst, sred);
-}
+  __device__ __forceinline__ double load(int64_t o, int v, int) const { return df_to_bits(ld_df(u, v * fs + o)); }
+};
 
 constexpr int SUM_BLOCKS_DF = 1024;
 constexpr int SUM_THREADS_DF = 256;
@@ -600,12 +555,6 @@ int rsst_launch_stage_df(const CUtensorMap* tin, const StageArgs<float2>& sa, cu
   return RSST_EINVAL;
 }
 
-static int grid_df(int64_t n) {
-  int64_t b = (n + 255) / 256;
-  if (b > 152 * 16) b = 152 * 16;
-  return (int)(b < 1 ? 1 : b);
-}
-
 static int err_df(const char* what) {
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) {
@@ -616,27 +565,18 @@ static int err_df(const char* what) {
 }
 
 int rsst_launch_pack_df(const double* src, float2* dst, const Geom& g, const Phys& p, const double* bg, int bg_len,
-                        cudaStream_t s) {
-  const int64_t total = (int64_t)(g.n[0] + 4) * (g.ndim >= 2 ? g.n[1] + 4 : 1) * (g.ndim >= 3 ? g.n[2] + 4 : 1);
-  pack_df_kernel<<<grid_df(total), 256, 0, s>>>(src, dst, g, p, bg, bg_len);
-  return err_df("pack (double-float)");
+                        double* cfl, unsigned int* flag, cudaStream_t s) {
+  const PhysDF q = make_physdf(p);
+#define PACK(NV) launch_pack(src, g, p, StoreDF<NV>{dst, g.fstride, bg, bg_len, q}, cfl, flag, "pack (double-float)", s)
+  return g.ndim == 1 ? PACK(3) : (g.ndim == 2 ? PACK(4) : PACK(5));
+#undef PACK
 }
 
 int rsst_launch_unpack_df(const float2* src, double* dst, const Geom& g, cudaStream_t s) {
-  unpack_df_kernel<<<grid_df(g.ncells), 256, 0, s>>>(src, dst, g);
-  return err_df("unpack (double-float)");
-}
-
-int rsst_launch_cfl_df(const float2* U, const Geom& g, const Phys& p, double* slot_ptr, unsigned int* flag,
-                       cudaStream_t s) {
-  const PhysDF q = make_physdf(p);
-  const int gb = grid_df(g.ncells);
-  switch (g.ndim) {
-    case 1: cfl_df_kernel<3><<<gb, 256, 0, s>>>(U, g, q, slot_ptr, flag); break;
-    case 2: cfl_df_kernel<4><<<gb, 256, 0, s>>>(U, g, q, slot_ptr, flag); break;
-    default: cfl_df_kernel<5><<<gb, 256, 0, s>>>(U, g, q, slot_ptr, flag); break;
-  }
-  return err_df("cfl (double-float)");
+#define UNPACK(NV) \
+  launch_unpack(dst, g, -1, StoreDF<NV>{const_cast<float2*>(src), g.fstride, nullptr, 0, PhysDF{}}, "unpack (double-float)", s)
+  return g.ndim == 1 ? UNPACK(3) : (g.ndim == 2 ? UNPACK(4) : UNPACK(5));
+#undef UNPACK
 }
 
 int rsst_launch_sums_df(const float2* U, const Geom& g, double* partial, double* out, double scale_, cudaStream_t s) {

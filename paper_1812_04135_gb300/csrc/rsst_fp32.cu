@@ -8,11 +8,14 @@
 // kernels then advance U1 with dU1/dt = R0 + [L(U0+U1) - L(U0)], every term
 // of the bracket formed from perturbation-sized quantities (see
 // rsst_math_fp32.cuh).  Tile structure is that of the float64 kernel.
+#include <climits>
+
 #include "rsst_common.cuh"
 #include "rsst_internal.h"
 #include "rsst_attr.h"
 #include "rsst_math_fp32.cuh"
 #include "rsst_math_fp64.cuh"
+#include "rsst_transfer.cuh"
 
 namespace rsst {
 
@@ -452,99 +455,58 @@ __device__ __forceinline__ void bg_at(const double* bg, int bg_len, int kpad, do
   }
 }
 
-// U1 = U - U0 at interior cells; ghosts: wrap, or mirror of U1 (normal momentum negated).
-__global__ void pack_fp32_kernel(const double* __restrict__ src, float* __restrict__ dst, Geom g, Phys p,
-                                 const double* __restrict__ bg, int bg_len) {
-  const int nv = g.ndim + 2;
-  const int ex = g.n[0] + 2 * RSST_G;
-  const int ey = g.ndim >= 2 ? g.n[1] + 2 * RSST_G : 1;
-  const int ez = g.ndim >= 3 ? g.n[2] + 2 * RSST_G : 1;
-  const int64_t total = (int64_t)ex * ey * ez;
-  for (int64_t id = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; id < total; id += (int64_t)gridDim.x * blockDim.x) {
-    const int c[3] = {(int)(id % ex) - RSST_G, g.ndim >= 2 ? (int)((id / ex) % ey) - RSST_G : 0,
-                      g.ndim >= 3 ? (int)(id / ((int64_t)ex * ey)) - RSST_G : 0};
-    int s[3] = {c[0], c[1], c[2]};
-    double sign[3] = {1.0, 1.0, 1.0};
-    for (int d = 0; d < g.ndim; ++d) {
-      const int n = g.n[d];
-      if (s[d] >= 0 && s[d] < n) continue;
-      if (p.bc[d] == RSST_BC_PERIODIC) {
-        s[d] = (s[d] + n) % n;
-      } else {
-        s[d] = s[d] < 0 ? -1 - s[d] : 2 * n - 1 - s[d];
-        sign[d] = -1.0;
-      }
+// Storage of a float32-perturbation run (rsst_transfer.cuh): U1 = U - U0 in
+// float32; ghosts wrap or mirror U1 (U0 taken at the source cell).
+template <int NV_>
+struct StoreF32 {
+  static constexpr int NV = NV_, ND = NV - 2;
+  float* u;
+  int64_t fs;
+  const double* bg;
+  int bg_len;
+  const float* tab;
+  PhysF pf;
+  __device__ __forceinline__ void store(int64_t o, double (&w)[NV], int sv, int) const {
+    if (bg != nullptr) {
+      double r0, e0;
+      bg_at(bg, bg_len, sv + RSST_G, r0, e0);
+      w[0] -= r0;
+      w[NV - 1] -= e0;
     }
-    double r0 = 0.0, e0 = 0.0;
-    if (p.vertical >= 0) bg_at(bg, bg_len, s[p.vertical] + RSST_G, r0, e0);
-    const int64_t si = ((int64_t)s[2] * g.n[1] + s[1]) * g.n[0] + s[0];
-    const int64_t di = pidx(g, c[0], c[1], c[2]);
-    for (int v = 0; v < nv; ++v) {
-      double w = src[v * g.ncells + si];
-      if (v == 0) w -= r0;
-      if (v == nv - 1) w -= e0;
-      if (v >= 1 && v <= g.ndim) w *= sign[v - 1];
-      dst[v * g.fstride + di] = (float)w;
-    }
+#pragma unroll
+    for (int v = 0; v < NV; ++v) u[v * fs + o] = d2f_rn(w[v]);
   }
-}
-
-__global__ void unpack_fp32_kernel(const float* __restrict__ src, double* __restrict__ dst, Geom g, Phys p,
-                                   const double* __restrict__ bg, int bg_len) {
-  const int nv = g.ndim + 2;
-  for (int64_t id = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; id < g.ncells; id += (int64_t)gridDim.x * blockDim.x) {
-    const int c[3] = {(int)(id % g.n[0]), (int)((id / g.n[0]) % g.n[1]), (int)(id / ((int64_t)g.n[0] * g.n[1]))};
-    const int64_t o = pidx(g, c[0], c[1], c[2]);
-    double r0 = 0.0, e0 = 0.0;
-    if (p.vertical >= 0) bg_at(bg, bg_len, c[p.vertical] + RSST_G, r0, e0);
-    for (int v = 0; v < nv; ++v) {
-      double w = (double)src[v * g.fstride + o];
-      if (v == 0) w += r0;
-      if (v == nv - 1) w += e0;
-      dst[v * g.ncells + id] = w;
-    }
-  }
-}
-
-template <int NV>
-__global__ void __launch_bounds__(256) cfl_fp32_kernel(const float* __restrict__ U, Geom g, Phys p, PhysF pf,
-                                                       const float* __restrict__ tab, int tab_len, double* dst,
-                                                       unsigned int* flag) {
-  constexpr int ND = NV - 2;
-  __shared__ double sred[8];
-  float rmax = 0.0f;
-  bool ok_all = true;
-  for (int64_t id = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; id < g.ncells; id += (int64_t)gridDim.x * blockDim.x) {
-    const int c[3] = {(int)(id % g.n[0]), (int)((id / g.n[0]) % g.n[1]), (int)(id / ((int64_t)g.n[0] * g.n[1]))};
-    const int64_t o = pidx(g, c[0], c[1], c[2]);
+  // after store: w holds U1
+  __device__ __forceinline__ double rate(const double (&w)[NV], int sv, bool& ok) const {
     float rho0 = 0.0f, P0 = 0.0f;
     if (tab) {
-      const int kp = c[p.vertical] + RSST_G;
-      rho0 = tab[TB_RHO0 * tab_len + kp];
-      P0 = tab[TB_P0 * tab_len + kp];
+      rho0 = tab[TB_RHO0 * bg_len + sv + RSST_G];
+      P0 = tab[TB_P0 * bg_len + sv + RSST_G];
     }
-    float u[NV];
+    float q[NV];
 #pragma unroll
-    for (int v = 0; v < NV; ++v) u[v] = U[v * g.fstride + o];
-    const float rn = rho0 + u[0];
+    for (int v = 0; v < NV; ++v) q[v] = d2f_rn(w[v]);
+    const float rn = rho0 + q[0];
     const float irn = 1.0f / rn;
     float w2 = 0.0f, mw = 0.0f;
-    bool fin = isfinite(u[0]) && isfinite(u[NV - 1]);
+    bool fin = isfinite(q[0]) && isfinite(q[NV - 1]);
 #pragma unroll
     for (int e = 0; e < ND; ++e) {
-      const float ve = u[1 + e] * irn;
+      const float ve = q[1 + e] * irn;
       w2 += ve * ve;
-      mw += u[1 + e] * ve;
-      fin = fin && isfinite(u[1 + e]);
+      mw += q[1 + e] * ve;
+      fin = fin && isfinite(q[1 + e]);
     }
-    const float Pn = P0 + pf.gm1 * (u[NV - 1] - 0.5f * mw);
-    const bool ok = fin && rn > 0.0f && Pn > 0.0f;
-    if (ok) rmax = fmaxf(rmax, (sqrtf(w2) + sound_over_xi_f(pf.gamma * Pn * irn, pf)) * pf.sum_inv_dx);
-    ok_all = ok_all && ok;
+    const float Pn = P0 + pf.gm1 * (q[NV - 1] - 0.5f * mw);
+    ok = fin && rn > 0.0f && Pn > 0.0f;
+    return f2d((sqrtf(w2) + sound_over_xi_f(pf.gamma * Pn * irn, pf)) * pf.sum_inv_dx);
   }
-  if (!ok_all) atomicOr(flag, RSST_FLAG_NONPHYSICAL);
-  block_max_to<256>((double)rmax, dst, sred);
-}
+  __device__ __forceinline__ double load(int64_t o, int v, int vi) const {
+    double x = f2d(u[v * fs + o]);
+    if (bg != nullptr && (v == 0 || v == NV - 1)) x += bg[(v == 0 ? 0 : bg_len) + vi + RSST_G];
+    return x;
+  }
+};
 
 constexpr int SUM_BLOCKS32 = 1024;
 constexpr int SUM_THREADS32 = 256;
@@ -668,34 +630,22 @@ int rsst_launch_bgtab(const double* bg, int bg_len, const Geom& g, const Phys& p
   return check_launch32("background table");
 }
 
-static int grid_for32(int64_t n) {
-  int64_t b = (n + 255) / 256;
-  if (b > 152 * 16) b = 152 * 16;
-  return (int)(b < 1 ? 1 : b);
-}
-
-int rsst_launch_pack_fp32(const double* src, float* dst, const Geom& g, const Phys& p, const double* bg, int bg_len,
+int rsst_launch_pack_fp32(const double* src, float* dst, const Geom& g, const Phys& p, const PhysF& pf,
+                          const double* bg, int bg_len, const float* tab, double* cfl, unsigned int* flag,
                           cudaStream_t s) {
-  const int64_t total = (int64_t)(g.n[0] + 4) * (g.ndim >= 2 ? g.n[1] + 4 : 1) * (g.ndim >= 3 ? g.n[2] + 4 : 1);
-  pack_fp32_kernel<<<grid_for32(total), 256, 0, s>>>(src, dst, g, p, bg, bg_len);
-  return check_launch32("pack (float32)");
+#define PACK(NV) launch_pack(src, g, p, StoreF32<NV>{dst, g.fstride, bg, bg_len, tab, pf}, cfl, flag, "pack (float32)", s)
+  return g.ndim == 1 ? PACK(3) : (g.ndim == 2 ? PACK(4) : PACK(5));
+#undef PACK
 }
 
 int rsst_launch_unpack_fp32(const float* src, double* dst, const Geom& g, const Phys& p, const double* bg, int bg_len,
                             cudaStream_t s) {
-  unpack_fp32_kernel<<<grid_for32(g.ncells), 256, 0, s>>>(src, dst, g, p, bg, bg_len);
-  return check_launch32("unpack (float32)");
-}
-
-int rsst_launch_cfl_fp32(const float* U, const Geom& g, const Phys& p, const PhysF& pf, const float* tab, int tab_len,
-                         double* slot_ptr, unsigned int* flag, cudaStream_t s) {
-  const int gb = grid_for32(g.ncells);
-  switch (g.ndim) {
-    case 1: cfl_fp32_kernel<3><<<gb, 256, 0, s>>>(U, g, p, pf, tab, tab_len, slot_ptr, flag); break;
-    case 2: cfl_fp32_kernel<4><<<gb, 256, 0, s>>>(U, g, p, pf, tab, tab_len, slot_ptr, flag); break;
-    default: cfl_fp32_kernel<5><<<gb, 256, 0, s>>>(U, g, p, pf, tab, tab_len, slot_ptr, flag); break;
-  }
-  return check_launch32("cfl (float32)");
+  const int vert = p.vertical;
+#define UNPACK(NV)                                                                                                   \
+  launch_unpack(dst, g, vert, StoreF32<NV>{const_cast<float*>(src), g.fstride, vert >= 0 ? bg : nullptr, bg_len,     \
+                                           nullptr, PhysF{}}, "unpack (float32)", s)
+  return g.ndim == 1 ? UNPACK(3) : (g.ndim == 2 ? UNPACK(4) : UNPACK(5));
+#undef UNPACK
 }
 
 int rsst_launch_sums_fp32(const float* U, const Geom& g, const Phys& p, const double* bg, int bg_len, double* partial,

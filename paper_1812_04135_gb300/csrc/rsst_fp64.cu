@@ -28,6 +28,7 @@
 // the block maximum, a per-thread dt division and unshared slope differences
 // on that pipe.  512^2: 123 -> 92 us a stage; 3D 256 x 128 x 128: 3090 -> 2500
 // us; 2048^2 runs the pipe 86 % busy.
+#include <climits>
 #include <cstdio>
 
 #include "rsst_common.cuh"
@@ -35,6 +36,7 @@
 #include "rsst_attr.h"
 #include "rsst_math_fp64.cuh"
 #include "rsst_tma.cuh"
+#include "rsst_transfer.cuh"
 
 namespace rsst {
 
@@ -362,83 +364,29 @@ __global__ void __launch_bounds__(NT, MINB)
 // Packing, CFL maximum, sums
 // ---------------------------------------------------------------------------
 
-// Caller layout [nvar][nz][ny][nx] -> padded layout, ghost cells included.
-// Each padded cell maps every out-of-range coordinate to its source by the
-// boundary rule (periodic wrap, or mirror with the normal momentum negated and
-// the background difference added); corner ghosts are filled too (unused).
-__global__ void pack_fp64_kernel(const double* __restrict__ src, double* __restrict__ dst, Geom g, Phys p,
-                                 const double* __restrict__ bg, int bg_len) {
-  const int nv = g.ndim + 2;
-  const int ex = g.n[0] + 2 * RSST_G;
-  const int ey = g.ndim >= 2 ? g.n[1] + 2 * RSST_G : 1;
-  const int ez = g.ndim >= 3 ? g.n[2] + 2 * RSST_G : 1;
-  const int64_t total = (int64_t)ex * ey * ez;
-  for (int64_t id = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; id < total; id += (int64_t)gridDim.x * blockDim.x) {
-    const int c[3] = {(int)(id % ex) - RSST_G, g.ndim >= 2 ? (int)((id / ex) % ey) - RSST_G : 0,
-                      g.ndim >= 3 ? (int)(id / ((int64_t)ex * ey)) - RSST_G : 0};
-    int s[3] = {c[0], c[1], c[2]};
-    double sign[3] = {1.0, 1.0, 1.0};
-    int vimg = 0, vgh = 0;
-    bool vmirror = false;
-    for (int d = 0; d < g.ndim; ++d) {
-      const int n = g.n[d];
-      if (s[d] >= 0 && s[d] < n) continue;
-      if (p.bc[d] == RSST_BC_PERIODIC) {
-        s[d] = (s[d] + n) % n;
-      } else {
-        const int img = s[d] < 0 ? -1 - s[d] : 2 * n - 1 - s[d];
-        if (d == p.vertical) { vgh = s[d]; vimg = img; vmirror = true; }
-        s[d] = img;
-        sign[d] = -1.0;
-      }
+// Storage of a float64 run (rsst_transfer.cuh): values as they are; a ghost
+// mirrored across a wall of the vertical axis gets the background's difference.
+template <int NV_, bool CV>
+struct StoreF64 {
+  static constexpr int NV = NV_;
+  double* u;
+  int64_t fs;
+  const double* bg;
+  int bg_len;
+  Phys p;
+  __device__ __forceinline__ void store(int64_t o, double (&w)[NV], int sv, int gv) const {
+    if (gv != INT_MIN && bg != nullptr) {
+      w[0] += bg[gv + RSST_G] - bg[sv + RSST_G];
+      w[NV - 1] += bg[bg_len + gv + RSST_G] - bg[bg_len + sv + RSST_G];
     }
-    const int64_t si = ((int64_t)s[2] * g.n[1] + s[1]) * g.n[0] + s[0];
-    const int64_t di = pidx(g, c[0], c[1], c[2]);
-    for (int v = 0; v < nv; ++v) {
-      double w = src[v * g.ncells + si];
-      if (v >= 1 && v <= g.ndim) w *= sign[v - 1];
-      if (bg != nullptr && vmirror && (v == 0 || v == nv - 1)) {
-        const double* row = bg + (v == 0 ? 0 : bg_len);
-        w += row[vgh + RSST_G] - row[vimg + RSST_G];
-      }
-      dst[v * g.fstride + di] = w;
-    }
-  }
-}
-
-__global__ void unpack_fp64_kernel(const double* __restrict__ src, double* __restrict__ dst, Geom g) {
-  const int nv = g.ndim + 2;
-  for (int64_t id = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; id < g.ncells; id += (int64_t)gridDim.x * blockDim.x) {
-    const int i = (int)(id % g.n[0]);
-    const int j = (int)((id / g.n[0]) % g.n[1]);
-    const int k = (int)(id / ((int64_t)g.n[0] * g.n[1]));
-    const int64_t o = pidx(g, i, j, k);
-    for (int v = 0; v < nv; ++v) dst[v * g.ncells + id] = src[v * g.fstride + o];
-  }
-}
-
-template <int NV, bool CV>
-__global__ void __launch_bounds__(256) cfl_fp64_kernel(const double* __restrict__ U, Geom g, Phys p, double* dst,
-                                                       unsigned int* flag) {
-  __shared__ double sred[8];
-  double rmax = 0.0;
-  bool ok_all = true;
-  for (int64_t id = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; id < g.ncells; id += (int64_t)gridDim.x * blockDim.x) {
-    const int i = (int)(id % g.n[0]);
-    const int j = (int)((id / g.n[0]) % g.n[1]);
-    const int k = (int)(id / ((int64_t)g.n[0] * g.n[1]));
-    const int64_t o = pidx(g, i, j, k);
-    double q[NV];
 #pragma unroll
-    for (int v = 0; v < NV; ++v) q[v] = U[v * g.fstride + o];
-    bool ok;
-    const double r = cfl_rate<NV, CV>(q, p, ok);
-    if (ok) rmax = max_nonneg(rmax, r);
-    ok_all = ok_all && ok;
+    for (int v = 0; v < NV; ++v) u[v * fs + o] = w[v];
   }
-  if (!ok_all) atomicOr(flag, RSST_FLAG_NONPHYSICAL);
-  block_max_to<256>(rmax, dst, sred);
-}
+  __device__ __forceinline__ double rate(const double (&w)[NV], int, bool& ok) const {
+    return cfl_rate<NV, CV>(w, p, ok);
+  }
+  __device__ __forceinline__ double load(int64_t o, int v, int) const { return u[v * fs + o]; }
+};
 
 // Deterministic sums: block b reduces a fixed contiguous chunk of cells with a
 // fixed thread striding and shared-memory tree; a single block then reduces
@@ -577,12 +525,6 @@ int rsst_launch_stage_fp64(const CUtensorMap* tin, const StageArgs<double>& a, c
   return RSST_EINVAL;
 }
 
-static int grid_for(int64_t n) {
-  int64_t b = (n + 255) / 256;
-  if (b > 152 * 16) b = 152 * 16;
-  return (int)(b < 1 ? 1 : b);
-}
-
 static int check_launch(const char* what) {
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) {
@@ -592,36 +534,31 @@ static int check_launch(const char* what) {
   return RSST_OK;
 }
 
+namespace rsst {
+__global__ void reset_kernel(double* scal, int slot, unsigned int* flag) {
+  scal[slot] = 0.0;
+  scal[3] = 0.0;  // simulated time
+  *flag = 0u;
+}
+}  // namespace rsst
+
+int rsst_launch_reset(double* scal, int slot, unsigned int* flag, cudaStream_t s) {
+  reset_kernel<<<1, 1, 0, s>>>(scal, slot, flag);
+  return check_launch("reset");
+}
+
 int rsst_launch_pack_fp64(const double* src, double* dst, const Geom& g, const Phys& p, const double* bg, int bg_len,
-                          cudaStream_t s) {
-  const int64_t total = (int64_t)(g.n[0] + 4) * (g.ndim >= 2 ? g.n[1] + 4 : 1) * (g.ndim >= 3 ? g.n[2] + 4 : 1);
-  pack_fp64_kernel<<<grid_for(total), 256, 0, s>>>(src, dst, g, p, bg, bg_len);
-  return check_launch("pack");
+                          double* cfl, unsigned int* flag, cudaStream_t s) {
+#define PACK(NV, CV) launch_pack(src, g, p, StoreF64<NV, CV>{dst, g.fstride, bg, bg_len, p}, cfl, flag, "pack", s)
+  if (p.covol != 0.0) return g.ndim == 1 ? PACK(3, true) : (g.ndim == 2 ? PACK(4, true) : PACK(5, true));
+  return g.ndim == 1 ? PACK(3, false) : (g.ndim == 2 ? PACK(4, false) : PACK(5, false));
+#undef PACK
 }
 
 int rsst_launch_unpack_fp64(const double* src, double* dst, const Geom& g, cudaStream_t s) {
-  unpack_fp64_kernel<<<grid_for(g.ncells), 256, 0, s>>>(src, dst, g);
-  return check_launch("unpack");
-}
-
-int rsst_launch_cfl_fp64(const double* U, const Geom& g, const Phys& p, double* slot_ptr, unsigned int* flag,
-                         cudaStream_t s) {
-  const int gb = grid_for(g.ncells);
-  switch (g.ndim) {
-    case 1:
-      if (p.covol != 0.0) cfl_fp64_kernel<3, true><<<gb, 256, 0, s>>>(U, g, p, slot_ptr, flag);
-      else cfl_fp64_kernel<3, false><<<gb, 256, 0, s>>>(U, g, p, slot_ptr, flag);
-      break;
-    case 2:
-      if (p.covol != 0.0) cfl_fp64_kernel<4, true><<<gb, 256, 0, s>>>(U, g, p, slot_ptr, flag);
-      else cfl_fp64_kernel<4, false><<<gb, 256, 0, s>>>(U, g, p, slot_ptr, flag);
-      break;
-    default:
-      if (p.covol != 0.0) cfl_fp64_kernel<5, true><<<gb, 256, 0, s>>>(U, g, p, slot_ptr, flag);
-      else cfl_fp64_kernel<5, false><<<gb, 256, 0, s>>>(U, g, p, slot_ptr, flag);
-      break;
-  }
-  return check_launch("cfl");
+#define UNPACK(NV) launch_unpack(dst, g, -1, StoreF64<NV, false>{const_cast<double*>(src), g.fstride, nullptr, 0, Phys{}}, "unpack", s)
+  return g.ndim == 1 ? UNPACK(3) : (g.ndim == 2 ? UNPACK(4) : UNPACK(5));
+#undef UNPACK
 }
 
 int rsst_launch_sums_fp64(const double* U, const Geom& g, double* partial, double* out, double scale, cudaStream_t s) {

@@ -142,11 +142,12 @@ int rsst_stage_fp64_tile(const Geom& g, int sms);
 // Short 1D float64 lines: many steps in one launch on a thread-block cluster.
 int rsst_line_fp64_ok(const Geom& g, const Phys& p);
 int rsst_launch_line_fp64(const StageArgs<double>& a, int nsteps, int* launches, cudaStream_t s);
-int rsst_launch_pack_fp64(const double* src, double* dst, const Geom& g, const Phys& p,
-                          const double* bg, int bg_len, cudaStream_t s);
+// Loading a state: ghosts filled, the CFL maximum added to *cfl and the flag set
+// for a non-physical state (both cleared before by rsst_launch_reset).
+int rsst_launch_reset(double* scal, int slot, unsigned int* flag, cudaStream_t s);
+int rsst_launch_pack_fp64(const double* src, double* dst, const Geom& g, const Phys& p, const double* bg, int bg_len,
+                          double* cfl, unsigned int* flag, cudaStream_t s);
 int rsst_launch_unpack_fp64(const double* src, double* dst, const Geom& g, cudaStream_t s);
-int rsst_launch_cfl_fp64(const double* U, const Geom& g, const Phys& p, double* slot_ptr,
-                         unsigned int* flag, cudaStream_t s);
 int rsst_launch_sums_fp64(const double* U, const Geom& g, double* partial, double* out,
                           double scale, cudaStream_t s);
 
@@ -156,21 +157,18 @@ int rsst_launch_stage_df(const CUtensorMap* tin, const StageArgs<float2>& a, cud
 void rsst_stage_df_box(const Geom& g, int tile, int* sx, int* sy, int* sz);
 int rsst_stage_df_tile(const Geom& g, int sms);
 int rsst_launch_pack_df(const double* src, float2* dst, const Geom& g, const Phys& p, const double* bg, int bg_len,
-                        cudaStream_t s);
+                        double* cfl, unsigned int* flag, cudaStream_t s);
 int rsst_launch_unpack_df(const float2* src, double* dst, const Geom& g, cudaStream_t s);
-int rsst_launch_cfl_df(const float2* U, const Geom& g, const Phys& p, double* slot_ptr, unsigned int* flag,
-                       cudaStream_t s);
 int rsst_launch_sums_df(const float2* U, const Geom& g, double* partial, double* out, double scale_, cudaStream_t s);
 int rsst_launch_stage2d_tma(const CUtensorMap* tin, const StageArgs<float>& a, cudaStream_t s);
 int rsst_launch_stage3d_tma(const CUtensorMap* tin, const StageArgs<float>& a, cudaStream_t s);
 int rsst_launch_bgtab(const double* bg, int bg_len, const Geom& g, const Phys& p, float* tab, float* tabr,
                       cudaStream_t s);
-int rsst_launch_pack_fp32(const double* src, float* dst, const Geom& g, const Phys& p, const double* bg,
-                          int bg_len, cudaStream_t s);
+int rsst_launch_pack_fp32(const double* src, float* dst, const Geom& g, const Phys& p, const PhysF& pf,
+                          const double* bg, int bg_len, const float* tab, double* cfl, unsigned int* flag,
+                          cudaStream_t s);
 int rsst_launch_unpack_fp32(const float* src, double* dst, const Geom& g, const Phys& p, const double* bg,
                             int bg_len, cudaStream_t s);
-int rsst_launch_cfl_fp32(const float* U, const Geom& g, const Phys& p, const PhysF& pf, const float* tab,
-                         int tab_len, double* slot_ptr, unsigned int* flag, cudaStream_t s);
 int rsst_launch_sums_fp32(const float* U, const Geom& g, const Phys& p, const double* bg, int bg_len,
                           double* partial, double* out, double scale, cudaStream_t s);
 

@@ -16,6 +16,7 @@
 // (Sec. 3.2, App. A) and force (App. B).
 #pragma once
 
+#include "rsst_common.cuh"
 #include "rsst_internal.h"
 
 namespace rsst {
@@ -92,6 +93,13 @@ __device__ __forceinline__ df df_from(double d) {
   return {h, __double2float_rn(d - (double)h)};
 }
 __device__ __forceinline__ double df_to(df x) { return (double)x.hi + (double)x.lo; }
+
+// The same two conversions with one float64 operation each (see d2f_rn).
+__device__ __forceinline__ df df_from_bits(double d) {
+  const float h = d2f_rn(d);
+  return {h, d2f_rn(d - f2d(h))};
+}
+__device__ __forceinline__ double df_to_bits(df x) { return f2d(x.hi) + f2d(x.lo); }
 
 // Constants of the step in double-float (split once on the host).
 struct PhysDF {
