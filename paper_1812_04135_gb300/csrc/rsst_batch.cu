@@ -54,7 +54,7 @@ __global__ void __launch_bounds__(C::NT) batch_stage_kernel(const BatchRun* __re
   __syncthreads();
   uint32_t phase = 0;
   // The next tile's list entry, this thread's word of its run descriptor and
-  // (thread 0) its CFL slot value are loaded one tile ahead, so that no
+  // (thread 32) its CFL slot value are loaded one tile ahead, so that no
   // dependent global load stands between two tiles.
   int t = blockIdx.x;
   int2 ti = make_int2(0, 0);
@@ -64,7 +64,7 @@ __global__ void __launch_bounds__(C::NT) batch_stage_kernel(const BatchRun* __re
     e = tile_info[u];
     const BatchRun& rb = runs[e.x];
     if (threadIdx.x < NW) dword = reinterpret_cast<const unsigned long long*>(&rb.r[stage - 1])[threadIdx.x];
-    if (threadIdx.x == 0) {
+    if (threadIdx.x == 32) {
       cfl = rb.r[0].p.cfl;
       cmax_slot = rb.scal[slot];
     }
@@ -73,7 +73,8 @@ __global__ void __launch_bounds__(C::NT) batch_stage_kernel(const BatchRun* __re
   for (; t < total_tiles; t += gridDim.x) {
     const BatchRun& br = runs[ti.x];
     if (threadIdx.x < NW) reinterpret_cast<unsigned long long*>(sr)[threadIdx.x] = dword;
-    if (threadIdx.x == 0) {
+    __syncthreads();
+    if (threadIdx.x == 32) {  // dt's float64 division runs beside the tile's copy
       const double dtd = cfl / cmax_slot;
       *sdt = (float)dtd;
       if (stage == 1 && ti.y == 0) {
@@ -82,7 +83,6 @@ __global__ void __launch_bounds__(C::NT) batch_stage_kernel(const BatchRun* __re
         br.scal[3] += dtd;
       }
     }
-    __syncthreads();
     int2 tnext = ti;
     if (t + (int)gridDim.x < total_tiles) fetch(t + gridDim.x, tnext);
     const int tx = ti.y % br.tiles_x, ty = ti.y / br.tiles_x;
@@ -94,11 +94,11 @@ __global__ void __launch_bounds__(C::NT) batch_stage_kernel(const BatchRun* __re
     const bool cm = sr->pf.use_cmax != 0;
     bool fine;
     if (br.vert == 1)
-      fine = cm ? tile2d_f<C, 1, -1, 1, ST>(map, *sr, *sdt, tx, ty, smem_raw, phase, rmax, ok)
-                : tile2d_f<C, 1, -1, 0, ST>(map, *sr, *sdt, tx, ty, smem_raw, phase, rmax, ok);
+      fine = cm ? tile2d_f<C, 1, -1, 1, ST>(map, *sr, sdt, tx, ty, smem_raw, phase, rmax, ok)
+                : tile2d_f<C, 1, -1, 0, ST>(map, *sr, sdt, tx, ty, smem_raw, phase, rmax, ok);
     else
-      fine = cm ? tile2d_f<C, -1, -1, 1, ST>(map, *sr, *sdt, tx, ty, smem_raw, phase, rmax, ok)
-                : tile2d_f<C, -1, -1, 0, ST>(map, *sr, *sdt, tx, ty, smem_raw, phase, rmax, ok);
+      fine = cm ? tile2d_f<C, -1, -1, 1, ST>(map, *sr, sdt, tx, ty, smem_raw, phase, rmax, ok)
+                : tile2d_f<C, -1, -1, 0, ST>(map, *sr, sdt, tx, ty, smem_raw, phase, rmax, ok);
     if (!fine) {
       // A bounded wait gave up (the tile routine has already waited for its
       // copy).  This block leaves the rest of the stage: every run that owns

@@ -41,7 +41,12 @@ __global__ void __launch_bounds__(T2::NT, 5) stage2d_tma_kernel(const __grid_con
   uint64_t* bar = t2_barrier<T2>(smem_raw);
   float* sdt = reinterpret_cast<float*>(bar + 1);
   if (threadIdx.x == 0) {
-    // the float64 division is done once per CTA, not per thread
+    mbar_init(bar, 1);
+    fence_mbar_init();
+  }
+  __syncthreads();
+  if (threadIdx.x == 32) {
+    // the float64 division is done once per CTA, beside the tile's copy
     const double dtd = a.dt_fixed > 0.0 ? a.dt_fixed : a.p.cfl / a.scal[a.slot];
     *sdt = (float)dtd;
     if (ST == 1 && blockIdx.x == 0 && blockIdx.y == 0) {
@@ -49,15 +54,11 @@ __global__ void __launch_bounds__(T2::NT, 5) stage2d_tma_kernel(const __grid_con
       a.scal[2] = dtd;
       a.scal[3] += dtd;
     }
-    mbar_init(bar, 1);
-    fence_mbar_init();
   }
-  __syncthreads();
-  const float dtf = *sdt;
   uint32_t phase = 0;
   float rmax = 0.0f;
   bool ok = true;
-  const bool fine = tile2d_f<T2, VERT, FORM, CM, ST>(&tin, r, dtf, blockIdx.x, blockIdx.y, smem_raw, phase, rmax, ok);
+  const bool fine = tile2d_f<T2, VERT, FORM, CM, ST>(&tin, r, sdt, blockIdx.x, blockIdx.y, smem_raw, phase, rmax, ok);
   if (!fine) return;
   if (ST == 2) {
     if (!ok) atomicOr(a.flag, RSST_FLAG_NONPHYSICAL);

@@ -92,10 +92,11 @@ struct TileRun {
 // Process tile (tx, ty) of run r: returns false if a bounded wait gave up
 // (flag set, nothing left in flight).  Accumulates the stage-2 CFL rate
 // maximum and physical check.  The caller initialised the barrier; `phase` is
-// its current parity.  FORM, CM and ST fix the form, the C_max law and the
+// its current parity.  *sdt (shared memory) may be written up to the routine's
+// first barriers: the tile's copy does not wait for dt's float64 division.  FORM, CM and ST fix the form, the C_max law and the
 // stage at compile time (-1, -1, 0: read from the run).
 template <class T2, int VERT, int FORM, int CM, int ST>
-__device__ __forceinline__ bool tile2d_f(const CUtensorMap* tin, const TileRun& r, float dt, int tx, int ty,
+__device__ __forceinline__ bool tile2d_f(const CUtensorMap* tin, const TileRun& r, const float* sdt, int tx, int ty,
                                          unsigned char* smem, uint32_t& phase, float& rmax, bool& ok_all) {
   constexpr int NV = 4;
   constexpr bool BG = VERT >= 0;
@@ -150,6 +151,7 @@ __device__ __forceinline__ bool tile2d_f(const CUtensorMap* tin, const TileRun& 
     }
   }
 
+  const float dt = *sdt;
   const int nx = g.n[0], ny = g.n[1];
   const int lane = tid & 31;
   // ---- x faces.  The slope cells of every row form one flat list; chunk k

@@ -84,6 +84,11 @@ __global__ void __launch_bounds__(T3::NT, 5) stage3d_tma_kernel(const __grid_con
   const int pfirst = k0 - 2, plast = k1 + 1;  // planes needed by this chunk
 
   if (tid == 0) {
+    for (int s = 0; s < T3::NS; ++s) mbar_init(&bar[s], 1);
+    fence_mbar_init();
+  }
+  __syncthreads();
+  if (tid == 32) {  // dt's float64 division runs beside the first planes' copies
     const double dtd = a.dt_fixed > 0.0 ? a.dt_fixed : p.cfl / a.scal[a.slot];
     *sdt = (float)dtd;
     if (ST == 1 && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0) {
@@ -91,10 +96,7 @@ __global__ void __launch_bounds__(T3::NT, 5) stage3d_tma_kernel(const __grid_con
       a.scal[2] = dtd;
       a.scal[3] += dtd;
     }
-    for (int s = 0; s < T3::NS; ++s) mbar_init(&bar[s], 1);
-    fence_mbar_init();
   }
-  __syncthreads();
   auto slot_of = [&](int pl) { return (pl - pfirst) % T3::NS; };
   auto phase_of = [&](int pl) { return (uint32_t)(((pl - pfirst) / T3::NS) & 1); };
   auto issue = [&](int pl) {
@@ -115,7 +117,6 @@ __global__ void __launch_bounds__(T3::NT, 5) stage3d_tma_kernel(const __grid_con
     for (int id = tid; id < N4; id += T3::NT)
       dst[id] = first4 + id < last4 ? src[first4 + id] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
   }
-  const float dt = *sdt;
   int waited = pfirst - 1;  // planes up to this one are resident
   auto wait_upto = [&](int pl) -> bool {
     for (int q = waited + 1; q <= pl; ++q) {
@@ -156,6 +157,7 @@ __global__ void __launch_bounds__(T3::NT, 5) stage3d_tma_kernel(const __grid_con
     }
   }
 
+  const float dt = *sdt;
   const int cx = lane, cy = tid >> 5;
   const int x = i0 + cx, y = j0 + cy;
   const bool colok = x < nx && y < ny;
