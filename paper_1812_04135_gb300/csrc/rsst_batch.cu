@@ -94,11 +94,11 @@ __global__ void __launch_bounds__(C::NT) batch_stage_kernel(const BatchRun* __re
     const bool cm = sr->pf.use_cmax != 0;
     bool fine;
     if (br.vert == 1)
-      fine = cm ? tile2d_f<C, 1, -1, 1, ST>(map, *sr, sdt, tx, ty, smem_raw, phase, rmax, ok)
-                : tile2d_f<C, 1, -1, 0, ST>(map, *sr, sdt, tx, ty, smem_raw, phase, rmax, ok);
+      fine = cm ? tile2d_f<C, 1, -1, true, ST>(map, *sr, sdt, tx, ty, smem_raw, phase, rmax, ok)
+                : tile2d_f<C, 1, -1, false, ST>(map, *sr, sdt, tx, ty, smem_raw, phase, rmax, ok);
     else
-      fine = cm ? tile2d_f<C, -1, -1, 1, ST>(map, *sr, sdt, tx, ty, smem_raw, phase, rmax, ok)
-                : tile2d_f<C, -1, -1, 0, ST>(map, *sr, sdt, tx, ty, smem_raw, phase, rmax, ok);
+      fine = cm ? tile2d_f<C, -1, -1, true, ST>(map, *sr, sdt, tx, ty, smem_raw, phase, rmax, ok)
+                : tile2d_f<C, -1, -1, false, ST>(map, *sr, sdt, tx, ty, smem_raw, phase, rmax, ok);
     if (!fine) {
       // A bounded wait gave up (the tile routine has already waited for its
       // copy).  This block leaves the rest of the stage: every run that owns
@@ -124,7 +124,7 @@ using TC1 = T2Cfg<32, 32, 8>;
 using TC2 = T2Cfg<64, 16, 4>;
 using TC3 = T2Cfg<128, 16, 8>;
 using TC4 = T2Cfg<64, 24, 8>;
-using TC5 = T2Cfg<128, 8, 8>;
+using TC5 = T2Cfg<128, 8, 4>;
 constexpr int NCAND = 6;
 static const int CAND_BX[NCAND] = {64, 32, 64, 128, 64, 128};
 static const int CAND_BY[NCAND] = {32, 32, 16, 16, 24, 8};

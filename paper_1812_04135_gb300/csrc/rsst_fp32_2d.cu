@@ -1,21 +1,29 @@
 // Float32 perturbation stage kernel for 2D grids, TMA-staged.
 //
-// One tile = 128 x 8 cells, 128 threads.
+// One tile = 128 x 8 cells, 128 threads, two neighbouring columns a thread.
 //   1. One thread issues a single cp.async.bulk.tensor load of the tile with
 //      its halo for all four fields (box 136 x 12 x 4 of the padded state, the
 //      x origin rounded down to a 16-byte boundary, out-of-range parts zero
-//      filled); the others copy the tile's rows of the row-major background
-//      table (float4).
-//   2. x faces, row by row, lanes along x (conflict-free): each lane's cell
-//      slope gives its face's right state and, by a warp shuffle, the next
-//      face's left state; twice the LLF flux into shared memory.
-//   3. Each thread owns one column of 8 cells and marches up it: one new
-//      half slope and one y-face flux per cell from a register window, then
-//      the cell's divergence (its two x fluxes from shared memory), the
-//      reduced tendency, force, RK combine, store and edge ghosts, and in
-//      stage 2 the CFL rate and physical check, all fused.
+//      filled); the others copy the tile's rows of the background table,
+//      each value twice.
+//   2. x pass, a warp over its own 64 columns by 4 rows: each lane's two cells'
+//      half slopes, the two faces they start (as one pair), and the cells' flux
+//      differences into shared memory (no block barrier before step 3).
+//   3. Each thread owns two columns of 4 cells and marches up them: a new
+//      pair of half slopes and y-face fluxes per row from a register window,
+//      then the cells' divergence, the reduced tendency, force, RK combine,
+//      store and edge ghosts, and in stage 2 the CFL rate and physical check,
+//      all fused.
 // The same tile routine serves the single-run grid and the batched
 // persistent kernel (rsst_batch.cu).
+//
+// What bounds it: instruction issue and its latencies.  Two columns a thread as
+// f32x2 pairs: 434 -> 342 thread instructions a stage-1 cell (ncu), at 58 % of
+// issue instead of 78 % (a pair instruction holds its pipe two cycles, and 126
+// registers leave four CTAs).  us a stage, one column a thread -> here: 2048^2
+// 68.5 -> 64.6, 1000^2 21.2 -> 19.3, and 4096^2 258 -> 244.  Other tiles (2048^2):
+// 64 x 16 66.3, 64 x 8 66.6, 64 x 32 69.6, 8-cell segments 78 to 84; x faces in the
+// march by shuffles 67.8; a fifth CTA spills (89).
 #include "rsst_common.cuh"
 #include "rsst_fp32_2d.cuh"
 #include "rsst_attr.h"
@@ -24,7 +32,7 @@ namespace rsst {
 
 // One launch per stage; FORM, CM (C_max law) and ST (stage) are compile-time.
 template <int VERT, int FORM, int CM, int ST>
-__global__ void __launch_bounds__(T2::NT, 5) stage2d_tma_kernel(const __grid_constant__ CUtensorMap tin,
+__global__ void __launch_bounds__(T2::NT, 4) stage2d_tma_kernel(const __grid_constant__ CUtensorMap tin,
                                                                  const StageArgs<float> a) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   TileRun r;
@@ -58,7 +66,7 @@ __global__ void __launch_bounds__(T2::NT, 5) stage2d_tma_kernel(const __grid_con
   uint32_t phase = 0;
   float rmax = 0.0f;
   bool ok = true;
-  const bool fine = tile2d_f<T2, VERT, FORM, CM, ST>(&tin, r, sdt, blockIdx.x, blockIdx.y, smem_raw, phase, rmax, ok);
+  const bool fine = tile2d_f<T2, VERT, FORM, CM != 0, ST>(&tin, r, sdt, blockIdx.x, blockIdx.y, smem_raw, phase, rmax, ok);
   if (!fine) return;
   if (ST == 2) {
     if (!ok) atomicOr(a.flag, RSST_FLAG_NONPHYSICAL);

@@ -3,58 +3,66 @@
 // The state is U = U0 + U1, U0 = (rho0, 0, 0, E0) a float64 background that
 // varies along y only (or is absent), U1 the stored float32 perturbation.
 // Every term that feeds an update is formed from perturbation-sized
-// quantities (see rsst_math_fp32.cuh for the splitting), with the arithmetic
-// arranged for few instructions per cell:
+// quantities (see rsst_math_fp32.cuh for the splitting).  A lane owns two
+// neighbouring columns and works on them as pairs (rsst_fp32_pair.cuh):
 //  - each cell's MC slope is computed once per axis, as a half slope h
-//    (face states U +- h); along x a lane hands its cell's right face state
-//    to the next lane by a warp shuffle, along y the column march carries it;
+//    (face states U +- h); along x a lane hands its right cell's right face
+//    state to the next lane by a warp shuffle, along y the column march
+//    carries it;
 //  - faces hold twice the LLF flux, 2F = F(qL) + F(qR) - alpha (qR - qL),
 //    and the exact 1/2 folds into 1/dx;
-//  - the background enters through one row-major table row per vertical
-//    index, read as float4 (broadcast: all lanes of a warp share the row).
+//  - the background enters through one table row per vertical index, each
+//    value held twice so that a 16-byte load gives two pair operands.
 #pragma once
 
 #include "rsst_common.cuh"
 #include "rsst_internal.h"
 #include "rsst_fp32_lean.cuh"
+#include "rsst_fp32_pair.cuh"
 #include "rsst_math_fp32.cuh"
 #include "rsst_tma.cuh"
 
 namespace rsst {
 
-// Tile geometry: BX_ x BY_ cells, each thread owning one column of SEG_
-// cells (BX_ * BY_ / SEG_ threads).  Shared memory: the TMA box (halo tile,
-// all fields), the x fluxes, the background rows, a barrier, dt, reduction.
+// Tile geometry: BX_ x BY_ cells, each thread owning two columns of SEG_
+// cells (BX_ * BY_ / (2 SEG_) threads).  Shared memory: the TMA box (halo
+// tile, all fields), the x flux differences, the background rows, a barrier,
+// dt, reduction.
 template <int BX_, int BY_, int SEG_>
 struct T2Cfg {
   static constexpr int NV = 4, BX = BX_, BY = BY_, SEG = SEG_;
-  static constexpr int NT = BX * (BY / SEG);
-  static constexpr int SXP = BX + 8;   // TMA box width: 4 columns each side (2 used), 16-byte aligned origin
+  static constexpr int PX = BX / 2;    // pairs of columns per row
+  static constexpr int NT = PX * (BY / SEG);
+  static constexpr int SXP = BX + 8;   // TMA box width: 4 columns each side (3 used), 16-byte aligned origin
   static constexpr int SYP = BY + 4;   // halo rows
   static constexpr int XO = 4;         // smem column of tile x = 0
-  static constexpr int FXW = BX + 1;   // x faces per row
   static constexpr int U_FLOATS = NV * SYP * SXP;
-  static constexpr int FX_FLOATS = NV * BY * FXW;
-  static constexpr int TAB_FLOATS = TR_W * SYP;
-  static constexpr size_t SCRATCH = (size_t)(U_FLOATS + FX_FLOATS + TAB_FLOATS) * 4;
-  // x-face pass: the slope cells -1 .. BX of every row, in one flat list
-  // walked by warps in chunks of 32 cells that overlap by one
-  // x-face pass: the slope cells -1 .. BX of every row (padded to CW2, an
-  // even count, with two cells beyond BX) form one flat list; a lane takes
-  // two neighbouring cells, a warp chunk 64 cells, chunks start every 62
-  static constexpr int CW2 = BX + 4;
-  static constexpr int NCHUNK2 = (BY * CW2 - 2 + 61) / 62;
+  static constexpr int DX_FLOATS = NV * BY * BX;
+  static constexpr int TR2 = 2 * TR_W;  // floats of a doubled table row
+  static constexpr int TAB_FLOATS = TR2 * SYP;
+  static constexpr size_t SCRATCH = (size_t)(U_FLOATS + DX_FLOATS + TAB_FLOATS) * 4;
+  // A warp owns the cells its lanes march up: WX pairs of columns by WY rows
+  // (64 x SEG cells; 32 x 2 SEG for BX = 32).  Its x pass takes the column
+  // pairs -1 .. WX of those rows as one flat list, 32 at a time, chunks
+  // starting every 30 (the first and the last lane only serve their
+  // neighbours), so no warp waits for another between the passes.
+  static constexpr int WX = PX < 32 ? PX : 32, WY = SEG * (32 / WX);
+  static constexpr int PW = WX + 2;
+  static constexpr int NPAIR = PW * WY;
+  static constexpr int NCHUNK = (NPAIR - 2 + 29) / 30;
   static constexpr uint32_t BOX_BYTES = U_FLOATS * 4;
   static constexpr size_t smem_bytes() { return SCRATCH + 16 + 8 * 8 + 512 + 128; }
   static_assert(BY % SEG == 0, "column segments must tile BY");
-  static_assert(BX % 32 == 0, "a warp of the column march covers 32 columns of one segment");
-  static_assert((U_FLOATS + FX_FLOATS) % 4 == 0, "the table rows start on a 16-byte boundary");
+  static_assert(PX % 32 == 0 || 32 % PX == 0, "a warp's columns");
+  static_assert((U_FLOATS + DX_FLOATS) % 4 == 0, "the table rows start on a 16-byte boundary");
   static_assert(NT % 32 == 0, "whole warps");
   static_assert(SCRATCH % 8 == 0, "the barriers after the scratch area need 8-byte alignment");
   static_assert(SXP <= 256 && SYP <= 256, "TMA box dimensions are at most 256");
 };
 
-using T2 = T2Cfg<128, 8, 8>;  // single-run default
+// Single-run tile: 128 x 8 with two 4-cell segments, so that four CTAs of four
+// warps fit an SM (46.5 KB each).
+using T2 = T2Cfg<128, 8, 4>;
 
 template <class C>
 __device__ __forceinline__ uint64_t* t2_barrier(unsigned char* smem) {
@@ -93,21 +101,20 @@ struct TileRun {
 // (flag set, nothing left in flight).  Accumulates the stage-2 CFL rate
 // maximum and physical check.  The caller initialised the barrier; `phase` is
 // its current parity.  *sdt (shared memory) may be written up to the routine's
-// first barriers: the tile's copy does not wait for dt's float64 division.  FORM, CM and ST fix the form, the C_max law and the
-// stage at compile time (-1, -1, 0: read from the run).
-template <class T2, int VERT, int FORM, int CM, int ST>
+// first barriers: the tile's copy does not wait for dt's float64 division.  FORM (-1: read from the run), the C_max law and the
+// stage are compile-time.
+template <class T2, int VERT, int FORM, bool CM, int ST>
 __device__ __forceinline__ bool tile2d_f(const CUtensorMap* tin, const TileRun& r, const float* sdt, int tx, int ty,
                                          unsigned char* smem, uint32_t& phase, float& rmax, bool& ok_all) {
   constexpr int NV = 4;
   constexpr bool BG = VERT >= 0;
   constexpr int PL = T2::SYP * T2::SXP;  // floats per field in the box
   float* sU = reinterpret_cast<float*>(smem);
-  float* sFx = sU + T2::U_FLOATS;
-  float* st = sFx + T2::FX_FLOATS;  // table rows of padded y j0 .. j0 + SYP - 1
+  float* sDx = sU + T2::U_FLOATS;   // [NV][BY][BX]: twice the x flux above minus below each cell
+  float* st = sDx + T2::DX_FLOATS;  // doubled table rows of padded y j0 .. j0 + SYP - 1
   uint64_t* bar = t2_barrier<T2>(smem);
   const Geom& g = r.g;
   const PhysF& pf = r.pf;
-  const int stage = ST > 0 ? ST : r.stage;
   const int i0 = tx * T2::BX, j0 = ty * T2::BY;
   const int tid = threadIdx.x;
 
@@ -118,13 +125,15 @@ __device__ __forceinline__ bool tile2d_f(const CUtensorMap* tin, const TileRun& 
     tma_load_3d(sU, tin, bar, i0 + g.xoff - T2::XO, j0, 0);
   }
   if constexpr (BG) {
-    // SYP consecutive table rows (16-byte aligned) as float4
-    const float4* src = reinterpret_cast<const float4*>(r.tabr);
+    // SYP consecutive table rows, every value twice
+    const float2* src = reinterpret_cast<const float2*>(r.tabr);
     float4* dst = reinterpret_cast<float4*>(st);
-    constexpr int N4 = T2::TAB_FLOATS / 4;
-    const int first4 = j0 * (TR_W / 4), last4 = r.tab_len * (TR_W / 4);
-    for (int id = tid; id < N4; id += T2::NT)
-      dst[id] = first4 + id < last4 ? src[first4 + id] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    constexpr int N2 = TR_W * T2::SYP / 2;
+    const int first = j0 * (TR_W / 2), last = r.tab_len * (TR_W / 2);
+    for (int id = tid; id < N2; id += T2::NT) {
+      const float2 q = first + id < last ? src[first + id] : make_float2(0.0f, 0.0f);
+      dst[id] = make_float4(q.x, q.x, q.y, q.y);
+    }
   }
   // the give-up decision is taken by the whole block (no thread may leave
   // while others wait at a barrier); a late copy gets one more bounded wait
@@ -154,161 +163,185 @@ __device__ __forceinline__ bool tile2d_f(const CUtensorMap* tin, const TileRun& 
   const float dt = *sdt;
   const int nx = g.n[0], ny = g.n[1];
   const int lane = tid & 31;
-  // ---- x faces.  The slope cells of every row form one flat list; chunk k
-  // holds cells 62k .. 62k + 63, lane l the pair A = 62k + 2l, A + 1 (a pair
-  // never straddles two rows: the rows hold an even number of cells).  The
-  // lane takes both cells' half slopes (four loads and three differences per
-  // field), forms the face between its two cells, and the face on A's left
-  // from its own state A - h_A and the state B + h_B passed one lane up.  So
-  // every face of the tile is formed (the two cells shared by consecutive
-  // chunks give one face twice, with equal values), no slope is recomputed
-  // within a chunk and no lane runs alone; lane 0's left face and faces
-  // across rows are left out.
+  const PhysF2 p2 = make_pf2(pf);
+  // ---- x pass.  Lane l of chunk k holds the column pair A, A + 1 numbered
+  // 30k + l of the flat list.  It takes both cells' half slopes (four loads
+  // and three differences a field), and as one pair the face on A's left
+  // (with the state B + h_B passed one lane up) and the face between its
+  // cells; the face on its right comes from the next lane.  Lanes 1 .. 30
+  // store the two cells' flux differences; faces across rows reach none.
   {
-    const int nwarp = T2::NT / 32;
-    for (int k = tid >> 5; k < T2::NCHUNK2; k += nwarp) {
-      int A = 62 * k + 2 * lane;  // my two cells A, A + 1 (same row: rows hold an even CW2 cells)
-      const bool inb = A < T2::BY * T2::CW2;
-      A = inb ? A : T2::BY * T2::CW2 - 2;  // keeps the loads inside the box
-      const int row = A / T2::CW2;
-      const int ca = A - row * T2::CW2 - 1;  // tile column of A: -1 .. BX + 1
+    const int wc = 2 * ((tid & ~31) % T2::PX), wr = (tid & ~31) / T2::PX * T2::SEG;  // my warp's first column and row
+#pragma unroll 1
+    for (int k = 0; k < T2::NCHUNK; ++k) {
+      int P = 30 * k + lane;
+      const bool inb = P < T2::NPAIR;
+      P = inb ? P : T2::NPAIR - 1;  // keeps the loads inside the box
+      const int row = wr + P / T2::PW;
+      const int j = P % T2::PW;
+      const int ca = wc + 2 * j - 2;  // tile column of A
       const int sr = row + 2;
       const float* ur = sU + sr * T2::SXP + T2::XO + ca;
-      float qRl[NV], qLl[NV], qLi[NV], qRi[NV];
+      f2 qL[NV], qR[NV], G[NV];
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
         const float* uv = ur + v * PL;
-        const float am = uv[-1], a = uv[0], b = uv[1], bp = uv[2];
-        const float d1 = a - am, d2 = b - a, d3 = bp - b;
-        const float ha = half_mc_f(d1, d2), hb = half_mc_f(d2, d3);
-        qRl[v] = a - ha;
-        qLi[v] = a + ha;
-        qRi[v] = b - hb;
-        qLl[v] = __shfl_up_sync(0xffffffffu, b + hb, 1);
+        const float am = uv[-1], bp = uv[2];
+        const float2 ab = *reinterpret_cast<const float2*>(uv);
+        const float d1 = ab.x - am, d2 = ab.y - ab.x, d3 = bp - ab.y;
+        const f2 u = mk2(ab.x, ab.y), h = half_mc2(mk2(d1, d2), mk2(d2, d3));
+        const f2 up = u + h;
+        qR[v] = u - h;
+        qL[v] = mk2(__shfl_up_sync(0xffffffffu, hi2(up), 1), lo2(up));
       }
-      float4 cb = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-      if constexpr (BG) cb = *reinterpret_cast<const float4*>(st + sr * TR_W + TR_RHO0);
-      const bool rowok = inb && j0 + row < ny;
-      float G[NV];
-      face_flat_cm<NV, 0, BG, CM>(qLi, qRi, cb, pf, G);  // face between A and A + 1: face index ca + 1
-      if (rowok && ca + 1 <= T2::BX && i0 + ca + 1 <= nx) {
+      face_flat2<NV, 0, BG, CM>(qL, qR, st + sr * T2::TR2, p2, G);
+      const bool put = inb && lane >= 1 && lane <= 30 && j >= 1 && j <= T2::WX;
+      float* dx = sDx + row * T2::BX + ca;
 #pragma unroll
-        for (int v = 0; v < NV; ++v) sFx[(v * T2::BY + row) * T2::FXW + ca + 1] = G[v];
-      }
-      face_flat_cm<NV, 0, BG, CM>(qLl, qRl, cb, pf, G);  // face between A - 1 and A: face index ca
-      if (rowok && lane > 0 && ca >= 0 && ca <= T2::BX && i0 + ca <= nx) {
-#pragma unroll
-        for (int v = 0; v < NV; ++v) sFx[(v * T2::BY + row) * T2::FXW + ca] = G[v];
+      for (int v = 0; v < NV; ++v) {
+        const float f0 = lo2(G[v]), f1 = hi2(G[v]), fr = __shfl_down_sync(0xffffffffu, f0, 1);
+        if (put) *reinterpret_cast<float2*>(dx + v * T2::BY * T2::BX) = make_float2(f1 - f0, fr - f1);
       }
     }
   }
-  __syncthreads();
+  __syncwarp();
 
-  // ---- column march with the fused epilogue: each thread owns tile column
-  // col, rows jb .. jb + SEG - 1; a register window carries the cell states,
-  // the y half slope and the lower face's flux.
-  const int col = tid % T2::BX;
-  const int jb = (tid / T2::BX) * T2::SEG;
+  // ---- column march with the fused epilogue: each thread owns tile columns
+  // col, col + 1, rows jb .. jb + SEG - 1; a register window carries the cell
+  // states, the y half slope and the lower face's flux.
+  const int col = 2 * (tid % T2::PX);
+  const int jb = (tid / T2::PX) * T2::SEG;
   const int x = i0 + col;
   if (x < nx && j0 + jb < ny) {
+    const bool two = x + 1 < nx;  // an odd grid's last column stands alone
     const float* uc = sU + T2::XO + col;
-    auto ld = [&](int srow, float (&u)[NV]) {
+    auto ld = [&](int srow, f2 (&u)[NV]) {
 #pragma unroll
-      for (int v = 0; v < NV; ++v) u[v] = uc[v * PL + srow * T2::SXP];
+      for (int v = 0; v < NV; ++v)
+        u[v].v = *reinterpret_cast<const unsigned long long*>(uc + v * PL + srow * T2::SXP);
     };
-    float u0[NV], u1[NV], h0[NV], Fm[NV];
+    f2 u0[NV], u1[NV], h0[NV], Fm[NV];
     {
-      float umm[NV], um[NV], hm[NV];
+      f2 umm[NV], um[NV], hm[NV], da[NV], db[NV], dc[NV];
       // cells jb-2 .. jb+1 live at smem rows jb .. jb+3
       ld(jb, umm);
       ld(jb + 1, um);
       ld(jb + 2, u0);
       ld(jb + 3, u1);
-      vslope_f<NV, BG>(umm, um, u0, st + (jb + 1) * TR_W, hm);  // cell jb-1
-      vslope_f<NV, BG>(um, u0, u1, st + (jb + 2) * TR_W, h0);   // cell jb
-      float qL[NV], qR[NV];
+#pragma unroll
+      for (int v = 0; v < NV; ++v) {
+        da[v] = um[v] - umm[v];
+        db[v] = u0[v] - um[v];
+        dc[v] = u1[v] - u0[v];
+      }
+      vslope2<NV, BG>(da, db, st + (jb + 1) * T2::TR2, hm);  // cell jb-1
+      vslope2<NV, BG>(db, dc, st + (jb + 2) * T2::TR2, h0);  // cell jb
+      f2 qL[NV], qR[NV];
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
         qL[v] = um[v] + hm[v];
         qR[v] = u0[v] - h0[v];
       }
-      face_vert_cm<NV, 1, BG, CM>(qL, qR, st + (jb + 2) * TR_W, pf, Fm);
+      face_vert2<NV, 1, BG, CM>(qL, qR, st + (jb + 2) * T2::TR2, p2, Fm);
     }
-    const float idx = 0.5f * pf.inv_dx[0], idy = 0.5f * pf.inv_dx[1];  // the faces hold 2F
+    const f2 nidx = dup2(-0.5f * pf.inv_dx[0]), nidy = dup2(-0.5f * pf.inv_dx[1]);  // the faces hold 2F
+    const f2 dt2 = dup2(dt);
     const int64_t fs = g.fstride;
-    const bool xghost = x < RSST_G || x >= nx - RSST_G;
+    const bool xghost = x < RSST_G || x + 1 >= nx - RSST_G;
     const int64_t o0 = pidx(g, x, j0 + jb, 0);
-    // stage 2: U^n of the next row's cell is loaded one row ahead, so its
+    // stage 2: U^n of the next row's cells is loaded one row ahead, so its
     // global-memory latency overlaps a row of arithmetic
-    float bnext[NV] = {0.0f, 0.0f, 0.0f, 0.0f};
-    if (stage == 2) {
+    f2 bnext[NV] = {};
+    if constexpr (ST == 2) {
 #pragma unroll
-      for (int v = 0; v < NV; ++v) bnext[v] = r.base[v * fs + o0];
+      for (int v = 0; v < NV; ++v) bnext[v].v = *reinterpret_cast<const unsigned long long*>(r.base + v * fs + o0);
     }
 #pragma unroll 1
     for (int jj = 0; jj < T2::SEG; ++jj) {
-      const int j = jb + jj;  // tile row of the cell
+      const int j = jb + jj;  // tile row of the cells
       if (j0 + j >= ny) break;
-      float bv[NV];
+      f2 bv[NV];
 #pragma unroll
       for (int v = 0; v < NV; ++v) bv[v] = bnext[v];
-      if (stage == 2 && jj + 1 < T2::SEG && j0 + j + 1 < ny) {
+      if (ST == 2 && jj + 1 < T2::SEG && j0 + j + 1 < ny) {
         const int64_t on = o0 + (int64_t)(jj + 1) * g.pitch;
 #pragma unroll
-        for (int v = 0; v < NV; ++v) bnext[v] = r.base[v * fs + on];
+        for (int v = 0; v < NV; ++v) bnext[v].v = *reinterpret_cast<const unsigned long long*>(r.base + v * fs + on);
       }
-      const int sr = j + 2;  // its smem row
-      float u2[NV], h1[NV], Fp[NV];
-      ld(j + 4, u2);                                          // cell j+2
-      vslope_f<NV, BG>(u0, u1, u2, st + (j + 3) * TR_W, h1);  // cell j+1
+      const int sr = j + 2;  // their smem row
+      f2 u2[NV], h1[NV], Fp[NV];
+      ld(j + 4, u2);  // cells j+2
       {
-        float qL[NV], qR[NV];
+        f2 da[NV], db[NV];
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+          da[v] = u1[v] - u0[v];
+          db[v] = u2[v] - u1[v];
+        }
+        vslope2<NV, BG>(da, db, st + (j + 3) * T2::TR2, h1);  // cells j+1
+      }
+      {
+        f2 qL[NV], qR[NV];
 #pragma unroll
         for (int v = 0; v < NV; ++v) {
           qL[v] = u0[v] + h0[v];
           qR[v] = u1[v] - h1[v];
         }
-        face_vert_cm<NV, 1, BG, CM>(qL, qR, st + (j + 3) * TR_W, pf, Fp);
+        face_vert2<NV, 1, BG, CM>(qL, qR, st + (j + 3) * T2::TR2, p2, Fp);
       }
-      float L[NV], Dl[NV];
+      f2 L[NV], Dl[NV];
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
-        const float* fr = sFx + (v * T2::BY + j) * T2::FXW + col;
-        L[v] = fmaf(-(Fp[v] - Fm[v]), idy, -(fr[1] - fr[0]) * idx);
+        f2 dx;
+        dx.v = *reinterpret_cast<const unsigned long long*>(sDx + (v * T2::BY + j) * T2::BX + col);
+        L[v] = fma2(Fp[v] - Fm[v], nidy, dx * nidx);
       }
-      float rho0 = 0.0f, P0 = 0.0f;
+      f2 rho0 = {}, P0 = {};
       if constexpr (BG) {
-        const float* tr = st + sr * TR_W;
-        const float4 cb = *reinterpret_cast<const float4*>(tr + TR_RHO0);
-        const float4 r0 = *reinterpret_cast<const float4*>(tr + TR_R0);
-        const float4 d0 = *reinterpret_cast<const float4*>(tr + TR_R0 + 4);  // R0[4] (unused in 2D), D0 rho, mv, E
-        rho0 = cb.x;
-        P0 = cb.y;
-        Dl[0] = L[0] + d0.y;
+        const float* tr = st + sr * T2::TR2;
+        const f2x2 cb = tab2(tr, TR_RHO0), r01 = tab2(tr, TR_R0), r23 = tab2(tr, TR_R0 + 2);
+        const f2x2 x0 = tab2(tr, TR_R0 + 4), x1 = tab2(tr, TR_R0 + 6);  // R0[4] (unused in 2D), D0 rho; mv, E
+        rho0 = cb.a;
+        P0 = cb.b;
+        Dl[0] = L[0] + x0.b;
         Dl[1] = L[1];
-        Dl[2] = L[2] + d0.z;
-        Dl[3] = L[3] + d0.w;
-        L[0] += r0.x;
-        L[1] += r0.y;
-        L[2] += r0.z;
-        L[3] += r0.w;
+        Dl[2] = L[2] + x1.a;
+        Dl[3] = L[3] + x1.b;
+        L[0] = L[0] + r01.a;
+        L[1] = L[1] + r01.b;
+        L[2] = L[2] + r23.a;
+        L[3] = L[3] + r23.b;
       } else {
 #pragma unroll
         for (int v = 0; v < NV; ++v) Dl[v] = L[v];
       }
       const int y = j0 + j;
       const int64_t o = o0 + (int64_t)jj * g.pitch;
-      float u[NV], rate;
-      bool ok;
-      cell_lean<NV, FORM, CM, ST>(u0, L, Dl, rho0, P0, pf, r.p.variant, r.p.has_grav != 0, stage, dt, bv, u, rate,
-                                  ok);
-      if (stage == 2) {
-        rmax = fmaxf(rmax, rate);
-        ok_all = ok_all && ok;
+      f2 u[NV], rate;
+      bool ok[2];
+      cell_lean2<NV, FORM, CM, ST>(u0, L, Dl, rho0, P0, pf, p2, r.p.variant, r.p.has_grav != 0, dt2, bv, u, rate, ok);
+      if constexpr (ST == 2) {
+        rmax = ok[0] ? fmaxf(rmax, lo2(rate)) : rmax;
+        rmax = two && ok[1] ? fmaxf(rmax, hi2(rate)) : rmax;
+        ok_all = ok_all && ok[0] && (ok[1] || !two);
       }
+      if (two) {
 #pragma unroll
-      for (int v = 0; v < NV; ++v) r.out[v * fs + o] = u[v];
-      if (xghost || y < RSST_G || y >= ny - RSST_G) store_mirror_ghosts<float, 4>(r.out, g, r.p, x, y, 0, u);
+        for (int v = 0; v < NV; ++v) *reinterpret_cast<unsigned long long*>(r.out + v * fs + o) = u[v].v;
+      } else {
+#pragma unroll
+        for (int v = 0; v < NV; ++v) r.out[v * fs + o] = lo2(u[v]);
+      }
+      if (xghost || y < RSST_G || y >= ny - RSST_G) {
+        float ua[NV], ub[NV];
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+          ua[v] = lo2(u[v]);
+          ub[v] = hi2(u[v]);
+        }
+        store_mirror_ghosts<float, 4>(r.out, g, r.p, x, y, 0, ua);
+        if (two) store_mirror_ghosts<float, 4>(r.out, g, r.p, x + 1, y, 0, ub);
+      }
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
         u0[v] = u1[v];
