@@ -287,6 +287,39 @@ __device__ __forceinline__ double rsqrt_nr(double w) {
   return fma(y * e, fma(0.375, e, 0.5), y);
 }
 
+// A float pair s + c with |c| within some ulps of s as a double, on the float32
+// and integer pipes.
+__device__ __forceinline__ double sum_to_double(float s, float c) {
+  const float h = s + c;
+  return pair_to_double(h, c - (h - s));
+}
+
+// c_tot under the C_max law from |V|^2 and (a/xi)^2, with three float64
+// instructions: the roots as float pairs (2^-42), one float64 Newton step on the
+// sound term, which carries c_tot in slow flow (a float pair's accuracy showed
+// there against a 64-bit evaluation).  Zero, NaN and values beyond a float's
+// range come as sqrt_pair gives them.
+__device__ __forceinline__ double ctot_cmax(double v2, double a2x) {
+  float s, c;
+  sqrt_pair(a2x, s, c);
+  const double y = sum_to_double(s, c);
+  const double a = s > 0.0f && s < __int_as_float(0x7f800000) ? fma(fma(-y, y, a2x), f2d_bits(__fdividef(0.5f, s)), y) : y;
+  sqrt_pair(v2, s, c);
+  return sum_to_double(s, c) + a;
+}
+
+// A non-negative double as a float pair (2^-48), on the float32 and integer
+// pipes; subnormal floats come as 0, NaN and negative values as NaN.
+__device__ __forceinline__ void to_pair(double x, float& h, float& l) {
+  int be;
+  split_pair(x, h, l, be);
+  const int k = be - 1023;
+  const float sc = k < -126 ? 0.0f : (k > 127 ? __int_as_float(0x7f800000) : __int_as_float((127 + k) << 23));
+  const bool fin = (unsigned)(be - 1) < 2046u;
+  h = fin ? h * sc : (be == 0 ? 0.0f : __int_as_float(0x7fc00000));
+  l = fin ? l * sc : 0.0f;
+}
+
 // Effective sound speed a/xi from a^2 and the factor f = 1 - 1/xi^2: constant
 // xi, or the C_max law xi = [1 + (a/C_max)^4]^(1/4) (Eq. cx, Sec. 4.3), for
 // which a/xi = sqrt(a^2 / sqrt(w)) and f = 1 - 1/sqrt(w), w = 1 + a^4/C_max^4.
@@ -305,7 +338,7 @@ template <bool CV>
 __device__ __forceinline__ void ctot_of(const Phys& p, double rho, double k, double P, double ir, float& h, float& l) {
   if (p.use_cmax) {
     const double a2 = Eos<CV>::sound2(p, rho, P, ir);
-    ctot_pair(k * ir, a2 * rsqrt_nr(fma(a2 * a2, p.inv_cmax4, 1.0)), h, l);
+    to_pair(ctot_cmax(k * ir, a2 * rsqrt_nr(fma(a2 * a2, p.inv_cmax4, 1.0))), h, l);
   } else if constexpr (CV) {
     ctot_pair(k * ir, Eos<CV>::sound2_over_xi2(p, rho, P, ir), h, l);
   } else {
@@ -487,7 +520,8 @@ __device__ __forceinline__ bool positive_finite(double x) {
 }
 
 // CFL rate sum_d c_tot/dx_d of a cell and its physical-state check.  c_tot is
-// the float pair of the LLF speed; the checks read bit patterns.
+// the float pair of the LLF speed (C_max law: in float64); the
+// checks read bit patterns.
 template <int NV, bool CV = false>
 __device__ __forceinline__ double cfl_rate(const double (&q)[NV], const Phys& p, bool& ok) {
   constexpr int ND = NV - 2;
@@ -502,6 +536,10 @@ __device__ __forceinline__ double cfl_rate(const double (&q)[NV], const Phys& p,
   }
   const double P = Eos<CV>::pressure(p, rho, q[NV - 1], k);
   ok = fin && positive_finite(rho) && positive_finite(P) && Eos<CV>::admissible(p, rho);
+  if (p.use_cmax) {
+    const double a2 = Eos<CV>::sound2(p, rho, P, ir);
+    return ctot_cmax(k * ir, a2 * rsqrt_nr(fma(a2 * a2, p.inv_cmax4, 1.0))) * p.sum_inv_dx;
+  }
   float ch, cl;
   ctot_of<CV>(p, rho, k, P, ir, ch, cl);
   return pair_to_double(ch, cl) * p.sum_inv_dx;
