@@ -374,6 +374,31 @@ int64_t rsst_kernel_launches(const rsst_handle* h);
  * Synchronous, current device. */
 int rsst_math_selftest(int32_t n, double* rcp_max_ulp, int32_t* mc_mismatches, double* sqrt_max_rel);
 
+/* Test entry (no counterpart in the paper): one of the device helpers of the
+ * step evaluated at n points.  `in` holds the helper's arguments as rows of n
+ * values, `out` gets n values (host pointers; float32 helpers round their
+ * arguments).  RSST_EINVAL for an unknown helper, a NULL pointer or n outside
+ * 1..2^26.  Synchronous, current device. */
+typedef enum {
+  RSST_EVAL_RCP = 0,          /* x: 1/x of the float64 step */
+  RSST_EVAL_SQRT_PAIR,        /* x: sqrt(x) as a float pair, its sum */
+  RSST_EVAL_CTOT,             /* rho |V|^2, P, 1/rho: the LLF speed's pair at gamma/xi^2 = RSST_EVAL_GAMMA_XI2 */
+  RSST_EVAL_CTOT_CMAX,        /* |V|^2, (a/xi)^2: c_tot under the C_max law */
+  RSST_EVAL_RSQRT,            /* x: 1/sqrt(x) of the C_max law */
+  RSST_EVAL_PAIR_TO_DOUBLE,   /* h, l of a normalised float pair */
+  RSST_EVAL_SPEED,            /* x: sqrt(x) of the adjoint's wave speeds */
+  RSST_EVAL_INV_SPEED,        /* x: its reciprocal */
+  RSST_EVAL_MC_SLOPE,         /* a, b: MC limited slope */
+  RSST_EVAL_HALF_MC,          /* a, b: half of it, as the adjoint forms it */
+  RSST_EVAL_DF_FLUX,          /* double-float, gas at rest, gamma - 1 = gamma/xi^2 = 1: rho left, rho right, E: twice
+                               * the mass flux */
+  RSST_EVAL_PAIR_TENDENCY,    /* float32 pairs: rho, m_x, m_y and the tendencies of rho, m_x, m_y, E: dP/(gamma - 1) */
+  RSST_EVAL_PAIR_DC           /* float32 pairs, gas at rest, gamma - 1 = gamma/xi^2 = 1: rho1, E1, rho0, P0:
+                               * c_tot - c_tot0 */
+} rsst_eval_fn;
+#define RSST_EVAL_GAMMA_XI2 (5.0 / 3.0 / 900.0)
+int rsst_math_eval(int32_t fn, int64_t n, const double* in, double* out);
+
 /* Float64 FMA throughput of the current device in TFLOP/s, measured by a
  * probe kernel (independent FMA chains on every SM, timed with CUDA events
  * after a warm-up launch; `iters` x 32 FMAs per thread), and the launch time

@@ -40,20 +40,6 @@
 
 namespace rsst {
 
-// Half the MC slope (Sec. 4.2) and the branch taken: 0 -> 0, 1 -> a, 2 -> b,
-// 3 -> (a+b)/4; decisions and values on the integer pipe as in mc_slope.
-__device__ __forceinline__ double half_mc(double a, double b, int& br) {
-  const long long two = 2ll << 52;             // x4 in the exponent field
-  const unsigned long long four = 1ull << 54;  // x4 in the shifted exponent field
-  const long long ia = __double_as_longlong(a), ib = __double_as_longlong(b);
-  const unsigned long long ua = (unsigned long long)ia << 1, ub = (unsigned long long)ib << 1;
-  const long long is = __double_as_longlong(a + b);
-  const unsigned long long us = (unsigned long long)is << 1;
-  const bool same = ((ia ^ ib) >= 0) && ua != 0 && ub != 0;
-  const bool pa = ua <= ub && ua + four <= us, pb = ub + four <= us;
-  br = !same ? 0 : (pa ? 1 : (pb ? 2 : 3));
-  return same ? __longlong_as_double(pa ? ia : (pb ? ib : is - two)) : 0.0;
-}
 // d(half slope)/da and /db of the taken branch, times the half slope's adjoint ds.
 __device__ __forceinline__ void mc_reverse(int br, double ds, double& da, double& db) {
   const double q = half_of(half_of(ds));
@@ -64,13 +50,6 @@ __device__ __forceinline__ void mc_reverse(int br, double ds, double& da, double
 // a/xi under the C_max law (Eq. cx).
 __device__ __forceinline__ double sound_cmax(double a2, const Phys& p) {
   return sqrt(a2 * rcp_nr(sqrt(1.0 + (a2 * a2) * p.inv_cmax4)));
-}
-
-// 1/x of a positive float pair as a double (relative error below 2^-43).
-__device__ __forceinline__ double rcp_of_pair(float h, float l) {
-  float r;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(h));
-  return pair_to_double(r, r * fmaf(-l, r, fmaf(-h, r, 1.0f)));
 }
 
 // The forward values of one face state that the reverse of its flux reuses.
@@ -164,15 +143,12 @@ __device__ __forceinline__ double face_vjp(const double (&s)[4][NV], const doubl
     ctot_pair_of(wL.k, wL.P, wL.ir, p, hL, lL);
     ctot_pair_of(wR.k, wR.P, wR.ir, p, hR, lR);
     left = hL > hR || (hL == hR && lL >= lR);
-    float h, l;
     const double ir = left ? wL.ir : wR.ir, k = left ? wL.k : wR.k, P = left ? wL.P : wR.P;
     alpha = pair_to_double(left ? hL : hR, left ? lL : lR);
-    sqrt_pair(k * ir, h, l);  // |V|
-    sv = h > 0.0f ? pair_to_double(h, l) : 0.0;
-    iv = h > 0.0f ? rcp_of_pair(h, l) : 0.0;
+    sqrt_rcp(k * ir, sv, iv);  // |V|
     const double gir = p.gamma_xi2 * ir;
-    sqrt_pair(gir * P, h, l);  // a/xi
-    const double ca = pair_to_double(h, l), ica = h > 0.0f ? rcp_of_pair(h, l) : 0.0;
+    double ca, ica;
+    sqrt_rcp(gir * P, ca, ica);  // a/xi
     const double dh = half_of(dalpha);
     cP = dh * (gir * ica);
     cr = dh * (ca * ir);

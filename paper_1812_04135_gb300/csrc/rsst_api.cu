@@ -217,6 +217,14 @@ static void make_physf(const Phys* p, PhysF* f) {
   f->gx = (float)(p->use_cmax ? p->gamma : p->gamma_xi2);
 }
 
+void rsst_split_gamma_xi2(Phys* p) {
+  int e;
+  const double m = 2.0 * std::frexp(p->gamma_xi2, &e);  // in [1, 2)
+  p->gxh = (float)m;
+  p->gxl = (float)(m - (double)p->gxh);
+  p->gxe = e - 1;
+}
+
 static void make_phys(const rsst_config* c, Phys* p) {
   memset(p, 0, sizeof *p);
   p->gamma = c->gamma;
@@ -227,13 +235,7 @@ static void make_phys(const rsst_config* c, Phys* p) {
   p->inv_xi = 1.0 / c->xi;
   p->f = 1.0 - 1.0 / (c->xi * c->xi);
   p->gamma_xi2 = c->gamma / (c->xi * c->xi);
-  {
-    int e;
-    const double m = 2.0 * std::frexp(p->gamma_xi2, &e);  // in [1, 2)
-    p->gxh = (float)m;
-    p->gxl = (float)(m - (double)p->gxh);
-    p->gxe = e - 1;
-  }
+  rsst_split_gamma_xi2(p);
   p->gam_gm1 = c->gamma / p->gm1;
   p->f_gm1 = p->f * p->gm1;
   p->use_cmax = c->cmax > 0.0;

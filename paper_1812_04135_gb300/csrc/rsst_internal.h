@@ -172,6 +172,11 @@ int rsst_launch_unpack_fp32(const float* src, double* dst, const Geom& g, const 
 int rsst_launch_sums_fp32(const float* U, const Geom& g, const Phys& p, const double* bg, int bg_len,
                           double* partial, double* out, double scale, cudaStream_t s);
 
+// gxh, gxl, gxe from gamma_xi2.
+void rsst_split_gamma_xi2(Phys* p);
+// Float32-pipe helpers of rsst_math_eval (device buffers, default stream).
+void rsst_launch_eval_fp32(int fn, int64_t n, const double* in, double* out);
+
 void rsst_set_error(const char* fmt, ...);
 
 // One run: configuration, padded state buffers, background, scalars.

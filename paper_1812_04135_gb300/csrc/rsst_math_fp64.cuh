@@ -320,6 +320,22 @@ __device__ __forceinline__ void to_pair(double x, float& h, float& l) {
   l = fin ? l * sc : 0.0f;
 }
 
+// 1/x of a positive float pair as a double (relative error below 2^-43).
+__device__ __forceinline__ double rcp_of_pair(float h, float l) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(h));
+  return pair_to_double(r, r * fmaf(-l, r, fmaf(-h, r, 1.0f)));
+}
+
+// sqrt(x) and its reciprocal as doubles on the float32 and integer pipes (for the
+// adjoint's derivatives of c_tot); both 0 at x = 0.
+__device__ __forceinline__ void sqrt_rcp(double x, double& s, double& r) {
+  float h, l;
+  sqrt_pair(x, h, l);
+  s = h == 0.0f ? 0.0 : pair_to_double(h, l);
+  r = h > 0.0f ? rcp_of_pair(h, l) : 0.0;
+}
+
 // Effective sound speed a/xi from a^2 and the factor f = 1 - 1/xi^2: constant
 // xi, or the C_max law xi = [1 + (a/C_max)^4]^(1/4) (Eq. cx, Sec. 4.3), for
 // which a/xi = sqrt(a^2 / sqrt(w)) and f = 1 - 1/sqrt(w), w = 1 + a^4/C_max^4.
@@ -408,6 +424,20 @@ __device__ __forceinline__ double mc_slope(double a, double b) {
   return same ? __longlong_as_double(pick) : 0.0;
 }
 
+// Half the MC slope (Sec. 4.2) and the branch taken: 0 -> 0, 1 -> a, 2 -> b,
+// 3 -> (a+b)/4; decisions and values on the integer pipe as in mc_slope.
+__device__ __forceinline__ double half_mc(double a, double b, int& br) {
+  const long long two = 2ll << 52;             // x4 in the exponent field
+  const unsigned long long four = 1ull << 54;  // x4 in the shifted exponent field
+  const long long ia = __double_as_longlong(a), ib = __double_as_longlong(b);
+  const unsigned long long ua = (unsigned long long)ia << 1, ub = (unsigned long long)ib << 1;
+  const long long is = __double_as_longlong(a + b);
+  const unsigned long long us = (unsigned long long)is << 1;
+  const bool same = ((ia ^ ib) >= 0) && ua != 0 && ub != 0;
+  const bool pa = ua <= ub && ua + four <= us, pb = ub + four <= us;
+  br = !same ? 0 : (pa ? 1 : (pb ? 2 : 3));
+  return same ? __longlong_as_double(pa ? ia : (pb ? ib : is - two)) : 0.0;
+}
 // Reduced tendency: dU <- dU - (1 - 1/xi^2) s r, then the external force.
 //   PVS: s = dP,   r = (1/a^2, V/a^2, (e+P+rho V^2/2)/(rho a^2))   Sec. 3.2, Eqs. pvs_dt, pvs_cons_rhs
 //   DVS: s = drho, r = (1, V, (e+P+rho V^2/2)/rho)                  App. A.1

@@ -3,7 +3,8 @@
 // correctly rounded division (largest error in ulps), the integer-pipe MC
 // limiter against the direct float64 form of the same definition, and the
 // c_tot square root against CUDA's sqrt (largest relative error, plus its
-// zero, subnormal and negative cases).
+// zero, subnormal and negative cases).  rsst_math_eval evaluates single helpers
+// on the caller's values, for tests that choose them.
 #include <cmath>
 #include <cstring>
 
@@ -74,6 +75,39 @@ __global__ void selftest_kernel(int n, unsigned long long* max_ulp, unsigned int
   }
 }
 
+__global__ void eval_kernel(int fn, int64_t n, const double* __restrict__ in, double* __restrict__ out, const Phys p) {
+  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const double x = in[i], y = in[n + i], z = in[2 * n + i];  // (the buffer holds at least three rows)
+  float h, l;
+  double s, r;
+  int br;
+  switch (fn) {
+    case RSST_EVAL_RCP: out[i] = rcp_nr(x); break;
+    case RSST_EVAL_SQRT_PAIR:
+      sqrt_pair(x, h, l);
+      out[i] = (double)h + (double)l;
+      break;
+    case RSST_EVAL_CTOT:
+      ctot_pair_of(x, y, z, p, h, l);
+      out[i] = (double)h + (double)l;
+      break;
+    case RSST_EVAL_CTOT_CMAX: out[i] = ctot_cmax(x, y); break;
+    case RSST_EVAL_RSQRT: out[i] = rsqrt_nr(x); break;
+    case RSST_EVAL_PAIR_TO_DOUBLE: out[i] = pair_to_double((float)x, (float)y); break;
+    case RSST_EVAL_SPEED:
+      sqrt_rcp(x, s, r);
+      out[i] = s;
+      break;
+    case RSST_EVAL_INV_SPEED:
+      sqrt_rcp(x, s, r);
+      out[i] = r;
+      break;
+    case RSST_EVAL_MC_SLOPE: out[i] = mc_slope(x, y); break;
+    default: out[i] = half_mc(x, y, br); break;
+  }
+}
+
 }  // namespace rsst
 
 extern "C" int rsst_math_selftest(int32_t n, double* rcp_max_ulp, int32_t* mc_mismatches, double* sqrt_max_rel) {
@@ -111,5 +145,38 @@ extern "C" int rsst_math_selftest(int32_t n, double* rcp_max_ulp, int32_t* mc_mi
   double rel;
   memcpy(&rel, &ulp[1], sizeof rel);
   *sqrt_max_rel = rel;
+  return RSST_OK;
+}
+
+extern "C" int rsst_math_eval(int32_t fn, int64_t n, const double* in, double* out) {
+  // rows of input per function, in the order of the enumeration
+  static const int rows[] = {1, 1, 3, 2, 1, 2, 1, 1, 2, 2, 3, 7, 4};
+  if (fn < 0 || fn >= (int)(sizeof rows / sizeof rows[0]) || n < 1 || n > (int64_t)1 << 26 || !in || !out) {
+    rsst_set_error("rsst_math_eval: unknown function, n outside 1..2^26 or a NULL pointer");
+    return RSST_EINVAL;
+  }
+  const int held = rows[fn] > 3 ? rows[fn] : 3;
+  double* d = nullptr;
+  if (cudaMalloc((void**)&d, (size_t)(held + 1) * n * sizeof(double)) != cudaSuccess) {
+    cudaGetLastError();
+    rsst_set_error("rsst_math_eval: allocation failed");
+    return RSST_ENOMEM;
+  }
+  Phys p = {};
+  p.gamma_xi2 = RSST_EVAL_GAMMA_XI2;
+  rsst_split_gamma_xi2(&p);
+  cudaError_t e = cudaMemset(d, 0, (size_t)held * n * sizeof(double));
+  if (e == cudaSuccess) e = cudaMemcpy(d, in, (size_t)rows[fn] * n * sizeof(double), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) {
+    if (fn >= RSST_EVAL_DF_FLUX) rsst_launch_eval_fp32(fn, n, d, d + held * n);
+    else rsst::eval_kernel<<<(unsigned)((n + 255) / 256), 256>>>(fn, n, d, d + held * n, p);
+    e = cudaGetLastError();
+  }
+  if (e == cudaSuccess) e = cudaMemcpy(out, d + held * n, (size_t)n * sizeof(double), cudaMemcpyDeviceToHost);
+  cudaFree(d);
+  if (e != cudaSuccess) {
+    rsst_set_error("rsst_math_eval: %s", cudaGetErrorString(e));
+    return RSST_ECUDA;
+  }
   return RSST_OK;
 }

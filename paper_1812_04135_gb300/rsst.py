@@ -68,6 +68,7 @@ def lib():
             "rsst_conserved_sums_noalloc": (i32, [vp, i32, C.POINTER(C.c_int32), pd, vp, vp]),
             "rsst_config_size": (C.c_size_t, []),
             "rsst_math_selftest": (i32, [i32, pd, C.POINTER(C.c_int32), pd]),
+            "rsst_math_eval": (i32, [i32, i64, pd, pd]),
             "rsst_fp64_fma_peak": (i32, [i32, pd, pd]),
             "rsst_adjoint_record": (i32, [vp, dbl, i32, i32]),
             "rsst_adjoint_segments": (i32, [vp, C.POINTER(C.c_int32)]),
@@ -282,6 +283,19 @@ def rsst_math_selftest(n: int = 1 << 20):
     rel = C.c_double()
     _check(lib().rsst_math_selftest(int(n), C.byref(ulp), C.byref(bad), C.byref(rel)), "rsst_math_selftest")
     return ulp.value, bad.value, rel.value
+
+
+EVAL_FNS = ("rcp", "sqrt_pair", "ctot", "ctot_cmax", "rsqrt", "pair_to_double", "speed", "inv_speed", "mc_slope",
+            "half_mc", "df_flux", "pair_tendency", "pair_dc")
+
+
+def rsst_math_eval(fn: str, *args) -> np.ndarray:
+    """One device helper (a name of EVAL_FNS) at arrays of arguments; rsst.h lists each one's arguments."""
+    a = np.ascontiguousarray(np.stack(np.broadcast_arrays(*[np.asarray(x, dtype=np.float64) for x in args])))
+    out = np.empty(a.shape[1])
+    pd = C.POINTER(C.c_double)
+    _check(lib().rsst_math_eval(EVAL_FNS.index(fn), a.shape[1], a.ctypes.data_as(pd), out.ctypes.data_as(pd)), "rsst_math_eval")
+    return out
 
 
 def rsst_fp64_fma_peak(iters: int = 20000):

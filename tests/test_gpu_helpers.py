@@ -1,0 +1,43 @@
+"""Single device helpers (rsst_math_eval) at the values where their bit
+arithmetic is tight, against numpy in float64."""
+import numpy as np
+import pytest
+
+from paper_1812_04135_gb300 import rsst
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    import os
+    if not os.path.exists(rsst.LIB_PATH):
+        import __graft_entry__
+        __graft_entry__.build()
+    rsst.lib()
+
+
+def significands(low, exponent=0):
+    """Every leading 24-bit significand with the given 29 low bits, times 2^exponent."""
+    return np.ldexp(1.0 + (np.arange(1 << 23) * 2.0 ** 29 + low) * 2.0 ** -52, exponent)
+
+
+LOWS = [0, 1, (1 << 28) - 1, 1 << 28, (1 << 29) - 1]
+
+
+@pytest.mark.parametrize("low", LOWS)
+@pytest.mark.parametrize("exponent", [0, -700])
+def test_reciprocal_at_every_leading_significand(low, exponent):
+    x = significands(low, exponent)
+    got, want = rsst.rsst_math_eval("rcp", x), 1.0 / x
+    assert np.abs(got.view(np.int64) - want.view(np.int64)).max() <= 1
+
+
+@pytest.mark.parametrize("low", LOWS)
+@pytest.mark.parametrize("exponent", [0, 1, -2])
+def test_adjoint_speeds_at_every_leading_significand(low, exponent):
+    x = significands(low, exponent)
+    s = np.sqrt(x)
+    # the root's pair 2^-42; its reciprocal's seed error 2^-22 squared and its roundings 2^-45 on top
+    assert np.abs(rsst.rsst_math_eval("speed", x) / s - 1.0).max() <= 2.0 ** -42
+    assert np.abs(rsst.rsst_math_eval("inv_speed", x) * s - 1.0).max() <= 2.0 ** -41
