@@ -374,11 +374,7 @@ int64_t rsst_kernel_launches(const rsst_handle* h);
  * Synchronous, current device. */
 int rsst_math_selftest(int32_t n, double* rcp_max_ulp, int32_t* mc_mismatches, double* sqrt_max_rel);
 
-/* Test entry (no counterpart in the paper): one of the device helpers of the
- * step evaluated at n points.  `in` holds the helper's arguments as rows of n
- * values, `out` gets n values (host pointers; float32 helpers round their
- * arguments).  RSST_EINVAL for an unknown helper, a NULL pointer or n outside
- * 1..2^26.  Synchronous, current device. */
+/* Helpers that rsst_math_eval evaluates, with their arguments. */
 typedef enum {
   RSST_EVAL_RCP = 0,          /* x: 1/x of the float64 step */
   RSST_EVAL_SQRT_PAIR,        /* x: sqrt(x) as a float pair, its sum */
@@ -397,6 +393,12 @@ typedef enum {
                                * c_tot - c_tot0 */
 } rsst_eval_fn;
 #define RSST_EVAL_GAMMA_XI2 (5.0 / 3.0 / 900.0)
+
+/* Test entry (no counterpart in the paper): one of the device helpers of the
+ * step evaluated at n points.  `in` holds the helper's arguments as rows of n
+ * values, `out` gets n values (host pointers; float32 helpers round their
+ * arguments).  RSST_EINVAL for an unknown helper, a NULL pointer or n outside
+ * 1..2^26.  Synchronous, current device. */
 int rsst_math_eval(int32_t fn, int64_t n, const double* in, double* out);
 
 /* Float64 FMA throughput of the current device in TFLOP/s, measured by a
