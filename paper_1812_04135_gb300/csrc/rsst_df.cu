@@ -513,6 +513,7 @@ static const int TILE2_DF[2] = {16, 8};
 int rsst_stage_df_tile(const Geom& g, int sms) {
   static const double offset[2] = {5.0, 5.2}, slope[2] = {4.1, 1.6};
   if (g.ndim != 2) return 0;
+  if ((g.n[1] + TILE2_DF[1] - 1) / TILE2_DF[1] > RSST_GRID_Y) return 0;  // beyond the launch grid's y limit
   double us[2];
   for (int t = 0; t < 2; ++t) {
     const int b = TILE2_DF[t];

@@ -482,7 +482,9 @@ using namespace rsst;
 // / 16 x 8 / 8 x 8): 64^2 16.9 / 11.8 / 8.7, 128^2 16.9 / 12.1 / 11.8, 192^2
 // 16.9 / 17.5 / 19.8, 224^2 30.4 / 24.9 / 31.0, 256^2 30.4 / 32.2 / 34.7,
 // 512^2 99.5 / 106.5 / 118.5, 2048^2 1493 / 1603 / 1840; the constants fit
-// these.  (4 x 4 tiles gained 0.1 us on 64^2 and lost elsewhere.)
+// these.  (4 x 4 tiles gained 0.1 us on 64^2 and lost elsewhere.)  A shape
+// whose rows of tiles exceed the launch grid's y limit is not taken (tall,
+// narrow grids).
 static const int TILE2[3][2] = {{16, 16}, {16, 8}, {8, 8}};
 
 int rsst_stage_fp64_tile(const Geom& g, int sms) {
@@ -491,7 +493,9 @@ int rsst_stage_fp64_tile(const Geom& g, int sms) {
   int best = 0;
   double tbest = 0.0;
   for (int t = 0; t < 3; ++t) {
-    const int64_t tiles = (int64_t)((g.n[0] + TILE2[t][0] - 1) / TILE2[t][0]) * ((g.n[1] + TILE2[t][1] - 1) / TILE2[t][1]);
+    const int rows = (g.n[1] + TILE2[t][1] - 1) / TILE2[t][1];
+    const int64_t tiles = (int64_t)((g.n[0] + TILE2[t][0] - 1) / TILE2[t][0]) * rows;
+    if (t > 0 && rows > RSST_GRID_Y) continue;
     const double us = offset[t] + slope[t] * (double)((tiles + sms - 1) / sms);
     if (t == 0 || us < tbest) {
       best = t;

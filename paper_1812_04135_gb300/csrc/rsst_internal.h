@@ -13,6 +13,8 @@
 // thread), so that a short line runs on many SMs instead of one CTA on one SM
 #define RSST_SMALL_1D (32 * 152 * 4)
 
+#define RSST_GRID_Y 65535  // blocks a launch takes along y and z
+
 // Bits of a run's device flag (sticky until the next rsst_set_state).
 #define RSST_FLAG_NONPHYSICAL 1u  // a stage produced rho <= 0, P <= 0 or a non-finite value
 #define RSST_FLAG_TIMEOUT 2u      // a bounded wait on a TMA copy or barrier gave up

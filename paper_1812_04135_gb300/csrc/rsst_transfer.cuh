@@ -27,7 +27,7 @@ static inline XferGrid xfer_grid(int cells_x, int64_t rows) {
   XferGrid x;
   x.block = dim3(32, 8);
   const int64_t by = (rows + 7) / 8;
-  x.grid = dim3((cells_x + 31) / 32, (unsigned)(by < 65535 ? by : 65535));
+  x.grid = dim3((cells_x + 31) / 32, (unsigned)(by < RSST_GRID_Y ? by : RSST_GRID_Y));
   return x;
 }
 

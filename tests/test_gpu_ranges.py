@@ -1,0 +1,55 @@
+"""Runs at the ends of the parameters that rsst_init accepts: grids that are
+narrow and very tall, reduction rates and C_max laws whose squares leave the
+range of a float."""
+import numpy as np
+import pytest
+import torch
+
+from paper_1812_04135_gb300 import rsst
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    import os
+    if not os.path.exists(rsst.LIB_PATH):
+        import __graft_entry__
+        __graft_entry__.build()
+    rsst.lib()
+
+
+def workload(n, **more):
+    w = {"ndim": len(n), "n": n, "dx": (1.0,) * len(n), "gamma": 5.0 / 3.0, "xi": 4.0, "variant": "pvs",
+         "bc": ("periodic",) * len(n), "grav": (0.0, 0.0, 0.0), "vertical": -1, "bg_rho": None, "bg_p": None, "cmax": 0.0,
+         "cfl_rule": 0, "covolume": 0.0, "cfl": 0.4}
+    w.update(more)
+    return w
+
+
+def uniform(n, rho, v, e):
+    U = torch.zeros((len(n) + 2,) + tuple(reversed(n)), dtype=torch.float64)
+    U[0], U[1], U[-1] = rho, rho * v, e + 0.5 * rho * v * v
+    return U.cuda()
+
+
+def advance(w, U, steps, dt=0.0, precision="fp64"):
+    s = rsst.Solver(w, precision)
+    try:
+        s.set_state(U)
+        s.step(steps, dt)
+        return s.get_state("cuda"), s.dt()
+    finally:
+        s.close()
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp64_df"])
+def test_narrow_and_very_tall_grid(precision):
+    """More rows than 65535 tiles of 8: the run equals that of one of its 40-row periods, bit for bit."""
+    nx, period, periods = 8, 40, 15000
+    rng = np.random.default_rng(1)
+    one = uniform((nx, period), 1.0, 0.0, 1.5)
+    one += 0.1 * torch.from_numpy(rng.uniform(-1.0, 1.0, tuple(one.shape))).cuda()
+    ref, _ = advance(workload((nx, period)), one, 2, 0.05, precision)
+    got, _ = advance(workload((nx, period * periods)), one.repeat(1, periods, 1), 2, 0.05, precision)
+    assert torch.equal(got, ref.repeat(1, periods, 1))
