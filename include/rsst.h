@@ -379,7 +379,7 @@ typedef enum {
   RSST_EVAL_RCP = 0,          /* x: 1/x of the float64 step */
   RSST_EVAL_SQRT_PAIR,        /* x: sqrt(x) as a float pair, its sum */
   RSST_EVAL_CTOT,             /* rho |V|^2, P, 1/rho: the LLF speed's pair at gamma/xi^2 = RSST_EVAL_GAMMA_XI2 */
-  RSST_EVAL_CTOT_CMAX,        /* |V|^2, (a/xi)^2: c_tot under the C_max law */
+  RSST_EVAL_CTOT_CMAX,        /* |V|^2, (a/xi)^2: c_tot under the C_max law, as dt takes it */
   RSST_EVAL_RSQRT,            /* x: 1/sqrt(x) of the C_max law */
   RSST_EVAL_PAIR_TO_DOUBLE,   /* h, l of a normalised float pair */
   RSST_EVAL_SPEED,            /* x: sqrt(x) of the adjoint's wave speeds */

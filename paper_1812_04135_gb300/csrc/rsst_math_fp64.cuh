@@ -155,7 +155,10 @@ __device__ __forceinline__ double sqrt_ctot(double x) {
 // Zero and subnormal x give 0, negative x and NaN give NaN, like sqrt_ctot;
 // 2^k is kept to the float range (x in [2^-252, 2^256), far outside any
 // physical speed^2).
-__device__ __forceinline__ void sqrt_pair(double x, float& s, float& c) {
+//
+// root_parts: s0 (in [1, 2]), c0 and k for a positive normal x (true), false
+// for any other.
+__device__ __forceinline__ bool root_parts(double x, float& s0, float& c0, int& k) {
   const long long ix = __double_as_longlong(x);
   const int be = (int)(ix >> 52);  // biased exponent for x >= 0, negative for x < 0
   const int e = be - 1023;
@@ -163,14 +166,20 @@ __device__ __forceinline__ void sqrt_pair(double x, float& s, float& c) {
   const float h = __int_as_float(((127 + odd) << 23) | (int)((ix >> 29) & 0x7fffff));
   const float l = __uint2float_rn((unsigned)(ix & 0x1fffffff)) * __int_as_float((75 + odd) << 23);  // * 2^(odd-52)
   const float r = rsqrtf(h);
-  const float s0 = h * r;
+  s0 = h * r;
   const float p = s0 * s0;
   const float d = ((h - p) - fmaf(s0, s0, -p)) + l;
-  const float c0 = d * (0.5f * r);
-  const int k = (e - odd) >> 1;
+  c0 = d * (0.5f * r);
+  k = (e - odd) >> 1;
+  return be > 0 && be < 2047;
+}
+__device__ __forceinline__ void sqrt_pair(double x, float& s, float& c) {
+  float s0, c0;
+  int k;
+  const bool fin = root_parts(x, s0, c0, k);
   const float sc = k < -126 ? 0.0f : (k > 127 ? __int_as_float(0x7f800000) : __int_as_float((127 + k) << 23));
-  const bool fin = be > 0 && be < 2047;
-  const float special = (ix >= 0 && be == 0) ? 0.0f : __int_as_float(0x7fc00000);
+  const long long ix = __double_as_longlong(x);
+  const float special = (ix >= 0 && (ix >> 52) == 0) ? 0.0f : __int_as_float(0x7fc00000);
   s = fin ? s0 * sc : special;
   c = fin ? c0 * sc : special;
 }
@@ -280,11 +289,12 @@ __device__ __forceinline__ void ctot_pair_of(double k, double P, double ir, cons
 // 1/sqrt(w): the hardware approximation (20 bits) and one third-order step,
 // y (1 + e/2 + 3 e^2/8) with e = 1 - w y^2, which cubes its error: about one
 // ulp in five float64 operations instead of an IEEE square root and division.
+// 0 for an infinite w.
 __device__ __forceinline__ double rsqrt_nr(double w) {
   double y;
   asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(w));
   const double e = fma(-(w * y), y, 1.0);
-  return fma(y * e, fma(0.375, e, 0.5), y);
+  return __double2hiint(w) == 0x7ff00000 ? 0.0 : fma(y * e, fma(0.375, e, 0.5), y);
 }
 
 // A float pair s + c with |c| within some ulps of s as a double, on the float32
@@ -294,12 +304,35 @@ __device__ __forceinline__ double sum_to_double(float s, float c) {
   return pair_to_double(h, c - (h - s));
 }
 
+// x times 2^k, on the integer pipe (x and the result positive normal).
+__device__ __forceinline__ double scale2(double x, int k) {
+  return __hiloint2double(__double2hiint(x) + (k << 20), __double2loint(x));
+}
+
 // c_tot under the C_max law from |V|^2 and (a/xi)^2, with three float64
 // instructions: the roots as float pairs (2^-42), one float64 Newton step on the
 // sound term, which carries c_tot in slow flow (a float pair's accuracy showed
-// there against a 64-bit evaluation).  Zero, NaN and values beyond a float's
-// range come as sqrt_pair gives them.
+// there against a 64-bit evaluation).  The LLF speed is a float pair in the end,
+// so its roots may have a float's range: beyond it, and for NaN, they come as
+// sqrt_pair gives them.  dt (WIDE) takes any magnitude of a double: there the
+// roots' exponents are added as integers.  (WIDE in the faces too cost 3.7 % of
+// the 250^2 case.)
+template <bool REFINE>
+__device__ __forceinline__ double root_any(double x) {
+  const long long ix = __double_as_longlong(x);
+  if (ix == 0) return 0.0;
+  const bool tiny = ix > 0 && ix < (1ll << 52);  // subnormal
+  if (tiny) x *= 0x1p108;
+  float s, c;
+  int k;
+  if (!root_parts(x, s, c, k)) return ix == 0x7ff0000000000000ll ? x : __longlong_as_double(0x7ff8000000000000ll);
+  double y = scale2(sum_to_double(s, c), k);
+  if constexpr (REFINE) y = fma(fma(-y, y, x), scale2(f2d_bits(__fdividef(0.5f, s)), -k), y);
+  return tiny ? scale2(y, -54) : y;
+}
+template <bool WIDE>
 __device__ __forceinline__ double ctot_cmax(double v2, double a2x) {
+  if constexpr (WIDE) return root_any<false>(v2) + root_any<true>(a2x);
   float s, c;
   sqrt_pair(a2x, s, c);
   const double y = sum_to_double(s, c);
@@ -354,7 +387,7 @@ template <bool CV>
 __device__ __forceinline__ void ctot_of(const Phys& p, double rho, double k, double P, double ir, float& h, float& l) {
   if (p.use_cmax) {
     const double a2 = Eos<CV>::sound2(p, rho, P, ir);
-    to_pair(ctot_cmax(k * ir, a2 * rsqrt_nr(fma(a2 * a2, p.inv_cmax4, 1.0))), h, l);
+    to_pair(ctot_cmax<false>(k * ir, a2 * rsqrt_nr(fma(a2 * a2, p.inv_cmax4, 1.0))), h, l);
   } else if constexpr (CV) {
     ctot_pair(k * ir, Eos<CV>::sound2_over_xi2(p, rho, P, ir), h, l);
   } else {
@@ -568,7 +601,7 @@ __device__ __forceinline__ double cfl_rate(const double (&q)[NV], const Phys& p,
   ok = fin && positive_finite(rho) && positive_finite(P) && Eos<CV>::admissible(p, rho);
   if (p.use_cmax) {
     const double a2 = Eos<CV>::sound2(p, rho, P, ir);
-    return ctot_cmax(k * ir, a2 * rsqrt_nr(fma(a2 * a2, p.inv_cmax4, 1.0))) * p.sum_inv_dx;
+    return ctot_cmax<true>(k * ir, a2 * rsqrt_nr(fma(a2 * a2, p.inv_cmax4, 1.0))) * p.sum_inv_dx;
   }
   float ch, cl;
   ctot_of<CV>(p, rho, k, P, ir, ch, cl);

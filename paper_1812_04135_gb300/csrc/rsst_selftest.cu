@@ -92,7 +92,7 @@ __global__ void eval_kernel(int fn, int64_t n, const double* __restrict__ in, do
       ctot_pair_of(x, y, z, p, h, l);
       out[i] = (double)h + (double)l;
       break;
-    case RSST_EVAL_CTOT_CMAX: out[i] = ctot_cmax(x, y); break;
+    case RSST_EVAL_CTOT_CMAX: out[i] = ctot_cmax<true>(x, y); break;
     case RSST_EVAL_RSQRT: out[i] = rsqrt_nr(x); break;
     case RSST_EVAL_PAIR_TO_DOUBLE: out[i] = pair_to_double((float)x, (float)y); break;
     case RSST_EVAL_SPEED:

@@ -41,3 +41,14 @@ def test_adjoint_speeds_at_every_leading_significand(low, exponent):
     # the root's pair 2^-42; its reciprocal's seed error 2^-22 squared and its roundings 2^-45 on top
     assert np.abs(rsst.rsst_math_eval("speed", x) / s - 1.0).max() <= 2.0 ** -42
     assert np.abs(rsst.rsst_math_eval("inv_speed", x) * s - 1.0).max() <= 2.0 ** -41
+
+
+def test_cmax_wave_speed_at_any_magnitude():
+    """The C_max law's c_tot: float64-accurate in its sound term, |V| to 2^-42, over the range of float64."""
+    rng = np.random.default_rng(9)
+    n = 1 << 16
+    x = np.ldexp(1.0 + rng.random(n), np.linspace(-1000, 1000, n).astype(int))
+    zero = np.zeros(n)
+    assert np.abs(rsst.rsst_math_eval("ctot_cmax", zero, x) / np.sqrt(x) - 1.0).max() <= 2.0 ** -52
+    assert np.abs(rsst.rsst_math_eval("ctot_cmax", x, zero) / np.sqrt(x) - 1.0).max() <= 2.0 ** -42
+    assert rsst.rsst_math_eval("rsqrt", [np.inf])[0] == 0.0

@@ -53,3 +53,23 @@ def test_narrow_and_very_tall_grid(precision):
     ref, _ = advance(workload((nx, period)), one, 2, 0.05, precision)
     got, _ = advance(workload((nx, period * periods)), one.repeat(1, periods, 1), 2, 0.05, precision)
     assert torch.equal(got, ref.repeat(1, periods, 1))
+
+
+@pytest.mark.parametrize("n", [(40,), (20, 12), (10, 9, 8)])
+@pytest.mark.parametrize("scale", [-200, 150])
+def test_cmax_law_at_speeds_beyond_floats(n, scale):
+    """Speeds and C_max times 2^scale: dt times 2^-scale (gas at rest and in motion)."""
+    for v in (0.0, 0.7):
+        _, dt = advance(workload(n, cmax=0.6), uniform(n, 1.3, v, 2.0), 0)
+        f = 2.0 ** scale
+        _, dt2 = advance(workload(n, cmax=0.6 * f), uniform(n, 1.3, v * f, 2.0 * f * f), 0)
+        assert dt2 * f == pytest.approx(dt, rel=1e-14)
+
+
+@pytest.mark.parametrize("n", [(40,), (20, 12), (10, 9, 8)])
+def test_cmax_law_with_an_unbounded_reduction(n):
+    """(a/C_max)^4 overflows: xi is infinite, a/xi = 0 and f = 1."""
+    U = uniform(n, 1.3, 0.7, 2.0)
+    got, dt = advance(workload(n, cmax=1e-78), U, 2)
+    assert dt == pytest.approx(0.4 / (0.7 * len(n)), rel=1e-12)
+    assert float((got - U).abs().max()) <= 1e-13
