@@ -218,6 +218,12 @@ static void make_physf(const Phys* p, PhysF* f) {
 }
 
 void rsst_split_gamma_xi2(Phys* p) {
+  if (p->gamma_xi2 == 0.0) {  // xi^2 beyond float64: a root of 2^gxe that is 0 as a float
+    p->gxh = 1.0f;
+    p->gxl = 0.0f;
+    p->gxe = -8192;
+    return;
+  }
   int e;
   const double m = 2.0 * std::frexp(p->gamma_xi2, &e);  // in [1, 2)
   p->gxh = (float)m;

@@ -56,6 +56,15 @@ def test_narrow_and_very_tall_grid(precision):
 
 
 @pytest.mark.parametrize("n", [(40,), (20, 12), (10, 9, 8)])
+def test_reduction_rate_whose_square_overflows(n):
+    """a/xi vanishes beside |V|: dt is that of the flow."""
+    U = uniform(n, 1.3, 0.7, 2.0)
+    got, dt = advance(workload(n, xi=1e160), U, 2)
+    assert dt == pytest.approx(0.4 / (0.7 * len(n)), rel=1e-12)
+    assert float((got - U).abs().max()) <= 1e-13
+
+
+@pytest.mark.parametrize("n", [(40,), (20, 12), (10, 9, 8)])
 @pytest.mark.parametrize("scale", [-200, 150])
 def test_cmax_law_at_speeds_beyond_floats(n, scale):
     """Speeds and C_max times 2^scale: dt times 2^-scale (gas at rest and in motion)."""
