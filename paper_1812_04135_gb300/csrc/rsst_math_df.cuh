@@ -104,7 +104,8 @@ __device__ __forceinline__ double df_to_bits(df x) { return f2d(x.hi) + f2d(x.lo
 // Constants of the step in double-float (split once on the host).
 struct PhysDF {
   df gamma, gm1, nhgm1, inv_gm1, gam_gm1;  // nhgm1 = -(gamma - 1)/2, gam_gm1 = gamma/(gamma - 1)
-  df gx;                                   // gamma/xi^2 (constant xi)
+  df gx;                                   // gamma/xi^2 (constant xi) over xs^2: in [1, 4)
+  float xs;                                // a power of two, 0 below the floats
   df nf, nf_gm1, inv_cmax4;                // -f, -f (gamma - 1)
   df grav[3], nhalf_inv_dx[3], sum_inv_dx;  // nhalf_inv_dx = -1/(2 dx): the faces hold twice the flux
   int variant, use_cmax, has_grav;
@@ -131,14 +132,15 @@ __device__ __forceinline__ df half_mc_df(df a, df b) {
 __device__ __forceinline__ df cmax_factor_df(df a2, const PhysDF& p) {
   return rcp(dsqrt(df_fma(a2 * a2, p.inv_cmax4, df_make(1.0f))));
 }
-// (a/xi)^2 from P/rho: constant xi, or the C_max law.
+// a/xi from P/rho: constant xi (gamma/xi^2 itself leaves a float's range from xi
+// = 1e19 on, long before a/xi does), or the C_max law.
 template <bool CMAX>
-__device__ __forceinline__ df sound2_df(df p_rho, const PhysDF& p) {
+__device__ __forceinline__ df sound_df(df p_rho, const PhysDF& p) {
   if constexpr (CMAX) {
     const df a2 = p.gamma * p_rho;
-    return a2 * cmax_factor_df(a2, p);
+    return dsqrt(a2 * cmax_factor_df(a2, p));
   }
-  return p.gx * p_rho;
+  return scale(dsqrt(p.gx * p_rho), p.xs);
 }
 
 // The Euler flux along D and c_tot of one state; k = rho |V|^2 = m.V feeds
@@ -154,7 +156,7 @@ __device__ __forceinline__ void euler_flux_df(const df (&q)[NV], const PhysDF& p
 #pragma unroll
   for (int e = 1; e < ND; ++e) k = df_fma(q[1 + e], v[e], k);
   const df P = df_fma(p.nhgm1, k, p.gm1 * q[NV - 1]);
-  c = dsqrt(k * ir) + dsqrt(sound2_df<CMAX>(P * ir, p));
+  c = dsqrt(k * ir) + sound_df<CMAX>(P * ir, p);
   F[0] = q[1 + D];
 #pragma unroll
   for (int e = 0; e < ND; ++e) F[1 + e] = (e == D) ? df_fma(q[1 + e], v[D], P) : q[1 + e] * v[D];
@@ -260,8 +262,8 @@ __device__ __forceinline__ df cfl_rate_df(const df (&q)[NV], const PhysDF& p, bo
   }
   const df P = df_fma(p.nhgm1, k, p.gm1 * q[NV - 1]);
   ok = fin && df_pos(rho) && df_pos(P);
-  const df s2 = p.use_cmax ? sound2_df<true>(P * ir, p) : sound2_df<false>(P * ir, p);
-  return (dsqrt(k * ir) + dsqrt(s2)) * p.sum_inv_dx;
+  const df a = p.use_cmax ? sound_df<true>(P * ir, p) : sound_df<false>(P * ir, p);
+  return (dsqrt(k * ir) + a) * p.sum_inv_dx;
 }
 
 }  // namespace rsst

@@ -48,6 +48,7 @@ void rsst_launch_eval_fp32(int fn, int64_t n, const double* in, double* out) {
   pf.gx = 1.0f;
   rsst::PhysDF pd = {};
   pd.gm1 = pd.inv_gm1 = pd.gx = {1.0f, 0.0f};
+  pd.xs = 1.0f;
   pd.nhgm1 = {-0.5f, 0.0f};
   rsst::eval_fp32_kernel<<<(unsigned)((n + 255) / 256), 256>>>(fn, n, in, out, pf, pd);
 }

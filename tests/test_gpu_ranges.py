@@ -64,6 +64,15 @@ def test_reduction_rate_whose_square_overflows(n):
     assert float((got - U).abs().max()) <= 1e-13
 
 
+@pytest.mark.parametrize("xi", [1e16, 1e20, 1e30])
+def test_double_float_large_reduction_rate(xi):
+    """Gas at rest: dt is that of a/xi, also where 1/xi^2 is below the floats."""
+    n = (24, 16)
+    got, dt = advance(workload(n, xi=xi), uniform(n, 1.3, 0.0, 2.0), 0, precision="fp64_df")
+    a = np.sqrt(5.0 / 3.0 * (2.0 / 3.0) * 2.0 / 1.3)
+    assert dt == pytest.approx(0.4 / (2.0 * a / xi), rel=1e-12)
+
+
 @pytest.mark.parametrize("n", [(40,), (20, 12), (10, 9, 8)])
 @pytest.mark.parametrize("scale", [-200, 150])
 def test_cmax_law_at_speeds_beyond_floats(n, scale):
