@@ -353,20 +353,20 @@ __device__ __forceinline__ void to_pair(double x, float& h, float& l) {
   l = fin ? l * sc : 0.0f;
 }
 
-// 1/x of a positive float pair as a double (relative error below 2^-43).
-__device__ __forceinline__ double rcp_of_pair(float h, float l) {
-  float r;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(h));
-  return pair_to_double(r, r * fmaf(-l, r, fmaf(-h, r, 1.0f)));
-}
-
-// sqrt(x) and its reciprocal as doubles on the float32 and integer pipes (for the
-// adjoint's derivatives of c_tot); both 0 at x = 0.
+// sqrt(x) (2^-42) and its reciprocal (2^-41) as doubles on the float32 and
+// integer pipes, for the adjoint's derivatives of c_tot at any magnitude of
+// the speeds.  Both corrections are added to their leading parts before they
+// become a double (a correction may exceed an ulp).  0 and 0 for zero and
+// subnormal x, NaN and 0 for any other that is not a positive normal number.
 __device__ __forceinline__ void sqrt_rcp(double x, double& s, double& r) {
-  float h, l;
-  sqrt_pair(x, h, l);
-  s = h == 0.0f ? 0.0 : pair_to_double(h, l);
-  r = h > 0.0f ? rcp_of_pair(h, l) : 0.0;
+  float h, c, y;
+  int k;
+  const bool fin = root_parts(x, h, c, k);
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(h));
+  const double sd = scale2(sum_to_double(h, c), k);
+  const double rd = scale2(sum_to_double(y, y * fmaf(-c, y, fmaf(-h, y, 1.0f))), -k);
+  s = fin ? sd : (((unsigned long long)__double_as_longlong(x) >> 52) == 0 ? 0.0 : __longlong_as_double(0x7ff8000000000000ll));
+  r = fin ? rd : 0.0;
 }
 
 // Effective sound speed a/xi from a^2 and the factor f = 1 - 1/xi^2: constant

@@ -43,6 +43,16 @@ def test_adjoint_speeds_at_every_leading_significand(low, exponent):
     assert np.abs(rsst.rsst_math_eval("inv_speed", x) * s - 1.0).max() <= 2.0 ** -41
 
 
+def test_adjoint_speeds_at_any_magnitude():
+    """The derivative of |V| is V/|V| however small the speed."""
+    x = np.ldexp(1.0 + np.random.default_rng(6).random(1 << 16), np.linspace(-1021, 1022, 1 << 16).astype(int))
+    s = np.sqrt(x)
+    assert np.abs(rsst.rsst_math_eval("speed", x) / s - 1.0).max() <= 2.0 ** -42
+    assert np.abs(rsst.rsst_math_eval("inv_speed", x) * s - 1.0).max() <= 2.0 ** -41
+    assert np.array_equal(rsst.rsst_math_eval("speed", [0.0, 5e-324]), [0.0, 0.0])
+    assert np.array_equal(rsst.rsst_math_eval("inv_speed", [0.0, 5e-324]), [0.0, 0.0])
+
+
 def test_cmax_wave_speed_at_any_magnitude():
     """The C_max law's c_tot: float64-accurate in its sound term, |V| to 2^-42, over the range of float64."""
     rng = np.random.default_rng(9)
