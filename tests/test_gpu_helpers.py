@@ -53,6 +53,23 @@ def test_adjoint_speeds_at_any_magnitude():
     assert np.array_equal(rsst.rsst_math_eval("inv_speed", [0.0, 5e-324]), [0.0, 0.0])
 
 
+def mc(a, b):
+    s = np.where((np.abs(a) <= np.abs(b)) & (4 * np.abs(a) <= np.abs(a + b)), 2 * a,
+                 np.where(4 * np.abs(b) <= np.abs(a + b), 2 * b, 0.5 * (a + b)))
+    return np.where((np.sign(a) * np.sign(b)) > 0, s, 0.0)
+
+
+@pytest.mark.parametrize("fn,factor", [("mc_slope", 1.0), ("half_mc", 0.5)])
+def test_limiter_next_to_the_subnormal_range(fn, factor):
+    """Differences in the far tail of a profile: no sign or exponent wraps (the values are exact up to the smallest
+    normal number)."""
+    rng = np.random.default_rng(7)
+    e = rng.integers(-1074, -1000, (2, 1 << 16))
+    a, b = np.ldexp(rng.uniform(0.5, 1.0, e.shape), e) * rng.choice([-1.0, 1.0], e.shape)
+    got = rsst.rsst_math_eval(fn, a, b)
+    assert np.abs(got - factor * mc(a, b)).max() <= 2.0 ** -1022
+
+
 def test_cmax_wave_speed_at_any_magnitude():
     """The C_max law's c_tot: float64-accurate in its sound term, |V| to 2^-42, over the range of float64."""
     rng = np.random.default_rng(9)

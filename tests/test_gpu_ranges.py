@@ -91,3 +91,14 @@ def test_cmax_law_with_an_unbounded_reduction(n):
     got, dt = advance(workload(n, cmax=1e-78), U, 2)
     assert dt == pytest.approx(0.4 / (0.7 * len(n)), rel=1e-12)
     assert float((got - U).abs().max()) <= 1e-13
+
+
+def test_limiter_in_the_far_tail_of_a_profile():
+    """A velocity profile whose tail passes through the subnormal numbers stays finite."""
+    x = torch.arange(400, dtype=torch.float64) / 10.0
+    v = 0.1 * torch.exp(-x * x).cuda()
+    U = uniform((400,), 1.0, 0.0, 2.0)
+    U[1] = v
+    U[2] += 0.5 * v * v
+    got, dt = advance(workload((400,), bc=("reflect",)), U, 3)
+    assert bool(torch.isfinite(got).all()) and dt > 0.0
