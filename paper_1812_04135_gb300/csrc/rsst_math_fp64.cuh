@@ -209,17 +209,17 @@ __device__ __forceinline__ void ctot_pair(double v2, double a2x, float& h, float
 }
 
 // A normalised non-negative float pair (h + l, |l| <= ulp(h)/2) as a double,
-// on the integer pipe: h's 24 bits shifted up plus l in units of 2^-52 of h's
-// exponent (l below that is dropped: 2^-53 relative).  Below a power of two
-// the unit halves, hence the doubled l there.  Outside h in [2^-74, 2^126]
-// (and for NaN) the two halves are added.
+// on the integer pipe: h's 24 bits shifted up plus l in units of the result's
+// last place (2^-52 of h's exponent; half of that below a power of two), rounded
+// as a float64 sum of the two would be.  Outside h in [2^-74, 2^126] (and for
+// NaN) the two halves are added.
 __device__ __forceinline__ double pair_to_double(float h, float l) {
   const unsigned hb = __float_as_uint(h);
   const int eh = (int)(hb >> 23);
   const unsigned mant = hb & 0x7fffffu;
   if (eh >= 53 && eh <= 253) {
-    int li = __float2int_rn(l * __int_as_float((306 - eh) << 23));
-    if (mant == 0u && li < 0) li += li;
+    const int unit = mant == 0u && l < 0.0f ? 307 : 306;
+    const int li = __float2int_rn(l * __int_as_float((unit - eh) << 23));
     return __longlong_as_double(((long long)(eh + 896) << 52) + ((long long)mant << 29) + (long long)li);
   }
   return f2d_bits(h) + f2d_bits(l);

@@ -33,6 +33,17 @@ def test_reciprocal_at_every_leading_significand(low, exponent):
     assert np.abs(got.view(np.int64) - want.view(np.int64)).max() <= 1
 
 
+def test_pair_to_double_rounds_the_sum():
+    """The nearest double of h + l, powers of two (the unit below them is half) among the h."""
+    rng = np.random.default_rng(5)
+    e = rng.integers(-70, 120, 1 << 20)
+    h = np.ldexp(1.0 + rng.integers(0, 1 << 23, e.size) * 2.0 ** -23 * (rng.random(e.size) < 0.5), e).astype(np.float32)
+    below = np.where(np.frexp(h)[0] == 0.5, 0.25, 0.5)
+    l = (rng.uniform(-1.0, 1.0, e.size) * 2.0 ** -rng.integers(0, 30, e.size) * below * np.spacing(h)).astype(np.float32)
+    got = rsst.rsst_math_eval("pair_to_double", h, l)
+    assert np.array_equal(got, h.astype(np.float64) + l.astype(np.float64))
+
+
 @pytest.mark.parametrize("low", LOWS)
 @pytest.mark.parametrize("exponent", [0, 1, -2])
 def test_adjoint_speeds_at_every_leading_significand(low, exponent):
