@@ -81,6 +81,23 @@ def test_limiter_next_to_the_subnormal_range(fn, factor):
     assert np.abs(got - factor * mc(a, b)).max() <= 2.0 ** -1022
 
 
+def test_wave_speed_pair_accuracy():
+    """|V| + a/xi from rho |V|^2, P and 1/rho.  Each square is a product of float pairs (2^-45: the two low parts'
+    product 2^-46 and two roundings 2^-47), halved by the root; a root's correction of 2^-22.4 has three
+    roundings (2^-44.8); the pairs' sum one (2^-46).  Together below 2^-43.7."""
+    rng = np.random.default_rng(8)
+    worst = 0.0
+    for _ in range(8):
+        n = 1 << 22
+        rho, P = np.exp(rng.uniform(-7, 7, n)), np.exp(rng.uniform(-7, 7, n))
+        ir = 1.0 / rho
+        k = P * np.exp(rng.uniform(-25, 5, n)) * (rng.random(n) < 0.9)
+        gx = 5.0 / 3.0 / 900.0
+        want = np.sqrt(k * ir) + np.sqrt(gx * (P * ir))
+        worst = max(worst, np.abs(rsst.rsst_math_eval("ctot", k, P, ir) / want - 1.0).max())
+    assert worst <= 2.0 ** -43.7, np.log2(worst)
+
+
 def test_cmax_wave_speed_at_any_magnitude():
     """The C_max law's c_tot: float64-accurate in its sound term, |V| to 2^-42, over the range of float64."""
     rng = np.random.default_rng(9)
