@@ -173,12 +173,13 @@ __device__ __forceinline__ void llf_flux_x2_df(const df (&qL)[NV], const df (&qR
 #pragma unroll
   for (int k = 0; k < NV; ++k) {
     // one three-term sum: the product's and the sums' exact errors are added
-    // up once, 31 float operations instead of 37
-    const df d = two_sum(qL[k].hi, -qR[k].hi);
-    const float dl = d.lo + (qL[k].lo - qR[k].lo);
+    // up once, 34 float operations instead of 37 (the difference is normalised:
+    // states that agree in their leading floats differ by the low ones alone)
+    const df t0 = two_sum(qL[k].hi, -qR[k].hi);
+    const df d = fast_two_sum(t0.hi, t0.lo + (qL[k].lo - qR[k].lo));
     const float pr = __fmul_rn(alpha.hi, d.hi);
     float e = fmaf(alpha.hi, d.hi, -pr);
-    e = fmaf(alpha.hi, dl, e);
+    e = fmaf(alpha.hi, d.lo, e);
     e = fmaf(alpha.lo, d.hi, e);
     const df s = two_sum(FL[k].hi, FR[k].hi);
     const df t = two_sum(s.hi, pr);

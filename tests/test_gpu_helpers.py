@@ -107,3 +107,16 @@ def test_cmax_wave_speed_at_any_magnitude():
     assert np.abs(rsst.rsst_math_eval("ctot_cmax", zero, x) / np.sqrt(x) - 1.0).max() <= 2.0 ** -52
     assert np.abs(rsst.rsst_math_eval("ctot_cmax", x, zero) / np.sqrt(x) - 1.0).max() <= 2.0 ** -42
     assert rsst.rsst_math_eval("rsqrt", [np.inf])[0] == 0.0
+
+
+def test_double_float_flux_of_a_small_difference():
+    """States that agree in their leading floats: the dissipation alpha (rho_L - rho_R) keeps its relative accuracy
+    (the speed 2^-44, the product 2^-46)."""
+    rng = np.random.default_rng(10)
+    n = 1 << 18
+    hi = (1.0 + rng.random(n)).astype(np.float32).astype(np.float64)
+    low = rng.integers(-(1 << 22), 1 << 22, (2, n)) * 2.0 ** -47
+    rl, rr, E = hi + low[0], hi + low[1], 1.0 + rng.random(n).astype(np.float32)
+    got = rsst.rsst_math_eval("df_flux", rl, rr, E)
+    want = np.sqrt(E / np.minimum(rl, rr)) * (rl - rr)
+    assert (np.abs(got - want) <= 2.0 ** -43 * np.abs(want)).all()
