@@ -236,10 +236,12 @@ __device__ __forceinline__ void cell_lean2(const f2 (&q)[NV], f2 (&L)[NV], const
     const bool mom = form == RSST_PVS || form == RSST_DVS;
     const f2 H = fma2(dup2(pf.gam_gm1), P, mom ? kin : kin * dup2(-1.0f));  // e + P +- rho V^2/2
     if (form == RSST_PVS || form == RSST_PMS || form == RSST_PD) {
-      f2 s = fma2(kin * ir, Dl[0], Dl[NV - 1]);
+      // minus dP/(gamma - 1), dE last: one rounding at its size (a float32 run
+      // amplifies this term's round-off by xi^2)
+      f2 ns = (k * dup2(-0.5f)) * ir * Dl[0];
 #pragma unroll
-      for (int e = 0; e < ND; ++e) s = s - v[e] * Dl[1 + e];
-      const f2 nfs = s * (fcell * dup2(-pf.gm1));  // -f dP
+      for (int e = 0; e < ND; ++e) ns = fma2(v[e], Dl[1 + e], ns);
+      const f2 nfs = (ns - Dl[NV - 1]) * (fcell * dup2(pf.gm1));  // -f dP
       if (form == RSST_PD) {
         L[NV - 1] = fma2(nfs, dup2(pf.inv_gm1), L[NV - 1]);
       } else {

@@ -120,3 +120,18 @@ def test_double_float_flux_of_a_small_difference():
     got = rsst.rsst_math_eval("df_flux", rl, rr, E)
     want = np.sqrt(E / np.minimum(rl, rr)) * (rl - rr)
     assert (np.abs(got - want) <= 2.0 ** -43 * np.abs(want)).all()
+
+
+def test_float32_pair_pressure_tendency_rounds_once_at_the_energy_tendency():
+    """dP/(gamma - 1) = |V|^2/2 drho - V.dm + dE with small first terms: their roundings (2^-22 of at most 2^-5 dE
+    together) and one of dE's size."""
+    rng = np.random.default_rng(11)
+    n = 1 << 20
+    f = np.float32
+    mx, my, dr, dx, dy = (rng.uniform(-0.125, 0.125, n).astype(f) for _ in range(5))
+    dE = (rng.choice([-1.0, 1.0], n) * (1.0 + rng.random(n))).astype(f)
+    got = rsst.rsst_math_eval("pair_tendency", np.ones(n), mx, my, dr, dx, dy, dE)
+    mx, my, dr, dx, dy, dE = (v.astype(np.float64) for v in (mx, my, dr, dx, dy, dE))
+    want = 0.5 * (mx * mx + my * my) * dr - (mx * dx + my * dy) + dE
+    half_ulp = 0.5 * np.spacing(np.abs(want).astype(f)).astype(np.float64)
+    assert (np.abs(got - want) <= half_ulp + 2.0 ** -22 * 2.0 ** -5).all()
