@@ -145,7 +145,7 @@ __device__ __forceinline__ void flux_lean2(const f2 (&q)[NV], f2 rho0, f2 P0, f2
     if constexpr (CMAX) {
       dc = vm + (ax - c0);
     } else {
-      const f2 da2x = (P1 * rho0 - P0 * q[0]) * (ir * gxr0);
+      const f2 da2x = fma2(P1, rho0, P0 * (q[0] * dup2(-1.0f))) * (ir * gxr0);  // one product rounded by itself
       dc = fma2(da2x, rcp2(ax + a0x), vm);
     }
   }

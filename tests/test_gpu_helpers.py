@@ -135,3 +135,22 @@ def test_float32_pair_pressure_tendency_rounds_once_at_the_energy_tendency():
     want = 0.5 * (mx * mx + my * my) * dr - (mx * dx + my * dy) + dE
     half_ulp = 0.5 * np.spacing(np.abs(want).astype(f)).astype(np.float64)
     assert (np.abs(got - want) <= half_ulp + 2.0 ** -22 * 2.0 ** -5).all()
+
+
+def test_float32_pair_speed_difference_rounds_one_product():
+    """c_tot - c_tot0 of a state whose P1 rho0 and P0 rho1 nearly cancel: one of the products is rounded (2^-24 of
+    it), the other goes into the sum exactly; 2^-20 of the result for everything after."""
+    rng = np.random.default_rng(12)
+    n = 1 << 20
+    f = np.float32
+    r0, P0, r1 = ((1.0 + rng.random(n)).astype(f) for _ in range(3))
+    r1 = (r1 * f(0.25)).astype(f)
+    P1 = (P0 * r1 / r0 * (1.0 + rng.uniform(-1.0, 1.0, n) * 2.0 ** -10)).astype(f)
+    got = rsst.rsst_math_eval("pair_dc", r1, P1, r0, P0)
+    r0, P0, r1, P1 = (v.astype(np.float64) for v in (r0, P0, r1, P1))
+    rho, P = r0 + r1, P0 + P1
+    a, a0 = np.sqrt(P / rho), np.sqrt(P0 / r0)
+    diff = P1 * r0 - P0 * r1
+    want = diff / (rho * r0) / (a + a0)
+    bound = 2.0 ** -24 * np.maximum(P1 * r0, P0 * r1) * 1.01 / (rho * r0) / (a + a0) + 2.0 ** -20 * np.abs(want)
+    assert (np.abs(got - want) <= bound).all()
