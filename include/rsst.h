@@ -205,6 +205,11 @@ int rsst_sync(rsst_handle* h);
  * runs).  Synchronous, launches nothing. */
 int rsst_debug_stall_wait(rsst_handle* h, int64_t limit_ns);
 
+/* The same test hook (no counterpart in the paper) for 2D/3D RSST_FP64_DF
+ * runs, whose kernel waits while its tile copy is in flight.  Errors as
+ * above. */
+int rsst_debug_stall_wait_df(rsst_handle* h, int64_t limit_ns);
+
 /* Sum over cells of each conserved variable times the cell volume, in
  * float64, deterministic order (fixed-shape two-level tree): the totals whose
  * conservation by form Sec. 5 and App. A discuss.  In

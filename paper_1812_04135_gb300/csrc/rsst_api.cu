@@ -617,18 +617,28 @@ extern "C" int rsst_set_graph_steps(rsst_handle* h, int32_t k) {
   return RSST_OK;
 }
 
-extern "C" int rsst_debug_stall_wait(rsst_handle* h, int64_t limit_ns) {
+static int set_stall(rsst_handle* h, int64_t limit_ns, bool has_wait, const char* where, const char* which) {
   if (!h || limit_ns < 0 || limit_ns > 1000000000LL) {
-    rsst_set_error("rsst_debug_stall_wait: need a handle and 0 <= limit_ns <= 1e9");
+    rsst_set_error("%s: need a handle and 0 <= limit_ns <= 1e9", where);
     return RSST_EINVAL;
   }
-  if (!h->use_tma2d && !h->use_tma3d && !h->use_tma_fp64) {
-    rsst_set_error("rsst_debug_stall_wait: only runs on the TMA-staged kernels (float32 perturbation 2D/3D, float64 2D/3D) have the test wait");
+  if (!has_wait) {
+    rsst_set_error("%s: only %s runs have this test wait", where, which);
     return RSST_EUNSUPPORTED;
   }
   if (limit_ns != h->stall_ns) drop_graphs(h);  // graphs hold the stage arguments by value
   h->stall_ns = limit_ns;
   return RSST_OK;
+}
+
+extern "C" int rsst_debug_stall_wait(rsst_handle* h, int64_t limit_ns) {
+  return set_stall(h, limit_ns, h && (h->use_tma2d || h->use_tma3d || h->use_tma_fp64), "rsst_debug_stall_wait",
+                   "float32 perturbation 2D/3D and float64 2D/3D");
+}
+
+extern "C" int rsst_debug_stall_wait_df(rsst_handle* h, int64_t limit_ns) {
+  return set_stall(h, limit_ns, h && h->cfg.precision == RSST_FP64_DF && h->cfg.ndim >= 2, "rsst_debug_stall_wait_df",
+                   "double-float 2D/3D");
 }
 
 extern "C" int rsst_step(rsst_handle* h, double dt, int nsteps) {

@@ -114,7 +114,8 @@ struct TileCfgDF {
   static constexpr bool ALL = NDIM <= 2;
   static constexpr int FMAX = ALL ? F0 + F1 : max3(F0, F1, F2);
   static constexpr int EMAX = ALL ? E0 + E1 : max3(E0, E1, E2);
-  // halo tile, faces, half slopes, the block reduction and dt (64 values), the tile copy's mbarrier
+  // halo tile, faces, half slopes, the block reduction and dt (64 values), two mbarriers (the tile copy; the
+  // failure-detection test wait)
   static constexpr size_t SMEM = sizeof(df) * ((size_t)NV * (SCELLS + FMAX + EMAX) + 64) + 16;
   static constexpr uint32_t TILE_BYTES = (uint32_t)(sizeof(df) * NV * SCELLS);
   static_assert(BX % 2 == 0 && (NDIM < 2 || BY % 2 == 0) && (NDIM < 3 || BZ % 2 == 0), "slopes are taken in pairs");
@@ -221,6 +222,7 @@ struct DFArgs {
   unsigned int* flag;
   int slot, stage;
   double dt_fixed;
+  int64_t stall_ns;  // as in StageArgs
 };
 
 template <int NDIM, int BX, int BY, int BZ, int NT, int MINB, bool CMAX, int ST>
@@ -250,17 +252,22 @@ __global__ void __launch_bounds__(NT, MINB)
     // the halo tile of all fields by one TMA copy (as in rsst_fp64.cu: a
     // double-float is an 8-byte element of the same layout)
     uint64_t* bar = reinterpret_cast<uint64_t*>(sred + 64);
+    uint64_t* test_bar = bar + 1;
+    const bool stall = a.stall_ns > 0;
     if (threadIdx.x == 32) {
       mbar_init(bar, 1);
+      if (stall) mbar_init(test_bar, 1);
       fence_mbar_init();
       fence_proxy_async_smem();
       mbar_expect_tx(bar, C::TILE_BYTES);
       if constexpr (NDIM == 2) tma_load_3d(su, &tin, bar, i0 + g.xoff - C::HX, j0, 0);
       else tma_load_4d(su, &tin, bar, i0 + g.xoff - C::HX, j0, k0, 0);
+      if (stall) mbar_expect_tx(test_bar, 16);  // bytes that no copy delivers, waited on while the tile's is in flight
     }
-    __syncthreads();  // the barrier is initialised, dt is there
+    __syncthreads();  // the barriers are initialised, dt is there
+    const bool landed = mbar_wait_bounded(stall ? test_bar : bar, 0u, stall ? (uint64_t)a.stall_ns : RSST_WAIT_NS);
     // giving up (flag, one more bounded wait for the copy) is decided by the whole block
-    if (__syncthreads_or(!mbar_wait_bounded(bar, 0u))) {
+    if (__syncthreads_or(!landed)) {
       if (threadIdx.x == 0) {
         atomicOr(a.flag, RSST_FLAG_TIMEOUT);
         mbar_wait_bounded(bar, 0u);
@@ -548,6 +555,7 @@ int rsst_launch_stage_df(const CUtensorMap* tin, const StageArgs<float2>& sa, cu
   a.slot = sa.slot;
   a.stage = sa.stage;
   a.dt_fixed = sa.dt_fixed;
+  a.stall_ns = sa.stall_ns;
   switch (a.g.ndim) {
     case 1:
       if (a.g.n[0] <= RSST_SMALL_1D) return launch_df<1, 16, 1, 1, 32, 1>(nullptr, a, s);

@@ -61,6 +61,7 @@ def lib():
             "rsst_dt": (i32, [vp, pd]),
             "rsst_sync": (i32, [vp]),
             "rsst_debug_stall_wait": (i32, [vp, i64]),
+            "rsst_debug_stall_wait_df": (i32, [vp, i64]),
             "rsst_batch_debug_stall_wait": (i32, [vp, i32, i64]),
             "rsst_time": (i32, [vp, pd]),
             "rsst_conserved_sums": (i32, [vp, pd]),
@@ -219,6 +220,11 @@ def rsst_debug_stall_wait(h: int, limit_ns: int) -> None:
     """Failure-detection test hook: each tile of the 2D float32 TMA kernel
     also waits limit_ns on a barrier nothing completes (0: off)."""
     _check(lib().rsst_debug_stall_wait(h, int(limit_ns)), "rsst_debug_stall_wait")
+
+
+def rsst_debug_stall_wait_df(h: int, limit_ns: int) -> None:
+    """The same for the 2D/3D double-float kernel."""
+    _check(lib().rsst_debug_stall_wait_df(h, int(limit_ns)), "rsst_debug_stall_wait_df")
 
 
 def rsst_conserved_sums(h: int, nvar: int) -> list:
