@@ -21,13 +21,18 @@ namespace rsst {
 struct XferGrid {
   dim3 grid, block;
 };
-// Blocks of 32 x 8 threads, one cell a thread: 256-byte pieces of eight rows,
-// so that a row of any length wastes less than one warp.
+// Blocks of 256 threads, one cell a thread: 32 x 8 (256-byte pieces of eight
+// rows, so that a row of any length wastes less than one warp), for shorter
+// rows the next power of two wide and the more rows (32 lanes to a row of two
+// cells would idle), for fewer rows than eight wider (a line: 256 x 1).
 static inline XferGrid xfer_grid(int cells_x, int64_t rows) {
+  int bx = 32;
+  while (bx > 2 && bx / 2 >= cells_x) bx /= 2;
+  while (bx >= 32 && bx < 256 && 256 / bx > rows) bx *= 2;
   XferGrid x;
-  x.block = dim3(32, 8);
-  const int64_t by = (rows + 7) / 8;
-  x.grid = dim3((cells_x + 31) / 32, (unsigned)(by < RSST_GRID_Y ? by : RSST_GRID_Y));
+  x.block = dim3(bx, 256 / bx);
+  const int64_t by = (rows + x.block.y - 1) / x.block.y;
+  x.grid = dim3((cells_x + bx - 1) / bx, (unsigned)(by < RSST_GRID_Y ? by : RSST_GRID_Y));
   return x;
 }
 
