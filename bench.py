@@ -549,9 +549,12 @@ def run_modes(dev, peaks, src):
     del w
     out["batched_fp32_pert_64runs"] = measure_batched(dev, peaks, src)
     out["adjoint_fp64_polytrope_256"] = measure_adjoint(dev)
-    # 1D N=256 sound wave, 2000 steps: launch-bound; CUDA-graph blocks vs plain launches
-    w = inputs.sound_wave_1d(256, xi=10.0, variant="pvs")
-    for k, name in ((16, "fp64_sound1d_256_graph"), (0, "fp64_sound1d_256_plain")):
+    # 1D sound waves, 2000 steps: 256 cells on the cluster kernel, 4096 cells on stage kernels in CUDA-graph blocks and
+    # as plain launches (lines of up to 2048 cells take no notice of the setting)
+    for n, k, name, bound in ((256, 16, "fp64_sound1d_256", "latency (dependent float64 instructions, cluster barrier)"),
+                              (4096, 16, "fp64_sound1d_4096_graph", "launch latency"),
+                              (4096, 0, "fp64_sound1d_4096_plain", "launch latency")):
+        w = inputs.sound_wave_1d(n, xi=10.0, variant="pvs")
         stream = torch.cuda.current_stream(dev)
         s = rsst.Solver(w, "fp64", stream=stream)
         s.set_graph_steps(k)
@@ -567,8 +570,8 @@ def run_modes(dev, peaks, src):
         s.sync()
         s.close()
         t = e0.elapsed_time(e1) / 1e3
-        out[name] = {"value": 256 * 2 * 2000 / t, "unit": UNIT, "steps_per_s": 2000 / t, "steps": 2000,
-                     "graph_steps": k, "bound": "launch latency", "clocks": clk.summary()}
+        out[name] = {"value": n * 2 * 2000 / t, "unit": UNIT, "steps_per_s": 2000 / t, "steps": 2000,
+                     "graph_steps": k, "bound": bound, "clocks": clk.summary()}
     return out
 
 
