@@ -518,12 +518,13 @@ using namespace rsst;
 
 // 2D tiles: the one that finishes first by a linear model, as for float64
 // (rsst_stage_fp64_tile): 16 x 16, or 8 x 8 where a grid is too small to fill
-// the SMs.  Measured per stage (us, 16 x 16 / 8 x 8): 64^2 9.5 / 6.7, 128^2
-// 9.6 / 7.5, 256^2 12.6 / 17.4, 512^2 33.7 / 47.8.
+// the SMs.  Measured per stage (us, 16 x 16 / 8 x 8): 64^2 7.4 / 5.5, 128^2
+// 7.5 / 6.2, 160^2 7.6 / 6.5, 192^2 7.9 / 7.2, 224^2 10.2 / 9.7, 256^2 10.1 /
+// 13.4, 512^2 27.4 / 39.2, 2048^2 388 / 558; the model takes the faster of each.
 static const int TILE2_DF[2] = {16, 8};
 
 int rsst_stage_df_tile(const Geom& g, int sms) {
-  static const double offset[2] = {5.0, 5.2}, slope[2] = {4.1, 1.6};
+  static const double offset[2] = {4.3, 2.6}, slope[2] = {3.55, 1.29};
   if (g.ndim != 2) return 0;
   if ((g.n[1] + TILE2_DF[1] - 1) / TILE2_DF[1] > RSST_GRID_Y) return 0;  // beyond the launch grid's y limit
   double us[2];

@@ -479,16 +479,16 @@ using namespace rsst;
 // most tiles any SM gets (the float64 pipe of an SM serves its tiles one
 // after the other).  16 x 16 has the fewest halo faces a cell, smaller tiles
 // spread a small grid over more SMs.  Measured per stage (us, GB300; 16 x 16
-// / 16 x 8 / 8 x 8): 64^2 16.9 / 11.8 / 8.7, 128^2 16.9 / 12.1 / 11.8, 192^2
-// 16.9 / 17.5 / 19.8, 224^2 30.4 / 24.9 / 31.0, 256^2 30.4 / 32.2 / 34.7,
-// 512^2 99.5 / 106.5 / 118.5, 2048^2 1493 / 1603 / 1840; the constants fit
-// these.  (4 x 4 tiles gained 0.1 us on 64^2 and lost elsewhere.)  A shape
-// whose rows of tiles exceed the launch grid's y limit is not taken (tall,
-// narrow grids).
+// / 16 x 8 / 8 x 8): 64^2 16.9 / 12.6 / 9.0, 128^2 16.9 / 12.9 / 11.0, 160^2
+// 17.1 / 17.3 / 13.7, 192^2 17.2 / 17.4 / 17.7, 224^2 28.6 / 23.3 / 25.3, 256^2
+// 28.6 / 29.7 / 33.2, 512^2 89.5 / 95.5 / 104, 2048^2 1338 / 1428 / 1610; with
+// these constants the model takes the fastest of each.  (4 x 4 tiles gained
+// 0.1 us on 64^2 and lost elsewhere.)  A shape whose rows of tiles exceed the
+// launch grid's y limit is not taken (tall, narrow grids).
 static const int TILE2[3][2] = {{16, 16}, {16, 8}, {8, 8}};
 
 int rsst_stage_fp64_tile(const Geom& g, int sms) {
-  static const double offset[3] = {3.4, 3.0, 4.6}, slope[3] = {13.5, 7.25, 4.05};
+  static const double offset[3] = {4.5, 5.0, 3.3}, slope[3] = {12.35, 6.6, 3.72};
   if (g.ndim != 2) return 0;
   int best = 0;
   double tbest = 0.0;
