@@ -165,14 +165,19 @@ int rsst_get_state(rsst_handle* h, double* U, int on_host);
  * (reconstruction, LLF flux, divergence, RSST correction, force, RK update,
  * ghost cells; the second also reduces the CFL maximum).  Whole blocks of
  * rsst_set_graph_steps() steps replay a captured CUDA graph; the results
- * are the same as with plain launches.  Asynchronous. */
+ * are the same as with plain launches.  A 1D RSST_FP64 run of up to 2048
+ * cells takes neither: up to 1024 steps run in one launch on a thread-block
+ * cluster (where the device can hold one of 16 CTAs), the same bits however
+ * the steps are split over calls.  Asynchronous. */
 int rsst_step(rsst_handle* h, double dt, int nsteps);
 
 /* Steps per replayed CUDA graph in rsst_step (default 16; 0 = plain
  * launches only).  k must be even and >= 0, else RSST_EINVAL.  A graph is
  * captured per CFL-slot parity on first use and again when a fixed dt
- * changes.  This is a launch-overhead control for small grids: the paper
- * has no counterpart. */
+ * changes.  A 1D RSST_FP64 run of up to 2048 cells has no use for it (see
+ * rsst_step): the value is checked and kept, its steps do not change.  This
+ * is a launch-overhead control for small grids: the paper has no
+ * counterpart. */
 int rsst_set_graph_steps(rsst_handle* h, int32_t k);
 
 /* The step the next adaptive rsst_step will take (cfl / CFL maximum of the
@@ -231,7 +236,9 @@ int rsst_conserved_sums(rsst_handle* h, double* sums);
  * counterpart in the paper).  All device memory the adjoint needs is
  * allocated here (library-owned): ceil(nsteps/every) checkpoints, 2 x every
  * recompute states and their Euler tendencies, and a few state-sized work
- * arrays; RSST_ENOMEM if that fails.  The handle ends at U^{nsteps}.
+ * arrays; RSST_ENOMEM if that fails.  A recording with the same `every` and
+ * number of segments takes over the last one's memory; another shape, or
+ * rsst_destroy, gives it back.  The handle ends at U^{nsteps}.
  * RSST_EUNSUPPORTED for runs that are not float64 or not the ideal gas
  * (covolume > 0).  Asynchronous. */
 int rsst_adjoint_record(rsst_handle* h, double dt, int nsteps, int every);
@@ -366,16 +373,15 @@ int64_t rsst_kernel_launches(const rsst_handle* h);
 
 /* Self-test of the float64 helpers the kernels use in place of compiler
  * sequences (no counterpart in the paper): over n seeded inputs, the largest
- * difference in ulps between the reciprocal (hardware seed and one
- * third-order step) and CUDA's correctly rounded 1.0/x (x in [2^-20, 2^20]);
+ * difference in ulps between the reciprocal (a float-pair seed and one
+ * Newton step) and CUDA's correctly rounded 1.0/x (x in [2^-20, 2^20]);
  * the number of inputs on which the integer-pipe MC limiter differs from
  * the direct float64 form (plus 2^20 if a c_tot square root misses one of
  * its special cases: 0 and subnormal -> 0, negative and NaN -> NaN, or the
  * float-to-double bit conversion a case); and the largest relative
- * difference between either c_tot square root (the float64 one of the
- * adjoint and the C_max law, the float-pair one of the LLF speed and the CFL
- * rate) and CUDA's
- * sqrt (x in [2^-200, 2^200]).  All outputs are host pointers.
+ * difference between either c_tot square root (the float64 one of |V| in
+ * the adjoint under the C_max law, the float-pair one of the other wave
+ * speeds) and CUDA's sqrt (x in [2^-200, 2^200]).  All outputs are host pointers.
  * Synchronous, current device. */
 int rsst_math_selftest(int32_t n, double* rcp_max_ulp, int32_t* mc_mismatches, double* sqrt_max_rel);
 

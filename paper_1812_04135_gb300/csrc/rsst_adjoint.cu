@@ -24,7 +24,7 @@
 // the chain rule backwards once.
 //
 // What bounds it: the float64 pipe, in the face kernel above all.  A 2D face
-// takes 173 float64 instructions (295 when both sides carried the wave speed's
+// takes 154 float64 instructions (295 when both sides carried the wave speed's
 // derivatives, speeds and their reciprocals came from float64 square roots,
 // limiter and flux halves were multiplications and each block summed its xi
 // partials by a float64 tree).  A stage's VJP on 256^2 (ncu, us): cells 21,

@@ -7,11 +7,11 @@
 //
 // What bounds it: instruction issue and the float32 pipe (a double-float
 // operation is 7 to 15 float32 instructions).  Thread instructions a 2D cell
-// in stage 1 (ncu, 512^2): 4100 -> 2743, by products fed unnormalised into
+// in stage 1 (ncu, 512^2): 4100 -> 2785, by products fed unnormalised into
 // sums (df_fma, the three-term sum of the LLF flux), twice-flux faces, slopes
 // in pairs that share a difference, rho |V|^2 = m.V, the C_max law and the
 // stage as template arguments, and the tile by TMA instead of loads and index
-// arithmetic.  512^2: 40.9 -> 27.2 us a stage; 3D 90 x 70 x 50: 112 -> 74 us.
+// arithmetic.  512^2: 40.9 -> 27.4 us a stage; 3D 90 x 70 x 50: 112 -> 74 us.
 #include <climits>
 #include <cmath>
 

@@ -17,8 +17,10 @@
 // The same tile routine serves the single-run grid and the batched
 // persistent kernel (rsst_batch.cu).
 //
-// What bounds it: instruction issue and its latencies.  Two columns a thread as
-// f32x2 pairs: 434 -> 342 thread instructions a stage-1 cell (ncu), at 58 % of
+// What bounds it: latencies that too few warps cover (at 2048^2 issue is 65 % busy
+// in stage 1 and 62 % in stage 2, the float32 pipe 54 and 50 %; stalls spread over
+// fixed latencies, the float32 pipe, barriers and loads).  Two columns a thread as
+// f32x2 pairs: 434 -> 344 thread instructions a stage-1 cell (ncu), at 65 % of
 // issue instead of 78 % (a pair instruction holds its pipe two cycles, and 126
 // registers leave four CTAs).  us a stage, one column a thread -> here: 2048^2
 // 68.5 -> 64.6, 1000^2 21.2 -> 19.3, and 4096^2 258 -> 244.  Other tiles (2048^2):

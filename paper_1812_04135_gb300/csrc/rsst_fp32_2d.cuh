@@ -101,8 +101,8 @@ struct TileRun {
 // (flag set, nothing left in flight).  Accumulates the stage-2 CFL rate
 // maximum and physical check.  The caller initialised the barrier; `phase` is
 // its current parity.  *sdt (shared memory) may be written up to the routine's
-// first barriers: the tile's copy does not wait for dt's float64 division.  FORM (-1: read from the run), the C_max law and the
-// stage are compile-time.
+// first barriers: the tile's copy does not wait for dt's float64 division.
+// FORM (-1: read from the run), the C_max law and the stage are compile-time.
 template <class T2, int VERT, int FORM, bool CM, int ST>
 __device__ __forceinline__ bool tile2d_f(const CUtensorMap* tin, const TileRun& r, const float* sdt, int tx, int ty,
                                          unsigned char* smem, uint32_t& phase, float& rmax, bool& ok_all) {

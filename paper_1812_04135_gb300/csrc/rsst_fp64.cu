@@ -23,7 +23,7 @@
 // What bounds it: the float64 pipe, which takes one warp instruction per 16
 // SM clocks (a warp alone one per 64, however few lanes it has active) while
 // every other pipe idles.  So the work is arranged for few float64
-// instructions: 165.7 a 2D cell in stage 1 and 181.7 in stage 2 (ncu), 205.5
+// instructions: 164.7 a 2D cell in stage 1 and 181.7 in stage 2 (ncu), 205.5
 // and 227.5 with the wave speeds' squares, the reciprocal's third-order step,
 // the block maximum, a per-thread dt division, unshared slope differences and
 // the RK halving's sign on that pipe.  512^2: 123 -> 89 us a stage; 3D 256 x

@@ -7,7 +7,7 @@
 // 64-bit index split per cell and a second pass for the CFL maximum; now the
 // instructions of address arithmetic and conversions (60 % of issue), and in
 // float64 runs the CFL rate on the float64 pipe.  Conversions run on the integer
-// pipe, a thread takes one cell of a 32 x 8 block, and the CFL maximum of the new
+// pipe, a thread takes one cell of a block shaped by the row, and the CFL maximum of the new
 // state is taken from the values being packed.  Load (CFL included) / read-back,
 // us: 4096^2 float32 535 / 313 -> 247 / 163, 3D 256 x 128 x 128 float32 194 / 116
 // -> 93 / 72, float64 238 / 73 -> 144 / 67, 512^2 double-float 32 / 28 -> 16 / 25.
