@@ -25,7 +25,10 @@
 // registers leave four CTAs).  us a stage, one column a thread -> here: 2048^2
 // 68.5 -> 64.6, 1000^2 21.2 -> 19.3, and 4096^2 258 -> 244.  Other tiles (2048^2):
 // 64 x 16 66.3, 64 x 8 66.6, 64 x 32 69.6, 8-cell segments 78 to 84; x faces in the
-// march by shuffles 67.8; a fifth CTA spills (89).
+// march by shuffles 67.8; a fifth CTA spills (89).  Small grids gain too (30 x 30 6.7
+// -> 6.0, 200^2 6.5 -> 5.8, 1500 x 300 9.1 -> 8.7); grids of at most four rows or
+// eight columns, where half the lanes of a pair tile idle, lose up to a fifth
+// (20000 x 4 5.8 -> 6.9, 4 x 20000 29.7 -> 33.1, 500 x 3 4.6 -> 5.2).
 #include "rsst_common.cuh"
 #include "rsst_fp32_2d.cuh"
 #include "rsst_attr.h"
